@@ -226,8 +226,9 @@ int32_t hippo_gather_kv(int32_t n_layers, const hippo_kv_cache_t *src, size_t sr
  * kv_len[b]-token context (their own K/V are already in the cache), every earlier key is visible.
  * The verification call is q_len = gamma + 1 rows against the full-length video cache, the draft call q_len = 1
  * against the short pruned cache.  Both names compute the same function for any q_len >= 1 and pick the kernel from
- * the shape: up to 8 packed rows over at most 1,024 keys run as one cluster of CTAs with a page each (latency-bound);
- * anything larger streams K/V tiles through one persistent CTA per SM.
+ * the shape: up to 16 packed rows over a short cache (up to tens of thousands of keys for one sequence, bf16, head_dim 64
+ * or 128) run as one cluster of CTAs per kv head (latency-bound); anything larger streams K/V tiles through one persistent
+ * CTA per SM.
  *   q        [batch][q_len][n_q_heads][head_dim] dtype        out  same shape and dtype as q
  *   kv_len   int32 [batch] (device), q_len <= kv_len[b] <= max_kv_len;  a sequence with kv_len[b] < q_len is skipped.
  *            NULL means the lengths are known on the host and all equal max_kv_len: the kernels then start their
@@ -238,7 +239,7 @@ int32_t hippo_gather_kv(int32_t n_layers, const hippo_kv_cache_t *src, size_t sr
  *            floating-point sums
  *   max_kv_len  host upper bound used to size the launch; <= max_pages_per_seq * 64
  *   softmax_scale  0 selects 1/sqrt(head_dim)
- *   num_splits  0 = automatic
+ *   num_splits  0 = automatic; > 0 asks for that many splits per kv head (ignored up to 1,024 keys and 8 packed rows)
  *   lse      optional fp32 [batch][q_len][n_q_heads], natural-log sum of exponentials of the scaled logits
  * bf16 with head_dim 64 or 128 runs on the tensor cores with TMA-staged tiles; fp32 (any head_dim that is a
  * multiple of 32, <= 256) runs on the CUDA cores.  q_len * G <= HIPPO_MAX_PACKED_ROWS.

@@ -1,26 +1,40 @@
 // Low-latency split-KV attention for few packed rows over a short cache: the draft model's decode step over the
-// pruned KV (Section 3.2, drafting phase: one query token, R = G <= 16 packed rows, a few hundred to a few thousand
-// keys).  Such a call moves well under a megabyte, so its cost is the length of the dependency chain, not bandwidth:
-// this kernel has no tensor-memory or TMA pipeline to fill and needs one launch.
+// pruned KV (Section 3.2, drafting phase: one or two query tokens, R = q_len * G <= 16 packed rows, some hundred to some
+// thousand keys).  Such a call moves a megabyte or two, so its cost is the length of the dependency chain, not bandwidth:
+// one launch, operands go from global memory straight into the registers the tensor instruction reads them from, and
+// every load of a step is in flight before the first one is used.
 //
-// One thread-block cluster per (sequence, kv head) unit.  The CTAs of a cluster split the unit's 64-key pages evenly.
-// Per page, in a CTA of 128 threads:
-//   scores   two threads per key, each holding half of the key's row in registers, dot it with the R query rows
-//            (fp32, query pre-scaled by scale*log2e and kept in shared memory)
-//   softmax  exact online update per page: row maxima by warp reduction, p = 2^(s - m) to shared memory
-//   output   thread (key group, 8-column group) accumulates R x 8 outputs over its keys of the page
-// The next page's K and V registers are loaded while the current page is computed.  At the end the key groups are
-// summed (warp shuffles, then one pass through shared memory).  Row r of the unit is merged by CTA r mod cluster
-// size: every CTA pushes its (m, l, O[r]) into that CTA's shared memory with remote stores, and after one cluster
-// barrier the owners merge what they received and write the output.
+// One thread-block cluster per (sequence, kv head) unit; the 32-key blocks of the unit's cache are dealt to the warps of
+// the cluster.  A warp does, per block of 32 keys, with mma.sync m16n8k16 (bf16 in, fp32 accumulate):
+//   scores  S[16 rows x 8 keys] = Q K^T.  The contraction index may be permuted as long as both operands agree, so lane
+//           (g, t) = (lane / 4, lane % 4) holds, of key g of a group of eight, the dimensions j*32 + t*8 .. + 7: plain
+//           16-byte loads, 64 contiguous bytes per key and load.
+//   softmax running row maxima per warp (two shuffles); the accumulator layout of S (row g, keys 2t, 2t + 1) is the
+//           layout of the second contraction's B operand, so probabilities never leave their registers.
+//   output  O^T[16 dims x 8 rows] += V^T P^T.  Lane (g, t) loads dimensions 8g .. 8g + 7 of keys 2t, 2t + 1, 2t + 8,
+//           2t + 9 of a group of sixteen (whole rows per load) and interleaves pairs of keys with byte permutes; the
+//           order of the output dimensions inside the instruction is free, so a lane ends with 8 neighbouring ones.
+// Probabilities are fp32: each is split into three bf16 terms (8 + 8 + 8 significant bits), three instructions per tile.
+// tcgen05 is not used: its 128 x N tile has one row block too many here and costs a tensor-memory allocation, barriers
+// and a descriptor round trip per call, which is most of the time this kernel takes in total.
+//
+// Bound by latency: two dependent round trips to memory (lengths and page ids, then keys and values; one for an
+// identity-mapped cache), the softmax and the merge.  Measured per call in a chain of 28: 755 keys (0.39 MB) 3.8 us, 5.8 us
+// with the CUDA-core kernel that stood here before; 3,537 keys (0.9 MB) 4.2 us, 10.2 us through tensor memory.
+//
+// The warps of a CTA merge through shared memory.  Row r of the unit is merged by CTA r mod cluster size: every CTA
+// pushes its (m, l, O[r]) into that CTA's shared memory with remote stores, and after one cluster barrier the owners
+// merge what they received and write the output.
 #include <math.h>
 
 #include "common.cuh"
 
 namespace hippo {
 
-constexpr int kSmThreads = 128;
-constexpr int kSmPage = kPageSize;     // keys per step
+constexpr int kSmBlock = 32;            // keys a warp takes at a time
+constexpr int kSmMaxWarps = 16;
+constexpr int kSmMaxCluster = 16;
+constexpr int kSmMaxRows = 16;
 constexpr float kSmLog2e = 1.4426950408889634f;
 constexpr float kSmLn2 = 0.6931471805599453f;
 
@@ -33,278 +47,317 @@ __device__ __forceinline__ uint32_t sm_cluster_map(uint32_t addr, uint32_t rank)
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-__device__ __forceinline__ void sm_st_cluster(uint32_t addr, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+__device__ __forceinline__ void sm_st_cluster_v2(uint32_t addr, float a, float b) {
+    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b) : "memory");
 }
 __device__ __forceinline__ void sm_st_cluster_v4(uint32_t addr, float4 v) {
     asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
-}
-__device__ __forceinline__ float sm_warp_max(float x) {
-    float y;
-    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(y) : "f"(x));
-    return y;
 }
 __device__ __forceinline__ float sm_ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ void unpack8(const uint4 &u, float *f) {
-    const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&u);
+__device__ __forceinline__ uint4 sm_ldg(const __nv_bfloat16 *p) { return __ldg(reinterpret_cast<const uint4 *>(p)); }
+__device__ __forceinline__ void sm_mma(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t sm_pack(float lo, float hi) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+// (x, y) as three bf16 pairs whose sums are x and y to fp32 precision
+__device__ __forceinline__ void sm_split3(float x, float y, uint32_t (&w)[3]) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) { const float2 t = __bfloat1622float2(h[i]); f[2 * i] = t.x; f[2 * i + 1] = t.y; }
+    for (int i = 0; i < 3; ++i) {
+        w[i] = sm_pack(x, y);
+        x -= __uint_as_float(w[i] << 16);
+        y -= __uint_as_float(w[i] & 0xffff0000u);
+    }
 }
 
-template <int D, int RMAX>
-struct SmallShared {
-    static constexpr int kHalf = D / 2;
-    static constexpr int kQHalfStride = RMAX * kHalf + 4;      // +4 floats: the two halves fall in different banks
-    static constexpr int kJG = kSmThreads / (D / 8);           // key groups of the output phase
-    float q[2 * kQHalfStride];                                 // [half][row][D/2], scaled by scale*log2e
-    float p[kSmPage][RMAX];                                    // probabilities of the current page
-    float wmax[4][RMAX];
-    float m[2][RMAX];                                          // running maxima, double buffered by page parity
-    float wsum[4][RMAX];
-    int limit[RMAX];
-    float red[4][RMAX][D];                                     // per-warp output partials
-    // partials pushed by the cluster peers for the rows this CTA merges: entry = slot * cluster size + peer,
-    // slot = r / cluster size; (slots x cluster size) <= max(RMAX, 16)
-    float recv_ml[16][2];
-    float recv_o[16][D];
+// Shared memory: warps' partials m[W][16] | l[W][16] | O[W][16 or 8 rows][D + 4], then what the cluster peers push:
+// (m, l)[32] | O[32][D].  A row's partials take an entry each: entry = (r / cluster size) * cluster size + peer < 32.
+template <int D, int NT>
+struct SmallSmem {
+    static constexpr int kRows = 8 * NT;
+    static constexpr int kOStride = D + 4;
+    static constexpr int kEntries = 2 * kSmMaxCluster;
+    __host__ __device__ static constexpr int ml_off() { return 0; }
+    __host__ __device__ static constexpr int o_off(int warps) { return 2 * warps * kRows; }
+    __host__ __device__ static constexpr int recv_ml_off(int warps) { return o_off(warps) + warps * kRows * kOStride; }
+    __host__ __device__ static constexpr int recv_o_off(int warps) { return recv_ml_off(warps) + 2 * kEntries; }
+    __host__ __device__ static constexpr size_t bytes(int warps) { return 4 * (size_t)(recv_o_off(warps) + kEntries * D); }
 };
 
-template <int D, int RMAX>
-__global__ void __launch_bounds__(kSmThreads) attn_small_kernel(const AttnParams p, const int cluster_size) {
-    using S = SmallShared<D, RMAX>;
-    constexpr int kHalf = D / 2, kKV4 = kHalf / 8;       // uint4 loads of a half row
-    constexpr int kDG = D / 8, kJG = S::kJG, kKPT = kSmPage / kJG;   // keys per thread in the output phase
-    __shared__ __align__(16) S sh;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+template <int D, int NT>   // head size; groups of eight packed rows
+__global__ void __launch_bounds__(D == 64 ? 512 : 256) attn_small_kernel(const AttnParams p, const int cluster_size) {
+    using S = SmallSmem<D, NT>;
+    constexpr int kKV4 = D / 32;          // 16-byte loads of a lane per key of the score operand
+    constexpr int kDT = D / 16;           // 16-dimension tiles of the output
+    extern __shared__ __align__(16) float smem[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    const int W = blockDim.x >> 5;
     const int R = p.rows, G = p.group, Hkv = p.n_kv_heads;
     const int unit = blockIdx.x / cluster_size, rank = blockIdx.x % cluster_size;
     const int b = unit / Hkv, hk = unit % Hkv;
-    const int kvl = p.kv_len ? p.kv_len[b] : p.max_kv_len;   // no length array: every sequence has max_kv_len keys
-    const bool skipped = kvl < p.q_len;
-    const int n_pages = skipped ? 0 : (kvl + kSmPage - 1) / kSmPage;
-    const int pg_begin = (int)((long long)n_pages * rank / cluster_size), pg_end = (int)((long long)n_pages * (rank + 1) / cluster_size);
+    const __nv_bfloat16 *kp = (const __nv_bfloat16 *)p.k_pages, *vp = (const __nv_bfloat16 *)p.v_pages;
+    const int stride = W * cluster_size;                        // blocks of 32 keys from one step of this warp to the next
+    const int first = warp * cluster_size + rank;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    int kvl = p.kv_len ? __ldg(p.kv_len + b) : p.max_kv_len;    // no length array: every sequence has max_kv_len keys
+    const int max_blocks = (p.max_kv_len + kSmBlock - 1) / kSmBlock;
+
+    // query rows as A operand; the contraction order is the one of the keys' loads
+    uint4 qr[NT][kKV4];
+#pragma unroll
+    for (int n = 0; n < NT; ++n) {
+        const int r = g + 8 * n, tq = r / G, gq = r - tq * G;
+#pragma unroll
+        for (int j = 0; j < kKV4; ++j)
+            qr[n][j] = r < R ? sm_ldg((const __nv_bfloat16 *)p.q + (((size_t)b * p.q_len + tq) * p.n_q_heads + hk * G + gq) * D + j * 32 + t * 8)
+                             : make_uint4(0, 0, 0, 0);
+    }
     const float sl2 = p.scale * kSmLog2e;
 
-    // ---- query rows (scaled) and per-row visibility limits
-    for (int x = tid; x < RMAX * (D / 8); x += kSmThreads) {
-        const int r = x / (D / 8), c8 = x % (D / 8);
-        float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        if (r < R) {
-            const int t = r / G, g = r % G;
-            unpack8(__ldg(reinterpret_cast<const uint4 *>((const __nv_bfloat16 *)p.q + (((size_t)b * p.q_len + t) * p.n_q_heads + hk * G + g) * D) + c8), v);
+    float o[NT][kDT][4], m[NT], l[NT];
+#pragma unroll
+    for (int n = 0; n < NT; ++n) {
+        m[n] = -INFINITY;
+        l[n] = 0.f;
+#pragma unroll
+        for (int i = 0; i < kDT; ++i) o[n][i][0] = o[n][i][1] = o[n][i][2] = o[n][i][3] = 0.f;
+    }
+
+    for (int blk = first; blk < max_blocks; blk += stride) {
+        // an identity-mapped cache is addressable up to max_kv_len, so its loads need not wait for the length; a page
+        // table is read only where the sequence has a page
+        int pid;
+        if (p.page_table) {
+            if (blk * kSmBlock >= kvl) break;
+            pid = __ldg(p.page_table + (size_t)b * p.max_pages_per_seq + blk / (kPageSize / kSmBlock));
+        } else {
+            pid = b * p.max_pages_per_seq + blk / (kPageSize / kSmBlock);
         }
-        float *dstq = sh.q + ((c8 * 8) / kHalf) * S::kQHalfStride + r * kHalf + (c8 * 8) % kHalf;
-        *reinterpret_cast<float4 *>(dstq) = make_float4(v[0] * sl2, v[1] * sl2, v[2] * sl2, v[3] * sl2);
-        *reinterpret_cast<float4 *>(dstq + 4) = make_float4(v[4] * sl2, v[5] * sl2, v[6] * sl2, v[7] * sl2);
-    }
-    if (tid < RMAX) {
-        sh.limit[tid] = tid < R ? kvl - p.q_len + tid / G : 0x7fffffff;
-        sh.m[0][tid] = -INFINITY;
-        sh.m[1][tid] = -INFINITY;
-    }
-    __syncthreads();
+        const size_t base = (((size_t)pid * Hkv + hk) * kPageSize + (blk % (kPageSize / kSmBlock)) * kSmBlock) * D;
+        uint4 kr[4][kKV4], vr[2][4][D / 64];
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int j = 0; j < kKV4; ++j) kr[x][j] = sm_ldg(kp + base + (x * 8 + g) * D + j * 32 + t * 8);
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+#pragma unroll
+            for (int y = 0; y < 4; ++y)
+#pragma unroll
+                for (int z = 0; z < D / 64; ++z)
+                    vr[x][y][z] = sm_ldg(vp + base + (x * 16 + (y >> 1) * 8 + 2 * t + (y & 1)) * D + z * 64 + g * 8);
 
-    const int key_j = tid >> 1, half = tid & 1;          // score phase: key of the page, half of the row
-    const int jg = tid / kDG, dg = tid % kDG;            // output phase: key group, 8-column group
-    const __nv_bfloat16 *kp = (const __nv_bfloat16 *)p.k_pages, *vp = (const __nv_bfloat16 *)p.v_pages;
-
-    float acc[RMAX][8], lpart[RMAX];
+        // ---- scores of the block: s[x] = rows (g, g + 8) x keys (8x + 2t, 8x + 2t + 1)
+        float s[4][4];
 #pragma unroll
-    for (int r = 0; r < RMAX; ++r) {
-        lpart[r] = 0.f;
+        for (int x = 0; x < 4; ++x) {
+            s[x][0] = s[x][1] = s[x][2] = s[x][3] = 0.f;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) acc[r][e] = 0.f;
-    }
-    uint4 kreg[kKV4], vreg[kKPT], knext[kKV4], vnext[kKPT];
-    auto load_page = [&](int pg, uint4 *kr, uint4 *vr) {
-        const int pid = page_of(p.page_table, p.max_pages_per_seq, b, pg);
-        const size_t base = ((size_t)pid * Hkv + hk) * kSmPage * D;
-        const int key0 = pg * kSmPage;
-#pragma unroll
-        for (int i = 0; i < kKV4; ++i)
-            kr[i] = key0 + key_j < kvl ? __ldg(reinterpret_cast<const uint4 *>(kp + base + (size_t)key_j * D + half * kHalf) + i) : make_uint4(0, 0, 0, 0);
-#pragma unroll
-        for (int i = 0; i < kKPT; ++i) {
-            const int j = jg * kKPT + i;
-            vr[i] = key0 + j < kvl ? __ldg(reinterpret_cast<const uint4 *>(vp + base + (size_t)j * D + dg * 8)) : make_uint4(0, 0, 0, 0);
-        }
-    };
-    if (pg_begin < pg_end) load_page(pg_begin, kreg, vreg);
-
-    for (int pg = pg_begin; pg < pg_end; ++pg) {
-        const int par = (pg - pg_begin) & 1;
-        if (pg + 1 < pg_end) load_page(pg + 1, knext, vnext);
-        // ---- scores of this thread's key against the R rows (half a row per thread, then the pair adds up)
-        float s[RMAX];
-#pragma unroll
-        for (int r = 0; r < RMAX; ++r) s[r] = 0.f;
-        const float *qh = sh.q + half * S::kQHalfStride;
-#pragma unroll
-        for (int i = 0; i < kKV4; ++i) {
-            float kf[8];
-            unpack8(kreg[i], kf);
-#pragma unroll
-            for (int r = 0; r < RMAX; ++r) {
-                const float4 q0 = *reinterpret_cast<const float4 *>(qh + r * kHalf + i * 8);
-                const float4 q1 = *reinterpret_cast<const float4 *>(qh + r * kHalf + i * 8 + 4);
-                s[r] = fmaf(kf[0], q0.x, fmaf(kf[1], q0.y, fmaf(kf[2], q0.z, fmaf(kf[3], q0.w, s[r]))));
-                s[r] = fmaf(kf[4], q1.x, fmaf(kf[5], q1.y, fmaf(kf[6], q1.z, fmaf(kf[7], q1.w, s[r]))));
+            for (int j = 0; j < kKV4; ++j) {
+                const uint4 a = qr[0][j], c = qr[NT - 1][j], k = kr[x][j];
+                sm_mma(s[x], a.x, NT > 1 ? c.x : 0u, a.y, NT > 1 ? c.y : 0u, k.x, k.y);
+                sm_mma(s[x], a.z, NT > 1 ? c.z : 0u, a.w, NT > 1 ? c.w : 0u, k.z, k.w);
             }
         }
-        const int key = pg * kSmPage + key_j;
+        const int key0 = blk * kSmBlock;
+        uint32_t pw[NT][4][3];
 #pragma unroll
-        for (int r = 0; r < RMAX; ++r) {
-            s[r] += __shfl_xor_sync(0xffffffffu, s[r], 1);
-            s[r] = key <= sh.limit[r] && key < kvl ? s[r] : -INFINITY;
-            const float wm = sm_warp_max(s[r]);
-            if (lane == r) sh.wmax[warp][r] = wm;
-        }
-        __syncthreads();
-        // ---- new maxima, probabilities, rescale of what has been accumulated
+        for (int n = 0; n < NT; ++n) {
+            const int limit = kvl - p.q_len + (g + 8 * n) / G;       // last key row g + 8n sees; rows beyond R are zeros
+            float mx = m[n];
 #pragma unroll
-        for (int r = 0; r < RMAX; ++r) {
-            const float m_old = sh.m[par][r];
-            const float m_new = fmaxf(fmaxf(m_old, fmaxf(sh.wmax[0][r], sh.wmax[1][r])), fmaxf(sh.wmax[2][r], sh.wmax[3][r]));
-            const float f = (m_old == -INFINITY) ? 0.f : sm_ex2(m_old - m_new);     // m_new = -inf implies m_old = -inf
-            const float pr = (s[r] == -INFINITY) ? 0.f : sm_ex2(s[r] - m_new);
-            lpart[r] = lpart[r] * f + (half == 0 ? pr : 0.f);
-            if (half == 0) sh.p[key_j][r] = pr;
-            if (tid == r) sh.m[par ^ 1][r] = m_new;
+            for (int x = 0; x < 4; ++x)
 #pragma unroll
-            for (int e = 0; e < 8; ++e) acc[r][e] *= f;
-        }
-        __syncthreads();
-        // ---- output: this thread's keys of the page, 8 columns, all rows
+                for (int e = 0; e < 2; ++e) {
+                    const int key = key0 + x * 8 + 2 * t + e;
+                    float &v = s[x][2 * n + e];
+                    v = key <= limit && key < kvl ? v * sl2 : -INFINITY;
+                    mx = fmaxf(mx, v);
+                }
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+            const float ref = mx == -INFINITY ? 0.f : mx;            // nothing visible yet: all probabilities are 0
+            const float f = sm_ex2(m[n] - ref);                      // m = -inf gives 0
+            float sum = 0.f;
 #pragma unroll
-        for (int i = 0; i < kKPT; ++i) {
-            const int j = jg * kKPT + i;
-            float vf[8];
-            unpack8(vreg[i], vf);
+            for (int x = 0; x < 4; ++x) {
+                const float p0 = sm_ex2(s[x][2 * n] - ref), p1 = sm_ex2(s[x][2 * n + 1] - ref);
+                sum += p0 + p1;
+                sm_split3(p0, p1, pw[n][x]);
+            }
+            l[n] = l[n] * f + sum;
+            m[n] = mx;
+            if (blk != first) {   // the rescale factors of the output's columns: rows 2t, 2t + 1 live in lanes g = 2t, 2t + 1
+                const float f0 = __shfl_sync(0xffffffffu, f, 8 * t), f1 = __shfl_sync(0xffffffffu, f, 8 * t + 4);
 #pragma unroll
-            for (int r4 = 0; r4 < RMAX; r4 += 4) {
-                const float4 pr = *reinterpret_cast<const float4 *>(&sh.p[j][r4]);
-                const float pw[4] = {pr.x, pr.y, pr.z, pr.w};
-#pragma unroll
-                for (int x = 0; x < 4; ++x)
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) acc[r4 + x][e] = fmaf(pw[x], vf[e], acc[r4 + x][e]);
+                for (int i = 0; i < kDT; ++i) { o[n][i][0] *= f0; o[n][i][1] *= f1; o[n][i][2] *= f0; o[n][i][3] *= f1; }
             }
         }
-        if (pg + 1 < pg_end) {
+        // ---- values of keys beyond the length may hold anything: 0 * NaN must not reach the output
+        if (key0 + kSmBlock > kvl) {
 #pragma unroll
-            for (int i = 0; i < kKV4; ++i) kreg[i] = knext[i];
+            for (int x = 0; x < 2; ++x)
 #pragma unroll
-            for (int i = 0; i < kKPT; ++i) vreg[i] = vnext[i];
+                for (int y = 0; y < 4; ++y)
+                    if (key0 + x * 16 + (y >> 1) * 8 + 2 * t + (y & 1) >= kvl)
+#pragma unroll
+                        for (int z = 0; z < D / 64; ++z) vr[x][y][z] = make_uint4(0, 0, 0, 0);
         }
-        // the next page's barrier after the scores separates these reads of p and wmax from their next writes
+        // ---- output
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+#pragma unroll
+            for (int z = 0; z < D / 64; ++z) {
+                const uint32_t *v0 = reinterpret_cast<const uint32_t *>(&vr[x][0][z]), *v1 = reinterpret_cast<const uint32_t *>(&vr[x][1][z]);
+                const uint32_t *v2 = reinterpret_cast<const uint32_t *>(&vr[x][2][z]), *v3 = reinterpret_cast<const uint32_t *>(&vr[x][3][z]);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const uint32_t a0 = __byte_perm(v0[i], v1[i], 0x5410), a1 = __byte_perm(v0[i], v1[i], 0x7632);
+                    const uint32_t a2 = __byte_perm(v2[i], v3[i], 0x5410), a3 = __byte_perm(v2[i], v3[i], 0x7632);
+#pragma unroll
+                    for (int n = 0; n < NT; ++n)
+#pragma unroll
+                        for (int w = 2; w >= 0; --w) sm_mma(o[n][z * 4 + i], a0, a1, a2, a3, pw[n][2 * x][w], pw[n][2 * x + 1][w]);
+                }
+            }
     }
-    const int par_end = (pg_end - pg_begin) & 1;
-    __syncthreads();
-    // ---- the CTA's partial: sums over the threads (l) and over the key groups (O)
+
+    // ---- the warp's partial: lane (g, t) has rows 2t, 2t + 1 (of each group of eight), dimensions 64z + 8g .. + 7
+    float *sm_ml = smem + S::ml_off(), *sm_o = smem + S::o_off(W);
 #pragma unroll
-    for (int r = 0; r < RMAX; ++r) {
-        float v = lpart[r];
-#pragma unroll
-        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == r) sh.wsum[warp][r] = v;
-    }
-    // key groups inside a warp (lane = key group * kDG + column group), then the four warps through shared memory
-#pragma unroll
-    for (int r = 0; r < RMAX; ++r)
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-#pragma unroll
-            for (int o = kDG; o < 32; o <<= 1) acc[r][e] += __shfl_xor_sync(0xffffffffu, acc[r][e], o);
-    if (lane < kDG) {
-#pragma unroll
-        for (int r = 0; r < RMAX; ++r) {
-            *reinterpret_cast<float4 *>(&sh.red[warp][r][lane * 8]) = make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
-            *reinterpret_cast<float4 *>(&sh.red[warp][r][lane * 8 + 4]) = make_float4(acc[r][4], acc[r][5], acc[r][6], acc[r][7]);
+    for (int n = 0; n < NT; ++n) {
+        float sum = l[n];
+        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+        sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+        if (t == 0) {
+            sm_ml[warp * S::kRows + 8 * n + g] = m[n];
+            sm_ml[(W + warp) * S::kRows + 8 * n + g] = sum;
         }
+#pragma unroll
+        for (int z = 0; z < D / 64; ++z)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                float *dst = sm_o + (warp * S::kRows + 8 * n + 2 * t + e) * S::kOStride + z * 64 + g * 8;
+                *reinterpret_cast<float4 *>(dst) = make_float4(o[n][z * 4][e], o[n][z * 4][2 + e], o[n][z * 4 + 1][e], o[n][z * 4 + 1][2 + e]);
+                *reinterpret_cast<float4 *>(dst + 4) = make_float4(o[n][z * 4 + 2][e], o[n][z * 4 + 2][2 + e], o[n][z * 4 + 3][e], o[n][z * 4 + 3][2 + e]);
+            }
     }
     __syncthreads();
-    // ---- push this CTA's partial of row r to the CTA that merges it
+    // ---- the CTA's partial of row r goes to the CTA that merges it
     {
-        const uint32_t a_ml = sm_smem_u32(sh.recv_ml), a_o = sm_smem_u32(sh.recv_o);
-        for (int x = tid; x < R * (D / 4); x += kSmThreads) {
+        const uint32_t a_ml = sm_smem_u32(smem + S::recv_ml_off(W)), a_o = sm_smem_u32(smem + S::recv_o_off(W));
+        for (int x = tid; x < R * (D / 4); x += blockDim.x) {
             const int r = x / (D / 4), c4 = x % (D / 4);
-            float4 v = *reinterpret_cast<const float4 *>(&sh.red[0][r][c4 * 4]);
-#pragma unroll
-            for (int w = 1; w < 4; ++w) {
-                const float4 t = *reinterpret_cast<const float4 *>(&sh.red[w][r][c4 * 4]);
-                v.x += t.x; v.y += t.y; v.z += t.z; v.w += t.w;
+            float M = -INFINITY, L = 0.f;
+            for (int w = 0; w < W; ++w) M = fmaxf(M, sm_ml[w * S::kRows + r]);
+            const float ref = M == -INFINITY ? 0.f : M;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int w = 0; w < W; ++w) {
+                const float f = sm_ex2(sm_ml[w * S::kRows + r] - ref);
+                const float4 a = *reinterpret_cast<const float4 *>(sm_o + (w * S::kRows + r) * S::kOStride + c4 * 4);
+                L = fmaf(sm_ml[(W + w) * S::kRows + r], f, L);
+                v.x = fmaf(a.x, f, v.x); v.y = fmaf(a.y, f, v.y); v.z = fmaf(a.z, f, v.z); v.w = fmaf(a.w, f, v.w);
             }
-            const int entry = (r / cluster_size) * cluster_size + rank;
-            sm_st_cluster_v4(sm_cluster_map(a_o, (uint32_t)(r % cluster_size)) + 4 * (entry * D + c4 * 4), v);
-        }
-        if (tid < R) {
-            const int r = tid, entry = (r / cluster_size) * cluster_size + rank;
-            const uint32_t dst = sm_cluster_map(a_ml, (uint32_t)(r % cluster_size)) + 8 * entry;
-            sm_st_cluster(dst, sh.m[par_end][r]);
-            sm_st_cluster(dst + 4, (sh.wsum[0][r] + sh.wsum[1][r]) + (sh.wsum[2][r] + sh.wsum[3][r]));
+            const int entry = (r / cluster_size) * cluster_size + rank, owner = r % cluster_size;
+            sm_st_cluster_v4(sm_cluster_map(a_o, (uint32_t)owner) + 4 * (entry * D + c4 * 4), v);
+            if (c4 == 0) sm_st_cluster_v2(sm_cluster_map(a_ml, (uint32_t)owner) + 8 * entry, M, L);
         }
     }
     sm_cluster_sync();   // release / acquire: the pushed partials are visible to their owners
     // ---- merge the rows r = rank, rank + cluster_size, ...: one warp per row, lanes over the columns
-    {
+    const float *recv_ml = smem + S::recv_ml_off(W), *recv_o = smem + S::recv_o_off(W);
+    for (int r = rank + cluster_size * warp; r < R; r += cluster_size * W) {
         constexpr int V = D / 32;
-        for (int r = rank + cluster_size * warp; r < R; r += cluster_size * (kSmThreads / 32)) {
-            const size_t ro = ((size_t)b * p.q_len + r / G) * p.n_q_heads + hk * G + r % G;
-            __nv_bfloat16 *o = (__nv_bfloat16 *)p.out + ro * D + lane * V;
-            const int e0 = (r / cluster_size) * cluster_size;
-            float M = -INFINITY, L = 0.f, av[V];
+        const size_t ro = ((size_t)b * p.q_len + r / G) * p.n_q_heads + hk * G + r % G;
+        const int e0 = (r / cluster_size) * cluster_size;
+        float M = -INFINITY, L = 0.f, av[V];
 #pragma unroll
-            for (int x = 0; x < V; ++x) av[x] = 0.f;
-            if (!skipped) {
-                for (int c = 0; c < cluster_size; ++c) M = fmaxf(M, sh.recv_ml[e0 + c][0]);
-                for (int c = 0; c < cluster_size; ++c) {
-                    const float m = sh.recv_ml[e0 + c][0];
-                    if (m == -INFINITY) continue;
-                    const float f = sm_ex2(m - M);
-                    L = fmaf(sh.recv_ml[e0 + c][1], f, L);
+        for (int x = 0; x < V; ++x) av[x] = 0.f;
+        for (int c = 0; c < cluster_size; ++c) M = fmaxf(M, recv_ml[2 * (e0 + c)]);
+        const float ref = M == -INFINITY ? 0.f : M;
+        for (int c = 0; c < cluster_size; ++c) {
+            const float f = sm_ex2(recv_ml[2 * (e0 + c)] - ref);
+            L = fmaf(recv_ml[2 * (e0 + c) + 1], f, L);
 #pragma unroll
-                    for (int x = 0; x < V; ++x) av[x] = fmaf(sh.recv_o[e0 + c][lane * V + x], f, av[x]);
-                }
-            }
-            const float inv = L > 0.f ? 1.f / L : 0.f;
-#pragma unroll
-            for (int x = 0; x < V; x += 2) {
-                __nv_bfloat162 h2 = __floats2bfloat162_rn(av[x] * inv, av[x + 1] * inv);
-                *reinterpret_cast<__nv_bfloat162 *>(o + x) = h2;
-            }
-            if (p.lse && lane == 0) p.lse[ro] = L > 0.f ? (M + log2f(L)) * kSmLn2 : -INFINITY;
+            for (int x = 0; x < V; ++x) av[x] = fmaf(recv_o[(e0 + c) * D + lane * V + x], f, av[x]);
         }
+        if (kvl < p.q_len) { L = 0.f; M = -INFINITY; }       // a sequence shorter than the query is skipped: zeros
+        const float inv = L > 0.f ? 1.f / L : 0.f;
+        __nv_bfloat16 *dst = (__nv_bfloat16 *)p.out + ro * D + lane * V;
+#pragma unroll
+        for (int x = 0; x < V; x += 2) {
+            const __nv_bfloat162 h2 = L > 0.f ? __floats2bfloat162_rn(av[x] * inv, av[x + 1] * inv) : __floats2bfloat162_rn(0.f, 0.f);
+            *reinterpret_cast<__nv_bfloat162 *>(dst + x) = h2;
+        }
+        if (p.lse && lane == 0) p.lse[ro] = L > 0.f ? (M + log2f(L)) * kSmLn2 : -INFINITY;
     }
 }
 
-// Pages of 64 keys a CTA may walk before the tensor-core kernel is the better choice (measured: beyond one page per
-// CTA, i.e. 1,024 keys with the largest cluster, the tensor-core kernel's deeper pipeline wins).
-constexpr int kSmMaxPagesPerCta = 1;
-constexpr int kSmMaxCluster = 16;
-
-bool attn_small_supported(const AttnParams &p, int dtype) {
-    if (dtype != HIPPO_DTYPE_BF16 || (p.head_dim != 64 && p.head_dim != 128) || p.rows > 8) return false;
-    const int pages = ceil_div(p.max_kv_len, kSmPage);
-    return ceil_div(pages, kSmMaxCluster) <= kSmMaxPagesPerCta && (long long)p.batch * p.n_kv_heads * kSmMaxCluster <= 65535;
+// How a call is laid out: warps per CTA, CTAs per unit (= cluster size), 32-key blocks per warp.  The fewest steps win,
+// then the fewest warps: with everything in flight at once a step costs 1.1 - 2 us, four warps instead of eight save 0.1.
+// Clusters of more than eight need most of a GPC; only six GPCs can be counted on to hold one (8 clusters of 12 CTAs with
+// an SM each ran in two waves: 1,500 keys, 8 units, head size 128: 11.3 us against 6.6 on clusters of 8).
+struct SmallPlan {
+    int warps, cluster, steps;
+};
+static SmallPlan small_plan(const AttnParams &p) {
+    const int blocks = ceil_div(p.max_kv_len, kSmBlock), units = p.batch * p.n_kv_heads;
+    const int most = p.head_dim == 64 ? kSmMaxWarps : kSmMaxWarps / 2;      // what the register file holds
+    SmallPlan best = {0, 0, 0};
+    for (int w = 4; w <= most; w *= 2) {
+        int lim = most * kNumSMs / (units * w);                              // all warps of the call resident together
+        const int widest = units * w <= 6 * most ? kSmMaxCluster : kSmMaxCluster / 2;
+        lim = lim < 1 ? 1 : lim > widest ? widest : lim;
+        const int want = ceil_div(blocks, w), cs = want < lim ? want : lim;
+        const int steps = ceil_div(blocks, w * cs);
+        if (!best.warps || steps < best.steps) best = {w, cs, steps};
+    }
+    return best;
 }
 
-template <int D, int RMAX>
+// Where this kernel ends and the tensor-memory kernel of attn_tc.cu begins, from calls of 28 layers (us per call, this one
+// against the other; one sequence unless noted).  Head size 64, 2 kv heads: 758 keys 3.8 / 8.1, 3,537 keys 4.2 / 10.2,
+// 8,000 5.8 / 12.4, 20,000 10.9 / 16.8, 33,000 (5 steps) 15.2 / 18.1; 4 kv heads 33,000 keys 15.9 / 19.1; eight sequences
+// of 4,000: 8.9 / 13.9.  Head size 128, 14 rows, 4 kv heads: 4,000 keys 8.4 / 11.8, 8,000 11.6 / 14.1, 16,000 (4 steps)
+// 18.0 / 18.5; 8 kv heads, 8,000 keys (4 steps) 18.3 / 18.7.  A caller that fixes the split of a long cache has the other
+// kernel, which can place that many CTAs on scattered SMs; up to 1,024 keys and 8 rows the request never mattered.
+bool attn_small_supported(const AttnParams &p, int dtype) {
+    if (dtype != HIPPO_DTYPE_BF16 || (p.head_dim != 64 && p.head_dim != 128) || p.rows > kSmMaxRows) return false;
+    if ((long long)p.batch * p.n_kv_heads * kSmMaxCluster > 65535) return false;
+    if (p.max_kv_len <= 1024 && p.rows <= 8) return true;
+    return p.num_splits == 0 && small_plan(p).steps <= (p.head_dim == 64 ? 5 : 3);
+}
+
+// Against the multi-layer launch, which pays its set-up once: better as long as a call is a single step (per layer, head
+// size 128: 1,000 keys, 8 rows, 8 kv heads 6.5 us against 11.0, 2,000 keys 7.3 / 8.3, 4,000 keys (2 steps) 14.0 / 8.2).
+bool attn_small_beats_layers(const AttnParams &p, int dtype) {
+    return attn_small_supported(p, dtype) && small_plan(p).steps == 1;
+}
+
+template <int D, int NT>
 static int32_t launch_small(const AttnParams &p, cudaStream_t stream) {
     static PerDeviceOnce attr_set;
     int dev;
     if (attr_set.needed(dev)) {
-        HIPPO_CUDA_TRY(cudaFuncSetAttribute(attn_small_kernel<D, RMAX>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        HIPPO_CUDA_TRY(cudaFuncSetAttribute(attn_small_kernel<D, NT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        HIPPO_CUDA_TRY(cudaFuncSetAttribute(attn_small_kernel<D, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)SmallSmem<D, NT>::bytes(kSmMaxWarps)));
         attr_set.mark(dev);
     }
-    const int pages = ceil_div(p.max_kv_len, kSmPage);
-    int cs = pages < kSmMaxCluster ? pages : kSmMaxCluster;
-    if (cs < 1) cs = 1;
+    const SmallPlan plan = small_plan(p);
+    const int warps = plan.warps;
+    int cs = plan.cluster;
     const int units = p.batch * p.n_kv_heads;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -313,27 +366,27 @@ static int32_t launch_small(const AttnParams &p, cudaStream_t stream) {
     attr[1].val.clusterDim.y = 1;
     attr[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(kSmThreads);
+    cfg.blockDim = dim3((unsigned)(32 * warps));
+    cfg.dynamicSmemBytes = SmallSmem<D, NT>::bytes(warps);
     cfg.stream = stream;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
     for (;;) {
         attr[1].val.clusterDim.x = (unsigned)cs;
         cfg.gridDim = dim3((unsigned)(units * cs));
-        const cudaError_t e = cudaLaunchKernelEx(&cfg, attn_small_kernel<D, RMAX>, p, cs);
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, attn_small_kernel<D, NT>, p, cs);
         if (e == cudaSuccess) break;
         (void)cudaGetLastError();
         if (cs <= 8) return cuda_fail(e, "attention (small) launch");
         cs = 8;   // clusters beyond the portable size are not available here
-        if (ceil_div(pages, cs) > 2 * kSmMaxPagesPerCta) return cuda_fail(e, "attention (small) launch");
     }
     count_launches(1);
     return HIPPO_OK;
 }
 
 int32_t launch_attn_small(const AttnParams &p, cudaStream_t stream) {
-    if (p.head_dim == 64) return launch_small<64, 8>(p, stream);
-    return launch_small<128, 8>(p, stream);
+    if (p.head_dim == 64) return p.rows <= 8 ? launch_small<64, 1>(p, stream) : launch_small<64, 2>(p, stream);
+    return p.rows <= 8 ? launch_small<128, 1>(p, stream) : launch_small<128, 2>(p, stream);
 }
 
 }  // namespace hippo

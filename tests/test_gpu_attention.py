@@ -207,6 +207,36 @@ def test_full_size_draft(hb, ci):
         assert_close(got, ref, TOL[cfg.dtype], "c%d draft keep %d%%" % (ci, pct))
 
 
+# (head size, q_len, query heads, kv heads, lengths): one key, edges of the 32-key blocks, of one and of several steps per
+# warp (4, 8 and 16 warps per CTA), more and fewer than eight packed rows, rows that see only part of the last block, ragged
+# batches whose short members leave CTAs idle, one more key than the longest cache of the path (the next path takes it)
+SHORT_CACHES = [(64, 1, 14, 2, [1]), (64, 1, 14, 2, [31]), (64, 2, 14, 2, [33]), (64, 1, 16, 2, [2048]), (64, 1, 16, 2, [2049]),
+                (64, 2, 16, 2, [4097]), (64, 1, 7, 1, [8193]), (64, 3, 10, 2, [40960]), (64, 3, 10, 2, [40961]), (64, 16, 1, 1, [130]),
+                (128, 4, 16, 4, [512]), (128, 2, 14, 2, [513]), (128, 2, 8, 1, [6145]), (128, 5, 3, 1, [12289]),
+                (64, 2, 14, 2, [1024, 2, 1, 65, 700, 64, 1023, 96]), (128, 3, 16, 4, [900, 3, 2, 1300]), (64, 1, 28, 4, [3000, 100, 4000, 33] * 2)]
+
+
+@pytest.mark.parametrize("D,q_len,Hq,Hkv,lens", SHORT_CACHES)
+def test_short_cache_path(hb, D, q_len, Hq, Hkv, lens):
+    """Few packed rows over short caches, with NaN in the unused slots, through shuffled pages and the identity mapping."""
+    rng = np.random.default_rng(D + q_len + Hq + sum(lens))
+    B = len(lens)
+    q = W.round_to_storage(rng.standard_normal((B, q_len, Hq, D)).astype(np.float32), "bf16")
+    k = W.round_to_storage(rng.standard_normal((B, max(lens), Hkv, D)).astype(np.float32), "bf16")
+    k *= 1.0 + (np.arange(max(lens)) // 500)[None, :, None, None] % 4          # later steps move the running maxima
+    v = W.round_to_storage(rng.standard_normal((B, max(lens), Hkv, D)).astype(np.float32), "bf16")
+    live = [b for b in range(B) if lens[b] >= q_len]
+    ref, ref_lse = oracle.attention(q[live], k[live], v[live], [lens[b] for b in live])
+    for seed in (None, 7):
+        if seed is None and B > 1:
+            continue
+        got, lse = run_case(hb, hb.hippo_draft_attention, q, k, v, lens, "bf16", shuffle_seed=seed, spare=2, fill=np.nan)
+        assert_close(got[live], ref, TOL["bf16"], "short cache")
+        assert_close(lse[live], ref_lse, 2e-3, "short cache lse")
+        for b in set(range(B)) - set(live):
+            assert np.all(got[b] == 0) and np.all(np.isneginf(lse[b]))
+
+
 @pytest.mark.parametrize("dtype,q_len,kvl", [("bf16", 6, 700), ("bf16", 1, 500), ("fp32", 3, 200)])
 def test_lengths_known_on_the_host(hb, dtype, q_len, kvl):
     """kv_len = NULL: every sequence has max_kv_len keys; same result as with the length array."""
