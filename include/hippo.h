@@ -239,7 +239,7 @@ int32_t hippo_gather_kv(int32_t n_layers, const hippo_kv_cache_t *src, size_t sr
  *            floating-point sums
  *   max_kv_len  host upper bound used to size the launch; <= max_pages_per_seq * 64
  *   softmax_scale  0 selects 1/sqrt(head_dim)
- *   num_splits  0 = automatic; > 0 asks for that many splits per kv head (ignored up to 1,024 keys and 8 packed rows)
+ *   num_splits  0 = automatic; > 0: at most that many CTAs per kv head
  *   lse      optional fp32 [batch][q_len][n_q_heads], natural-log sum of exponentials of the scaled logits
  * bf16 with head_dim 64 or 128 runs on the tensor cores with TMA-staged tiles; fp32 (any head_dim that is a
  * multiple of 32, <= 256) runs on the CUDA cores.  q_len * G <= HIPPO_MAX_PACKED_ROWS.

@@ -317,7 +317,8 @@ static SmallPlan small_plan(const AttnParams &p) {
     SmallPlan best = {0, 0, 0};
     for (int w = 4; w <= most; w *= 2) {
         int lim = most * kNumSMs / (units * w);                              // all warps of the call resident together
-        const int widest = units * w <= 6 * most ? kSmMaxCluster : kSmMaxCluster / 2;
+        int widest = units * w <= 6 * most ? kSmMaxCluster : kSmMaxCluster / 2;
+        if (p.num_splits > 0 && p.num_splits < widest) widest = p.num_splits;
         lim = lim < 1 ? 1 : lim > widest ? widest : lim;
         const int want = ceil_div(blocks, w), cs = want < lim ? want : lim;
         const int steps = ceil_div(blocks, w * cs);
@@ -330,13 +331,14 @@ static SmallPlan small_plan(const AttnParams &p) {
 // against the other; one sequence unless noted).  Head size 64, 2 kv heads: 758 keys 3.8 / 8.1, 3,537 keys 4.2 / 10.2,
 // 8,000 5.8 / 12.4, 20,000 10.9 / 16.8, 33,000 (5 steps) 15.2 / 18.1; 4 kv heads 33,000 keys 15.9 / 19.1; eight sequences
 // of 4,000: 8.9 / 13.9.  Head size 128, 14 rows, 4 kv heads: 4,000 keys 8.4 / 11.8, 8,000 11.6 / 14.1, 16,000 (4 steps)
-// 18.0 / 18.5; 8 kv heads, 8,000 keys (4 steps) 18.3 / 18.7.  A caller that fixes the split of a long cache has the other
-// kernel, which can place that many CTAs on scattered SMs; up to 1,024 keys and 8 rows the request never mattered.
+// 18.0 / 18.5; 8 kv heads, 8,000 keys (4 steps) 18.3 / 18.7.  A caller that asks for more than eight splits of a long
+// cache has the other kernel, which can place that many CTAs on scattered SMs (a cluster of more than eight beside a
+// verification pass on 96 SMs waited for its end: 32k-token step 2.36 ms against 1.57 ms on clusters of eight).
 bool attn_small_supported(const AttnParams &p, int dtype) {
     if (dtype != HIPPO_DTYPE_BF16 || (p.head_dim != 64 && p.head_dim != 128) || p.rows > kSmMaxRows) return false;
     if ((long long)p.batch * p.n_kv_heads * kSmMaxCluster > 65535) return false;
     if (p.max_kv_len <= 1024 && p.rows <= 8) return true;
-    return p.num_splits == 0 && small_plan(p).steps <= (p.head_dim == 64 ? 5 : 3);
+    return p.num_splits <= kSmMaxCluster / 2 && small_plan(p).steps <= (p.head_dim == 64 ? 5 : 3);
 }
 
 // Against the multi-layer launch, which pays its set-up once: better as long as a call is a single step (per layer, head

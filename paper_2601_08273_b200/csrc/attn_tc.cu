@@ -1433,6 +1433,10 @@ AttnLayersWsLayout attn_layers_ws_layout(int n_layers, int batch, int q_len, int
     return L;
 }
 
+// Bounded multi-layer grids are launched as clusters of eight, up to a grid of which all clusters are sure to be resident
+// together (a GPC of 16 - 20 SMs holds two: 12 clusters need six of the eight GPCs).
+constexpr int kPackCtas = 8, kPackMaxCtas = 96;
+
 template <int D>
 static int32_t launch_tc_layers(AttnParams p, int n_layers, const void *const *q, const hippo_kv_cache_t *kv, void *const *out,
                                 float *const *lse, int max_ctas, void *workspace, cudaStream_t stream) {
@@ -1488,9 +1492,13 @@ static int32_t launch_tc_layers(AttnParams p, int n_layers, const void *const *q
         if (grid > 1 && a == 1) { mc.rot = cand % grid; break; }
     }
     HIPPO_CUDA_TRY(cudaMemsetAsync(mc.done, 0, L.done_bytes, stream));
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = kPackCtas;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(kTcThreads + 32);
     cfg.gridDim = dim3((unsigned)grid);
@@ -1498,6 +1506,10 @@ static int32_t launch_tc_layers(AttnParams p, int n_layers, const void *const *q
     cfg.stream = stream;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    // A caller that bounds the grid means to run something beside it.  Spread over all GPCs the CTAs leave a few SMs in
+    // each, where no cluster of a draft call fits; launched as clusters (of which the kernel makes no use) they fill whole
+    // GPCs and leave whole ones.  32k-token step, grid 96, draft calls as clusters of 8: 2.06 ms spread, 1.57 ms packed.
+    if (max_ctas > 0 && max_ctas <= kPackMaxCtas && grid % kPackCtas == 0) cfg.numAttrs = 2;
     for (int l0 = 0; l0 < n_layers; l0 += NL) {
         LayerSetT<NL> set;
         memset(&set, 0, sizeof(set));

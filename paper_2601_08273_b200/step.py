@@ -41,8 +41,8 @@ class HippoStep:
         #   verify_max_ctas       grid bound of the multi-layer verification kernel; the SMs it leaves free are where the
         #                         draft stream's kernels run (a persistent CTA holds all of its SM's shared memory)
         #   verify_beside_select  True: verification is forked first and also runs beside select and gather
-        #   draft_num_splits      work split of the draft attention calls (0: automatic, which may pick clusters of up to 16
-        #                         CTAs that do not fit into a few scattered free SMs)
+        #   draft_num_splits      most CTAs per kv head of a draft attention call (0: automatic, up to clusters of 16, which
+        #                         find no room beside a verification pass)
         self.verify_max_ctas = verify_max_ctas
         self.verify_beside_select = False
         self.draft_num_splits = 0
@@ -129,16 +129,17 @@ class HippoStep:
         self.stream_d = torch.cuda.Stream(device=self.device)
         self.stream_v = torch.cuda.Stream(device=self.device)
         if verify_max_ctas == 0 and multi_layer_verify:
-            # Default sharing, from the two legs' sizes: when the draft leg (latency-bound calls, about 10 us each) outlasts the
-            # verification leg (bandwidth-bound), verification gives up 84 of the 148 SMs to it; measured on B200 this takes
-            # the 6k-token step from 1.55 ms to 1.12 ms and the 32k-token step from 3.52 ms to 3.03 ms.  When verification is
-            # the longer leg (64k tokens, 80 layers) it keeps every SM: the draft calls then run in its shadow or after it,
-            # and holding SMs back only slows the step down (7.05 ms against 7.37 ms with 116 CTAs).
+            # Default sharing, from the two legs' sizes.  A draft call (latency-bound, about 4.5 us) finds no SM beside a
+            # verification pass on all of them, so the legs add up; on 96 SMs verification (bandwidth-bound) is 1.3 times as
+            # long and the draft calls run beside it.  Measured on B200, 32k tokens, 96 against all SMs: 7 draft tokens
+            # 1.57 ms / 2.12, 3 draft tokens (the draft leg 0.44 of the verification leg) 1.41 / 1.56; 64k tokens with 80
+            # target layers (0.24) 6.11 / 5.39.
             verify_s = self.verify_kv_bytes_per_layer() * self.Lt / 5.4e12
-            draft_s = g * self.Ld * 10e-6
-            if draft_s > verify_s:
-                self.verify_max_ctas = 64
-        self.draft_num_splits = 16 if max(self.n_keep) + g > 1024 and B * h <= 4 else 0
+            draft_s = g * self.Ld * 4.5e-6
+            if draft_s > 0.33 * verify_s:
+                self.verify_max_ctas = 96
+        if self.verify_max_ctas:
+            self.draft_num_splits = 8
 
     # ---- algorithmic bytes (the roofline numerators) ------------------------------------------------------------
     @property
