@@ -11,8 +11,8 @@
 // depends on the final rounding of the fused score to fp32.
 //
 // Kernels:  dots (norms + next-frame dot, one warp per token)  ->  spatial (one CTA per crop, fp64 tensor instructions)  ->
-//           fuse (one CTA per frame: s_temp, three standardisations, sum)  ->  topk (one CTA per sequence,
-//           bisection on order-preserving keys, ordered compaction).
+//           fuse (one CTA per frame: s_temp, three standardisations, sum)  ->  topk (one cluster of CTAs per
+//           sequence, histograms of the digits of order-preserving keys, ordered compaction).
 //
 // hippo_select_tokens_policy adds the selection rules the paper compares itself with, as rules only: a uniform budget
 // per frame (the attention-guided uniform pruning of earlier video speculative decoding, related-work section), the k
@@ -23,6 +23,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace hippo {
 
@@ -51,18 +52,6 @@ __device__ __forceinline__ double ld_as_double(const __nv_bfloat16 *p, size_t i)
 __device__ __forceinline__ double warp_sum(double v) {
     for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
-}
-
-// Sum over the block, result valid in every thread.  Fixed reduction order.
-__device__ double block_sum(double v, double *scratch /* [32] shared */) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    v = warp_sum(v);
-    __syncthreads();
-    if (lane == 0) scratch[warp] = v;
-    __syncthreads();
-    double t = 0.0;
-    for (int w = 0; w < nw; ++w) t += scratch[w];
-    return t;
 }
 
 __device__ __forceinline__ int find_seq(const int *off, int n, int x) {  // largest b with off[b] <= x
@@ -354,17 +343,26 @@ __global__ void __launch_bounds__(kMmaThreads, 3) select_spatial_mma_kernel(cons
 }
 
 // ---- per-frame standardisation and fusion: one CTA per frame ---------------------------------------------------
-__device__ double standardise(double x, bool valid, int n, double *scratch) {
-    const double mu = block_sum(valid ? x : 0.0, scratch) / n;
-    const double dv = valid ? x - mu : 0.0;
-    const double var = block_sum(dv * dv, scratch) / n;
-    const double floor_ = 1e-24 * fmax(1.0, mu * mu);
-    if (var <= floor_) return 0.0;
-    return dv / sqrt(var);
+// Sums of three values over the block, the results valid in every thread.  Fixed reduction order.
+__device__ __forceinline__ void block_sum3(double (&v)[3], double (*scratch)[3] /* [32] shared */) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) v[i] = warp_sum(v[i]);
+    if (lane == 0)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) scratch[warp][i] = v[i];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 3; ++i) v[i] = 0.0;
+    for (int w = 0; w < nw; ++w)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) v[i] += scratch[w][i];
 }
 
+// Bound: latency (loads, then two reductions).  The three terms go through the two reductions (mean, variance) together
+// instead of one term after the other.
 __global__ void __launch_bounds__(1024) select_fuse_kernel(const SelectParams p) {
-    __shared__ double scratch[32];
+    __shared__ double scratch[2][32][3];
     const int gframe = blockIdx.x;
     const int b = find_seq(p.frame_off, p.batch, gframe);
     const int f = gframe - p.frame_off[b];
@@ -375,12 +373,13 @@ __global__ void __launch_bounds__(1024) select_fuse_kernel(const SelectParams p)
     const int c = threadIdx.x;
     const bool valid = c < nf;
     const int j = p.seq_off[b] + f * p.tpf + c;
-    double fused = 0.0;
-    if (p.mask & HIPPO_SCORE_ATTN) fused += standardise(valid ? (double)p.attn_mass[j] : 0.0, valid, nf, scratch);
-    if (p.mask & HIPPO_SCORE_SPA) fused += standardise(valid ? p.s_spa[j] : 0.0, valid, nf, scratch);
-    if (p.mask & HIPPO_SCORE_TEMP) {
-        double st = 0.0;
-        if (valid) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    double x[3] = {0.0, 0.0, 0.0};
+    if (valid) {
+        if (p.mask & HIPPO_SCORE_ATTN) x[0] = (double)p.attn_mass[j];
+        if (p.mask & HIPPO_SCORE_SPA) x[1] = p.s_spa[j];
+        if (p.mask & HIPPO_SCORE_TEMP) {
             double sum = 0.0;
             int cnt = 0;
             const double nj = p.norm2[j];
@@ -394,220 +393,160 @@ __global__ void __launch_bounds__(1024) select_fuse_kernel(const SelectParams p)
                 sum += (nj > 0.0 && nk > 0.0) ? p.tdot[j] / (sqrt(nj) * sqrt(nk)) : 0.0;
                 ++cnt;
             }
-            st = 1.0 - (cnt ? sum / cnt : 0.0);
+            x[2] = 1.0 - (cnt ? sum / cnt : 0.0);
         }
-        fused += standardise(st, valid, nf, scratch);
+    }
+    double mu[3] = {x[0], x[1], x[2]}, dv[3], var[3];
+    block_sum3(mu, scratch[0]);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        mu[i] /= nf;
+        dv[i] = valid ? x[i] - mu[i] : 0.0;
+        var[i] = dv[i] * dv[i];
+    }
+    block_sum3(var, scratch[1]);
+    double fused = 0.0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const unsigned bit = i == 0 ? HIPPO_SCORE_ATTN : i == 1 ? HIPPO_SCORE_SPA : HIPPO_SCORE_TEMP;
+        var[i] /= nf;
+        const double floor_ = 1e-24 * fmax(1.0, mu[i] * mu[i]);
+        if ((p.mask & bit) && !(var[i] <= floor_)) fused += dv[i] / sqrt(var[i]);
     }
     if (valid) p.fused[j] = (float)fused;
 }
 
-// ---- top-k: one CTA per sequence --------------------------------------------------------------------------------
+// ---- top-k: one cluster of CTAs per sequence ----------------------------------------------------------------------
 __device__ __forceinline__ uint32_t order_key(float x) {  // larger float -> larger key
     const uint32_t u = __float_as_uint(x);
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// smem_keys: keys beyond the 32 per thread that live in registers are staged in this many words of dynamic shared memory
-__global__ void __launch_bounds__(1024) select_topk_kernel(const SelectParams p, const int smem_keys) {
-    extern __shared__ uint32_t skeys[];
-    __shared__ int warp_cnt[32];
-    __shared__ uint32_t s_prefix;
-    __shared__ int s_remaining, s_base_eq, s_base_out;
-    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int n = p.seq_off[b + 1] - p.seq_off[b];
-    const int k = p.k[b];
-    if (k <= 0) return;
+// A sequence's keys are dealt to the CTAs of a cluster in contiguous shares, to a CTA's threads in groups of eight neighbours
+// (a share of more than one round is read again per pass).  The key T of the k-th largest element comes from three histogram
+// passes over its digits (11, 11 and 10 bits, top first): every CTA counts its own keys that agree with T so far, reads the
+// others' counts through distributed shared memory and finds the digit by a scan of its own.  Then one scan of the pairs
+// (keys > T, keys == T) gives every thread its first output position: the kept ones among the equal are those with the lowest
+// indices, so position = (larger ones before) + min(equal ones before, equal ones to keep).
+// Bound: latency (three passes of count, exchange, scan).  65,536 tokens 28 us, 160 us with one CTA and two bits per step (three
+// block barriers each, keys beyond 32 per thread in shared memory); 6,272 tokens 19 us, 27 us.
+constexpr int kTopThreads = 1024, kTopPerThread = 8, kTopTile = kTopThreads * kTopPerThread, kTopBins = 2048;
+
+__global__ void __launch_bounds__(kTopThreads, 1) select_topk_kernel(const SelectParams p, const int cluster) {
+    __shared__ uint32_t hist[3][kTopBins];       // one per pass: peers may still read the one before
+    __shared__ uint32_t wsum[32], s_digit, s_above;
+    __shared__ unsigned long long w64[32];
+    __shared__ unsigned long long share_total;   // this CTA's (keys > T) << 32 | (keys == T)
+    const int b = blockIdx.x / cluster, rank = blockIdx.x % cluster, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int n = p.seq_off[b + 1] - p.seq_off[b], k = p.k[b];
+    for (int i = tid; i < 3 * kTopBins; i += kTopThreads) (&hist[0][0])[i] = 0;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const float *score = p.fused + p.seq_off[b];
     int32_t *out = p.kept + p.k_off[b];
-    // The key T of the k-th largest element, two bits at a time from the top: T is the largest value with at least k
-    // keys >= T.  Each thread keeps its keys in registers (32 per thread), the next ones in shared memory, and only
-    // what is left beyond both is read again from memory, so a step is a few compares and one block-wide sum of three
-    // counters.
-    constexpr int kKeysPerThread = 32;
-    __shared__ int warp_cnt3[32][3];
-    __shared__ int s_cnt3[3];
-    uint32_t keys[kKeysPerThread];
-    const int n_regs = kKeysPerThread * (int)blockDim.x;            // keys [0, n_regs) in registers
-    const int n_staged = min(n, n_regs + smem_keys);                 // keys [n_regs, n_staged) in shared memory
+    if (k <= 0) return;                           // the same for the whole cluster
+    const int begin = (int)((long long)n * rank / cluster), end = (int)((long long)n * (rank + 1) / cluster);
+    const int rounds = (end - begin + kTopTile - 1) / kTopTile;
+    uint32_t key[kTopPerThread];
+    auto load = [&](int round) {
 #pragma unroll
-    for (int e = 0; e < kKeysPerThread; ++e) {
-        const int i = e * blockDim.x + tid;
-        keys[e] = i < n ? order_key(score[i]) : 0u;   // padding: key 0 is never counted (candidates are > 0)
-    }
-    for (int i = n_regs + tid; i < n_staged; i += blockDim.x) skeys[i - n_regs] = order_key(score[i]);
+        for (int e = 0; e < kTopPerThread; ++e) {
+            const int i = begin + round * kTopTile + tid * kTopPerThread + e;
+            key[e] = i < end ? order_key(score[i]) : 0u;
+        }
+    };
+    auto live = [&](int round, int e) { return begin + round * kTopTile + tid * kTopPerThread + e < end; };
+    load(0);
     __syncthreads();
-    const int per_thread = min(kKeysPerThread, (n + (int)blockDim.x - 1) / (int)blockDim.x);
-    // counts of keys >= c1, >= c2, >= c3 over the sequence (candidates are non-zero)
-    auto count3 = [&](uint32_t c1, uint32_t c2, uint32_t c3) {
-        int a1 = 0, a2 = 0, a3 = 0;
+    uint32_t T = 0, mask = 0;
+    int need = k;                                 // the wanted element is the need-th largest among the keys that agree with T so far
 #pragma unroll
-        for (int e0 = 0; e0 < kKeysPerThread; e0 += 8) {
-            if (e0 < per_thread) {      // uniform: only the groups of eight that hold keys
+    for (int pass = 0; pass < 3; ++pass) {
+        const int shift = pass == 0 ? 21 : pass == 1 ? 10 : 0;
+        const uint32_t digits = pass == 2 ? 1023u : 2047u;
+        for (int r = 0; r < rounds; ++r) {
+            if (rounds > 1) load(r);
 #pragma unroll
-                for (int e = e0; e < e0 + 8; ++e) {
-                    a1 += keys[e] >= c1 ? 1 : 0; a2 += keys[e] >= c2 ? 1 : 0; a3 += keys[e] >= c3 ? 1 : 0;
+            for (int e = 0; e < kTopPerThread; ++e)
+                if (live(r, e) && (key[e] & mask) == T) atomicAdd(&hist[pass][(key[e] >> shift) & digits], 1u);
+        }
+        if (cluster > 1) cluster_sync_all(); else __syncthreads();
+        // counts over the cluster and their sums from the top: thread t owns the bins 2 t, 2 t + 1 counted from the top
+        uint32_t c[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int bin = kTopBins - 1 - (2 * tid + h);
+            c[h] = hist[pass][bin];
+            for (int q = 1; q < cluster; ++q)
+                c[h] += ld_cluster_u32(cluster_map(smem_u32(&hist[pass][bin]), (uint32_t)((rank + q) % cluster)));
+        }
+        uint32_t inc = c[0] + c[1];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += v; }
+        if (lane == 31) wsum[warp] = inc;
+        __syncthreads();
+        if (warp == 0) {
+            uint32_t v = wsum[lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { const uint32_t w = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += w; }
+            wsum[lane] = v;
+        }
+        __syncthreads();
+        uint32_t before = (warp ? wsum[warp - 1] : 0u) + inc - c[0] - c[1];      // keys in higher bins
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (before < (uint32_t)need && (uint32_t)need <= before + c[h]) { s_digit = (uint32_t)(kTopBins - 1 - (2 * tid + h)); s_above = before; }
+            before += c[h];
+        }
+        __syncthreads();
+        T |= s_digit << shift;
+        mask |= digits << shift;
+        need -= (int)s_above;                     // after the last pass: elements equal to T to keep
+    }
+    unsigned long long base = 0;                  // (larger, equal) in front of this CTA's share
+    for (int ph = cluster > 1 ? 0 : 1; ph < 2; ++ph) {
+        // first the share's totals (only where there are other shares), then the output
+        unsigned long long run = ph ? base : 0;
+        for (int r = 0; r < rounds; ++r) {
+            if (rounds > 1) load(r);
+            unsigned long long mine = 0;
+#pragma unroll
+            for (int e = 0; e < kTopPerThread; ++e)
+                if (live(r, e)) mine += key[e] > T ? 1ull << 32 : key[e] == T ? 1ull : 0ull;
+            unsigned long long inc = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { const unsigned long long v = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += v; }
+            __syncthreads();                      // w64 of the round before has been read
+            if (lane == 31) w64[warp] = inc;
+            __syncthreads();
+            unsigned long long at = run + inc - mine, all = 0;
+            for (int w = 0; w < kTopThreads / 32; ++w) {
+                const unsigned long long v = w64[w];
+                at += w < warp ? v : 0ull;
+                all += v;
+            }
+            run += all;
+            if (ph) {
+                uint32_t gt = (uint32_t)(at >> 32), eq = (uint32_t)at;
+#pragma unroll
+                for (int e = 0; e < kTopPerThread; ++e) {
+                    if (!live(r, e)) continue;
+                    const bool g = key[e] > T, q = key[e] == T;
+                    if (g || (q && eq < (uint32_t)need)) out[gt + min(eq, (uint32_t)need)] = begin + r * kTopTile + tid * kTopPerThread + e;
+                    gt += g; eq += q;
                 }
             }
         }
-        for (int i = n_regs + tid; i < n_staged; i += blockDim.x) {
-            const uint32_t key = skeys[i - n_regs];
-            a1 += key >= c1 ? 1 : 0; a2 += key >= c2 ? 1 : 0; a3 += key >= c3 ? 1 : 0;
-        }
-        for (int i = n_staged + tid; i < n; i += blockDim.x) {
-            const uint32_t key = order_key(score[i]);
-            a1 += key >= c1 ? 1 : 0; a2 += key >= c2 ? 1 : 0; a3 += key >= c3 ? 1 : 0;
-        }
-        a1 = __reduce_add_sync(0xffffffffu, a1);
-        a2 = __reduce_add_sync(0xffffffffu, a2);
-        a3 = __reduce_add_sync(0xffffffffu, a3);
-        __syncthreads();                 // the counters of the previous step have been read
-        if (lane == 0) { warp_cnt3[warp][0] = a1; warp_cnt3[warp][1] = a2; warp_cnt3[warp][2] = a3; }
-        __syncthreads();
-        if (warp == 0) {
-            const bool has = lane < (int)(blockDim.x >> 5);
-            int t1 = has ? warp_cnt3[lane][0] : 0, t2 = has ? warp_cnt3[lane][1] : 0, t3 = has ? warp_cnt3[lane][2] : 0;
-            t1 = __reduce_add_sync(0xffffffffu, t1);
-            t2 = __reduce_add_sync(0xffffffffu, t2);
-            t3 = __reduce_add_sync(0xffffffffu, t3);
-            if (lane == 0) { s_cnt3[0] = t1; s_cnt3[1] = t2; s_cnt3[2] = t3; }
-        }
-        __syncthreads();
-    };
-    uint32_t Tsel = 0;
-    for (int bit = 30; bit >= 0; bit -= 2) {
-        // candidates with the two bits set to 01, 10, 11 (ascending): keep the largest that still has k keys above it
-        const uint32_t c1 = Tsel | (1u << bit), c2 = Tsel | (2u << bit), c3 = Tsel | (3u << bit);
-        count3(c1, c2, c3);
-        if (s_cnt3[2] >= k) Tsel = c3; else if (s_cnt3[1] >= k) Tsel = c2; else if (s_cnt3[0] >= k) Tsel = c1;
-    }
-    int n_gt = 0;
-    if (Tsel != 0xffffffffu) { count3(Tsel + 1, Tsel + 1, Tsel + 1); n_gt = s_cnt3[0]; }
-    __syncthreads();
-    if (tid == 0) { s_prefix = Tsel; s_remaining = k - n_gt; }
-    __syncthreads();
-    const uint32_t T = s_prefix;
-    const int need_eq = s_remaining;  // elements equal to T to keep: those with the smallest indices
-    if (tid == 0) { s_base_eq = 0; s_base_out = 0; }
-    __syncthreads();
-    // Ordered compaction.  Element i = e * blockDim.x + tid of the first n_regs sits in this thread's register e, so the
-    // output position of a kept element is (kept elements of rows e' < e) + (kept elements of row e in lower threads).
-    // Three sweeps over the registers, ballots only, and two scans of the 32 x 32 table of per-(row, warp) counts in
-    // between: first the ranks of the elements equal to the threshold (only the need_eq lowest indices among them are
-    // kept), then the output positions.
-    __shared__ int cnt[32][33];
-    __shared__ int row_tot[32];
-    const int nw = blockDim.x >> 5;
-    const int rows_used = min(kKeysPerThread, (n + (int)blockDim.x - 1) / (int)blockDim.x);
-    // exclusive scan of cnt[e][w] in (e, w) order, in place; returns the grand total through row_tot[31]
-    auto scan_counts = [&]() {
-        __syncthreads();
-        if (warp < rows_used) {
-            const int c = lane < nw ? cnt[warp][lane] : 0;
-            int inc = c;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += v; }
-            cnt[warp][lane] = inc - c;
-            if (lane == 31) row_tot[warp] = inc;
-        } else if (lane == 31) {
-            row_tot[warp] = 0;
-        }
-        __syncthreads();
-        if (warp == 0) {
-            const int c = row_tot[lane];
-            int inc = c;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += v; }
-            row_tot[lane] = inc - c;
-            if (lane == 31) s_base_eq = inc;      // scratch: the grand total
-        }
-        __syncthreads();
-    };
-    const unsigned lt_mask = (1u << lane) - 1;
-#pragma unroll
-    for (int e = 0; e < kKeysPerThread; ++e) {
-        if (e < rows_used) {   // uniform
-            const unsigned bal = __ballot_sync(0xffffffffu, e * (int)blockDim.x + tid < n && keys[e] == T);
-            if (lane == 0) cnt[e][warp] = __popc(bal);
+        if (!ph) {
+            if (tid == 0) share_total = run;
+            cluster_sync_all();
+            for (int q = 0; q < rank; ++q) {
+                unsigned long long v;
+                asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(cluster_map(smem_u32(&share_total), (uint32_t)q)) : "memory");
+                base += v;
+            }
         }
     }
-    scan_counts();
-    const int eq_in_regs = s_base_eq;
-    __syncthreads();
-    __shared__ int eq_off[32][33];
-    __shared__ int eq_row[32];
-    for (int x = tid; x < 32 * 32; x += blockDim.x) eq_off[x >> 5][x & 31] = cnt[x >> 5][x & 31];
-    if (tid < 32) eq_row[tid] = row_tot[tid];
-    __syncthreads();
-#pragma unroll
-    for (int e = 0; e < kKeysPerThread; ++e) {
-        if (e < rows_used) {
-            const bool in = e * (int)blockDim.x + tid < n;
-            const bool eq = in && keys[e] == T, gt = in && keys[e] > T;
-            const unsigned bal_eq = __ballot_sync(0xffffffffu, eq);
-            const int rank = eq_row[e] + eq_off[e][warp] + __popc(bal_eq & lt_mask);
-            const unsigned bal = __ballot_sync(0xffffffffu, gt || (eq && rank < need_eq));
-            if (lane == 0) cnt[e][warp] = __popc(bal);
-        }
-    }
-    scan_counts();
-    const int out_in_regs = s_base_eq;
-    __syncthreads();
-#pragma unroll
-    for (int e = 0; e < kKeysPerThread; ++e) {
-        if (e < rows_used) {
-            const int i = e * (int)blockDim.x + tid;
-            const bool in = i < n;
-            const bool eq = in && keys[e] == T, gt = in && keys[e] > T;
-            const unsigned bal_eq = __ballot_sync(0xffffffffu, eq);
-            const int rank = eq_row[e] + eq_off[e][warp] + __popc(bal_eq & lt_mask);
-            const bool sel = gt || (eq && rank < need_eq);
-            const unsigned bal = __ballot_sync(0xffffffffu, sel);
-            const int pos = row_tot[e] + cnt[e][warp] + __popc(bal & lt_mask);
-            if (sel && pos < k) out[pos] = i;
-        }
-    }
-    __syncthreads();
-    if (tid == 0) { s_base_eq = eq_in_regs; s_base_out = out_in_regs; }
-    __syncthreads();
-    // what lies beyond the registers (more than 32 keys per thread): blockDim.x elements at a time, ranks from ballots,
-    // warp offsets from a scan by warp 0
-    __shared__ int tail_eq_off[33], sel_off[33];
-    for (int start = n_regs; start < n; start += blockDim.x) {
-        const int i = start + tid;
-        const uint32_t key = i < n ? order_key(score[i]) : 0u;
-        const bool gt = i < n && key > T, eq = i < n && key == T;
-        const unsigned bal_eq = __ballot_sync(0xffffffffu, eq);
-        if (lane == 0) warp_cnt[warp] = __popc(bal_eq);
-        __syncthreads();
-        if (warp == 0) {
-            const int c = lane < nw ? warp_cnt[lane] : 0;
-            int inc = c;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += v; }
-            tail_eq_off[lane] = inc - c;
-            if (lane == 31) tail_eq_off[32] = inc;
-        }
-        __syncthreads();
-        const int eq_rank2 = s_base_eq + tail_eq_off[warp] + __popc(bal_eq & lt_mask);
-        const bool sel = gt || (eq && eq_rank2 < need_eq);
-        const unsigned bal = __ballot_sync(0xffffffffu, sel);
-        if (lane == 0) warp_cnt[warp] = __popc(bal);
-        __syncthreads();
-        if (warp == 0) {
-            const int c = lane < nw ? warp_cnt[lane] : 0;
-            int inc = c;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += v; }
-            sel_off[lane] = inc - c;
-            if (lane == 31) sel_off[32] = inc;
-        }
-        __syncthreads();
-        const int pos = s_base_out + sel_off[warp] + __popc(bal & lt_mask);
-        if (sel && pos < k) out[pos] = i;
-        __syncthreads();
-        if (tid == 0) { s_base_eq += tail_eq_off[32]; s_base_out += sel_off[32]; }
-        __syncthreads();
-    }
+    if (cluster > 1) cluster_sync_all();          // nobody leaves while its shared memory may be read
 }
 
 // ---- uniform budget per frame ------------------------------------------------------------------------------------
@@ -683,6 +622,25 @@ __global__ void select_frames_kernel(const SelectParams p) {
 __global__ void select_copy_keys_kernel(const float *keys, float *fused, int n) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) fused[i] = keys[i];
+}
+
+// A kernel that begins with griddepcontrol.wait: its launch overlaps the end of its predecessor in the stream.
+template <typename... Args>
+static cudaError_t launch_dependent(void (*kernel)(Args...), int grid, int threads, int cluster, cudaStream_t s, Args... args) {
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 struct SelectWs { size_t norm2_off, tdot_off, spa_off, budget_off, total; };
@@ -810,7 +768,7 @@ int32_t hippo_select_tokens_policy(int32_t batch, const int32_t *n_visual, int32
     }
     const int fuse_threads = ((p.tpf + 31) / 32) * 32;
     if (scored) {
-        select_fuse_kernel<<<(unsigned)frames, fuse_threads, 0, s>>>(p);
+        HIPPO_CUDA_TRY(launch_dependent(select_fuse_kernel, (int)frames, fuse_threads, 1, s, p));
         count_launches(1);
     }
     if (ksum > 0 && policy == HIPPO_SELECT_UNIFORM_PER_FRAME) {
@@ -818,18 +776,12 @@ int32_t hippo_select_tokens_policy(int32_t batch, const int32_t *n_visual, int32
         select_frame_topk_kernel<<<(unsigned)frames, fuse_threads, 0, s>>>(p);
         count_launches(2);
     } else if (ksum > 0) {
-        // shared-memory staging for the keys beyond 32 per thread, up to 48K of them
+        // half of the threads' key registers in use: 8 CTAs from 16k tokens on
         int longest = 0;
         for (int b = 0; b < batch; ++b) longest = n_visual[b] > longest ? n_visual[b] : longest;
-        int smem_keys = longest - 32 * 1024;
-        smem_keys = smem_keys < 0 ? 0 : (smem_keys > 48 * 1024 ? 48 * 1024 : smem_keys);
-        static PerDeviceOnce topk_attr;
-        int dev;
-        if (topk_attr.needed(dev)) {
-            HIPPO_CUDA_TRY(cudaFuncSetAttribute(select_topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 48 * 1024 * 4));
-            topk_attr.mark(dev);
-        }
-        select_topk_kernel<<<batch, 1024, (size_t)smem_keys * 4, s>>>(p, smem_keys);
+        int cluster = 1;
+        while (cluster < 8 && longest > cluster * kTopTile / 2) cluster *= 2;
+        HIPPO_CUDA_TRY(launch_dependent(select_topk_kernel, batch * cluster, kTopThreads, cluster, s, p, cluster));
         count_launches(1);
     }
     HIPPO_CUDA_TRY(cudaGetLastError());

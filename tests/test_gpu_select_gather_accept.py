@@ -177,6 +177,22 @@ def test_select_policies_ragged_batch_with_partial_frames(hb):
             np.testing.assert_array_equal(host(fused), keys)
 
 
+@pytest.mark.parametrize("lens", [[1], [7], [4096], [4097, 300, 2], [16385], [65536], [140001, 5]])
+def test_topk_sizes_and_ties(hb, lens):
+    """The k best keys at the edges of the cluster sizes and of a CTA's share, with distinct, few-valued and all-equal keys."""
+    rng = np.random.default_rng(sum(lens))
+    for levels in (0, 5, 1):
+        keys = [rng.standard_normal(n).astype(np.float32) if levels == 0 else (rng.integers(levels, size=n) - 2).astype(np.float32) for n in lens]
+        for share in (0.0, 0.1, 0.5, 1.0):
+            ks = [int(round(n * share)) for n in lens]
+            kept, _ = hb.hippo_select_tokens(None, None, lens, ks, 14, 14, policy=hb.HIPPO_SELECT_RANDOM, random_keys=dev(np.concatenate(keys)))
+            kept, at = host(kept), 0
+            for key, k in zip(keys, ks):
+                want = np.sort(np.argsort(-key, kind="stable")[:k])
+                np.testing.assert_array_equal(kept[at:at + k], want)
+                at += k
+
+
 def test_select_random_and_frames_need_no_embeddings(hb):
     cfg = W.CONFIGS[2]
     n, tpf = W.visual_lengths(cfg)[0], cfg.tokens_per_frame
