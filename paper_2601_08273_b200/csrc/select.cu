@@ -7,12 +7,13 @@
 //
 // The standardisation of s_spa divides by a sigma of ~1e-4 on near-orthogonal embeddings, which magnifies any
 // rounding in the Gram entries by four orders of magnitude.  All dot products, crop statistics and frame
-// statistics are therefore accumulated in fp64 (bf16 x bf16 products are exact in fp64), so the kept set only
+// statistics therefore have the accuracy of fp64 sums (bf16 x bf16 products are exact in fp64), so the kept set only
 // depends on the final rounding of the fused score to fp32.
 //
-// Kernels:  dots (norms + next-frame dot, one warp per token)  ->  spatial (one CTA per crop, fp64 tensor instructions)  ->
-//           fuse (one CTA per frame: s_temp, three standardisations, sum)  ->  topk (one cluster of CTAs per
-//           sequence, histograms of the digits of order-preserving keys, ordered compaction).
+// Kernels:  bf16: gram (select_gram.cu: norms, next-frame dots and spatial scores from integer tensor instructions);
+//           fp32 and small bf16 calls: dots (norms + next-frame dot, one warp per token) -> spatial (one CTA per crop, fp64
+//           tensor instructions);  then fuse (one CTA per frame: s_temp, three standardisations, sum) -> topk (one cluster of
+//           CTAs per sequence, histograms of the digits of order-preserving keys, ordered compaction).
 //
 // hippo_select_tokens_policy adds the selection rules the paper compares itself with, as rules only: a uniform budget
 // per frame (the attention-guided uniform pruning of earlier video speculative decoding, related-work section), the k
@@ -22,29 +23,10 @@
 
 #include <type_traits>
 
-#include "common.cuh"
+#include "select.cuh"
 #include "tc_ptx.cuh"
 
 namespace hippo {
-
-constexpr int kMaxCrop = 32;       // tokens per crop
-constexpr int kSelMaxBatch = 64;   // sequences per call (kernel-parameter tables)
-
-struct SelectParams {
-    const void *embeds;
-    const float *attn_mass;
-    float *fused;
-    int32_t *kept;
-    double *norm2, *tdot, *s_spa;   // [total tokens]
-    int batch, grid_h, grid_w, crop_h, crop_w, d, tpf, crops_y, crops_x;
-    unsigned mask;
-    int seq_off[kSelMaxBatch + 1];    // token offset of each sequence
-    int frame_off[kSelMaxBatch + 1];  // frame offset of each sequence
-    int k[kSelMaxBatch];
-    int k_off[kSelMaxBatch + 1];
-    int *frame_budget;               // per-frame policy: [frames] tokens kept / [frames] first output position
-    int *frame_out;
-};
 
 __device__ __forceinline__ double ld_as_double(const float *p, size_t i) { return (double)p[i]; }
 __device__ __forceinline__ double ld_as_double(const __nv_bfloat16 *p, size_t i) { return (double)__bfloat162float(p[i]); }
@@ -52,12 +34,6 @@ __device__ __forceinline__ double ld_as_double(const __nv_bfloat16 *p, size_t i)
 __device__ __forceinline__ double warp_sum(double v) {
     for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
-}
-
-__device__ __forceinline__ int find_seq(const int *off, int n, int x) {  // largest b with off[b] <= x
-    int b = 0;
-    while (b + 1 < n && off[b + 1] <= x) ++b;
-    return b;
 }
 
 // ---- norms and the dot product with the same cell of the next frame ------------------------------------------
@@ -428,18 +404,23 @@ __device__ __forceinline__ uint32_t order_key(float x) {  // larger float -> lar
 // others' counts through distributed shared memory and finds the digit by a scan of its own.  Then one scan of the pairs
 // (keys > T, keys == T) gives every thread its first output position: the kept ones among the equal are those with the lowest
 // indices, so position = (larger ones before) + min(equal ones before, equal ones to keep).
-// Bound: latency (three passes of count, exchange, scan).  65,536 tokens 28 us, 160 us with one CTA and two bits per step (three
-// block barriers each, keys beyond 32 per thread in shared memory); 6,272 tokens 19 us, 27 us.
+// Bound: latency (three passes of count, exchange, scan).  65,536 tokens 20 us, 160 us with one CTA and two bits per step (three
+// block barriers each, keys beyond 32 per thread in shared memory); 28 us with the remote counts loaded one after the other.
 constexpr int kTopThreads = 1024, kTopPerThread = 8, kTopTile = kTopThreads * kTopPerThread, kTopBins = 2048;
 
 __global__ void __launch_bounds__(kTopThreads, 1) select_topk_kernel(const SelectParams p, const int cluster) {
-    __shared__ uint32_t hist[3][kTopBins];       // one per pass: peers may still read the one before
+    // one histogram per pass, since peers may still read the one before.  The first digit (sign, exponent, two bits) of most keys
+    // falls into a few bins, so it is counted in four copies, lane modulo 4.
+    __shared__ __align__(16) uint32_t copies[kTopBins * 4];
+    __shared__ uint32_t hist1[kTopBins], hist2[kTopBins / 2];
+    uint32_t *hist0 = copies;
     __shared__ uint32_t wsum[32], s_digit, s_above;
     __shared__ unsigned long long w64[32];
     __shared__ unsigned long long share_total;   // this CTA's (keys > T) << 32 | (keys == T)
     const int b = blockIdx.x / cluster, rank = blockIdx.x % cluster, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = p.seq_off[b + 1] - p.seq_off[b], k = p.k[b];
-    for (int i = tid; i < 3 * kTopBins; i += kTopThreads) (&hist[0][0])[i] = 0;
+    for (int i = tid; i < kTopBins; i += kTopThreads) { reinterpret_cast<uint4 *>(hist0)[i] = make_uint4(0, 0, 0, 0); hist1[i] = 0; }
+    hist2[tid] = 0;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const float *score = p.fused + p.seq_off[b];
     int32_t *out = p.kept + p.k_off[b];
@@ -459,26 +440,44 @@ __global__ void __launch_bounds__(kTopThreads, 1) select_topk_kernel(const Selec
     __syncthreads();
     uint32_t T = 0, mask = 0;
     int need = k;                                 // the wanted element is the need-th largest among the keys that agree with T so far
-#pragma unroll
-    for (int pass = 0; pass < 3; ++pass) {
-        const int shift = pass == 0 ? 21 : pass == 1 ? 10 : 0;
-        const uint32_t digits = pass == 2 ? 1023u : 2047u;
+    auto find_digit = [&](auto pass_tag) {
+        constexpr int pass = decltype(pass_tag)::value, shift = pass == 0 ? 21 : pass == 1 ? 10 : 0;
+        constexpr uint32_t digits = pass == 2 ? 1023u : 2047u;
         for (int r = 0; r < rounds; ++r) {
             if (rounds > 1) load(r);
 #pragma unroll
             for (int e = 0; e < kTopPerThread; ++e)
-                if (live(r, e) && (key[e] & mask) == T) atomicAdd(&hist[pass][(key[e] >> shift) & digits], 1u);
+                if (live(r, e) && (key[e] & mask) == T) {
+                    const uint32_t bin = (key[e] >> shift) & digits;
+                    atomicAdd(pass == 0 ? &hist0[bin * 4 + (lane & 3)] : pass == 1 ? &hist1[bin] : &hist2[bin], 1u);
+                }
+        }
+        if (pass == 0) {
+            __syncthreads();
+            const uint4 v0 = reinterpret_cast<const uint4 *>(copies)[2 * tid], v1 = reinterpret_cast<const uint4 *>(copies)[2 * tid + 1];
+            __syncthreads();                      // folded in place
+            hist0[2 * tid] = (v0.x + v0.y) + (v0.z + v0.w);
+            hist0[2 * tid + 1] = (v1.x + v1.y) + (v1.z + v1.w);
         }
         if (cluster > 1) cluster_sync_all(); else __syncthreads();
         // counts over the cluster and their sums from the top: thread t owns the bins 2 t, 2 t + 1 counted from the top
-        uint32_t c[2];
+        constexpr int kBins = pass == 2 ? kTopBins / 2 : kTopBins;
+        uint32_t c[2], w[2][7];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int bin = kTopBins - 1 - (2 * tid + h);
-            c[h] = hist[pass][bin];
-            for (int q = 1; q < cluster; ++q)
-                c[h] += ld_cluster_u32(cluster_map(smem_u32(&hist[pass][bin]), (uint32_t)((rank + q) % cluster)));
+        for (int h = 0; h < 2; ++h) {             // every remote load is in flight before the first is used
+            const int bin = kBins - 1 - (2 * tid + h);
+            c[h] = bin < 0 ? 0u : pass == 0 ? hist0[bin] : pass == 1 ? hist1[bin] : hist2[bin];
+#pragma unroll
+            for (int q = 1; q < 8; ++q) {
+                w[h][q - 1] = 0;
+                if (bin >= 0 && q < cluster)
+                    w[h][q - 1] = ld_cluster_u32(cluster_map(smem_u32(pass == 0 ? &hist0[bin] : pass == 1 ? &hist1[bin] : &hist2[bin]), (uint32_t)(rank ^ q)));
+            }
         }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int q = 0; q < 7; ++q) c[h] += w[h][q];
         uint32_t inc = c[0] + c[1];
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) { const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += v; }
@@ -494,14 +493,17 @@ __global__ void __launch_bounds__(kTopThreads, 1) select_topk_kernel(const Selec
         uint32_t before = (warp ? wsum[warp - 1] : 0u) + inc - c[0] - c[1];      // keys in higher bins
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            if (before < (uint32_t)need && (uint32_t)need <= before + c[h]) { s_digit = (uint32_t)(kTopBins - 1 - (2 * tid + h)); s_above = before; }
+            if (before < (uint32_t)need && (uint32_t)need <= before + c[h]) { s_digit = (uint32_t)(kBins - 1 - (2 * tid + h)); s_above = before; }
             before += c[h];
         }
         __syncthreads();
         T |= s_digit << shift;
         mask |= digits << shift;
         need -= (int)s_above;                     // after the last pass: elements equal to T to keep
-    }
+    };
+    find_digit(std::integral_constant<int, 0>{});
+    find_digit(std::integral_constant<int, 1>{});
+    find_digit(std::integral_constant<int, 2>{});
     unsigned long long base = 0;                  // (larger, equal) in front of this CTA's share
     for (int ph = cluster > 1 ? 0 : 1; ph < 2; ++ph) {
         // first the share's totals (only where there are other shares), then the output
@@ -518,13 +520,12 @@ __global__ void __launch_bounds__(kTopThreads, 1) select_topk_kernel(const Selec
             __syncthreads();                      // w64 of the round before has been read
             if (lane == 31) w64[warp] = inc;
             __syncthreads();
-            unsigned long long at = run + inc - mine, all = 0;
-            for (int w = 0; w < kTopThreads / 32; ++w) {
-                const unsigned long long v = w64[w];
-                at += w < warp ? v : 0ull;
-                all += v;
-            }
-            run += all;
+            unsigned long long sums = w64[lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { const unsigned long long v = __shfl_up_sync(0xffffffffu, sums, o); if (lane >= o) sums += v; }
+            const unsigned long long in_front = __shfl_sync(0xffffffffu, sums, warp ? warp - 1 : 0);
+            const unsigned long long at = run + (warp ? in_front : 0ull) + inc - mine;
+            run += __shfl_sync(0xffffffffu, sums, 31);
             if (ph) {
                 uint32_t gt = (uint32_t)(at >> 32), eq = (uint32_t)at;
 #pragma unroll
@@ -539,11 +540,14 @@ __global__ void __launch_bounds__(kTopThreads, 1) select_topk_kernel(const Selec
         if (!ph) {
             if (tid == 0) share_total = run;
             cluster_sync_all();
-            for (int q = 0; q < rank; ++q) {
-                unsigned long long v;
-                asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(cluster_map(smem_u32(&share_total), (uint32_t)q)) : "memory");
-                base += v;
+            unsigned long long v[7];
+#pragma unroll
+            for (int q = 0; q < 7; ++q) {
+                v[q] = 0;
+                if (q < rank) asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v[q]) : "r"(cluster_map(smem_u32(&share_total), (uint32_t)q)) : "memory");
             }
+#pragma unroll
+            for (int q = 0; q < 7; ++q) base += v[q];
         }
     }
     if (cluster > 1) cluster_sync_all();          // nobody leaves while its shared memory may be read
@@ -746,14 +750,21 @@ int32_t hippo_select_tokens_policy(int32_t batch, const int32_t *n_visual, int32
         count_launches(1);
     }
     const bool need_emb = scored && (score_mask & (HIPPO_SCORE_TEMP | HIPPO_SCORE_SPA)) != 0;
-    if (need_emb) {
+    // bf16: the integer tensor path, except where its fixed cost (set-up, merge and scores of a tile, about 17 us) outweighs the
+    // shorter loop.  Whole selection, integer path against fp64 kernels: 2,000 tokens of 2,048 44.9 / 37.6 us, 1,000 of 3,584
+    // 45.9 / 45.4, 512 of 8,192 56 / 70, 3,000 of 4,096 59 / 68, 32,768 of 4,096 201 / 289, 65,536 of 8,192 544 / 917.
+    const bool gram = dtype == HIPPO_DTYPE_BF16 && embed_dim <= kGramMaxDim && (embed_dim >= 4096 || tok * embed_dim >= 5000000);
+    if (need_emb && gram) {
+        const int32_t rc = launch_select_gram(p, (WsHeader *)workspace, s);
+        if (rc != HIPPO_OK) return rc;
+    } else if (need_emb) {
         const int warps = 8;
         dim3 g1((unsigned)((tok + warps - 1) / warps));
         if (dtype == HIPPO_DTYPE_FP32) select_dots_kernel<float><<<g1, warps * 32, 0, s>>>(p);
         else select_dots_kernel<__nv_bfloat16><<<g1, warps * 32, 0, s>>>(p);
         count_launches(1);
     }
-    if (scored && (score_mask & HIPPO_SCORE_SPA)) {
+    if (scored && (score_mask & HIPPO_SCORE_SPA) && !gram) {
         dim3 g2((unsigned)(frames * p.crops_y * p.crops_x));
         static PerDeviceOnce spa_attr;
         int dev;

@@ -114,6 +114,51 @@ def test_c4_select_whole_sequence(hb):
         check_kept(host(kept), host(fused), ref_idx, ref_fused, kth, "c4 keep %d%%" % pct)
 
 
+# (tokens, dim, grid, crop, values): one and several frames, partial frames, clipped crops, tiles that share a frame, dims that
+# are not a multiple of a step, few and many parts of a tile, two launches (more tiles than SMs), and values that the integer
+# digits cannot hold: outlier dimensions, heavy tails (more large elements than are noted singly), zeros, equal frames
+GRAM_CASES = [([64], 4096, (8, 8), (5, 5), "normal"), ([1], 4096, (14, 14), (5, 5), "normal"), ([700, 65, 3], 4104, (8, 8), (5, 5), "normal"),
+              ([1000], 5000, (14, 14), (5, 5), "outlier"), ([600], 4160, (12, 20), (5, 5), "lognormal"), ([512], 4096, (8, 8), (2, 3), "sparse"),
+              ([784], 8192, (14, 14), (5, 5), "static"), ([900], 4096, (16, 16), (4, 8), "nearly static"), ([9000], 1032, (14, 14), (5, 5), "normal"),
+              ([30000], 256, (16, 16), (5, 5), "normal"), ([400], 4096, (3, 5), (5, 5), "tiny")]
+
+
+@pytest.mark.parametrize("lens,dim,grid,crop,values", GRAM_CASES)
+def test_scores_on_the_integer_path(hb, lens, dim, grid, crop, values):
+    """Fused scores against the fp64 oracle.  An fp32 result is within half a unit of the exact score (6e-8 relative) plus the
+    error of the fp64 sums: a cosine is good to d * 2^-53 and the standardisation divides by the smallest sigma that these inputs
+    have, 1e-5, so 1e-6 * (1 + |score|) holds with a factor of ten to spare; equal frames give a temporal score of exactly 0."""
+    rng = np.random.default_rng(sum(lens) + dim)
+    E, n = [], sum(lens)
+    for m in lens:
+        x = rng.standard_normal((m, dim))
+        tpf = grid[0] * grid[1]
+        if values == "outlier":
+            x[:, 7] *= 500; x[:, dim // 2 + 3] *= 80
+        elif values == "lognormal":
+            x = np.sign(x) * np.exp(4 * x)
+        elif values == "sparse":
+            x *= rng.random((m, dim)) < 0.02
+            x[5] = 0
+        elif values in ("static", "nearly static"):
+            x = np.tile(rng.standard_normal((tpf, dim)), (-(-m // tpf), 1))[:m] + (0.05 * x if values != "static" else 0)
+        elif values == "tiny":
+            x *= 1e-30
+        E.append(W.round_to_storage(x.astype(np.float32), "bf16"))
+    mass = [rng.random(m).astype(np.float32) for m in lens]
+    ks = [W.keep_count(m, 25) for m in lens]
+    kept, fused = hb.hippo_select_tokens(dev(np.concatenate(E), "bf16"), dev(np.concatenate(mass)), lens, ks, grid[0], grid[1], crop[0], crop[1])
+    kept, fused = host(kept), host(fused)
+    at = out = 0
+    for e, w, m, k in zip(E, mass, lens, ks):
+        ref_fused, _, _ = oracle.select_scores(e, w, grid[0], grid[1], crop[0], crop[1])
+        got = fused[at:at + m].astype(np.float64)
+        assert np.all(np.abs(got - ref_fused) <= 1e-6 * (1 + np.abs(ref_fused))), (values, np.abs(got - ref_fused).max())
+        want = np.sort(np.argsort(-fused[at:at + m], kind="stable")[:k])        # the kept set is that of the scores returned
+        np.testing.assert_array_equal(kept[out:out + k], want)
+        at += m; out += k
+
+
 # ---- the other selection rules ------------------------------------------------------------------------------------
 
 def check_kept_per_frame(got_idx, ref_fused, k, tpf, what):
