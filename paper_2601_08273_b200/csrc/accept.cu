@@ -11,7 +11,7 @@
 //   stats   per (sequence, logit row, 4096-token chunk): max and sum of exponentials
 //   weigh   per (sequence, chunk): every CTA merges the chunk stats of its sequence and runs the accept tests
 //           itself (a few hundred values; cheaper than a launch of its own), then scans the residual (or bonus)
-//           weights of its chunk in token order and stores the running sum after each thread's 16 tokens
+//           weights of its chunk in token order and stores the running sum after every 16 tokens
 //   pick    per sequence: locate the chunk, then the 16-token group, then the token where the CDF crosses
 //           u * total; only that one group's weights are evaluated again
 #include <math.h>
@@ -23,9 +23,14 @@
 
 namespace hippo {
 
-constexpr int kAccThreads = 256;
-constexpr int kAccPerThread = 16;
+// The steps are bound by the latency of fp64 exponentials, so a chunk goes to many threads with few tokens each (and a short
+// code path: the unrolled exponentials are most of it).
+constexpr int kAccThreads = 1024;
+constexpr int kAccWarps = kAccThreads / 32;
+constexpr int kAccPerThread = 4;
 constexpr int kAccChunk = kAccThreads * kAccPerThread;  // 4096 vocabulary entries per chunk
+constexpr int kAccGroup = 16;                           // tokens per stored running sum
+constexpr int kAccGroups = kAccChunk / kAccGroup;
 constexpr int kAccMaxRows = 2 * 64 + 1;
 constexpr bool kAcceptFusedByDefault = false;
 
@@ -42,7 +47,7 @@ struct AcceptParams {
     int32_t *n_acc, *out;
     double2 *stats;  // [B][2*gamma+1][n_chunks]: (max, sum exp)
     double *wsum;    // [B][n_chunks]
-    double *tscan;   // [B][n_chunks][kAccThreads]: in-chunk running sum after each thread's tokens
+    double *tscan;   // [B][n_chunks][kAccGroups]: in-chunk running sum after each group of 16 tokens
     RowInfo *info;   // [B]
     int B, gamma, V, n_chunks;
 };
@@ -55,41 +60,41 @@ __device__ __forceinline__ const float *logit_row(const AcceptParams &p, int b, 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// In-order inclusive scan over the block's threads (thread i holds element i).  Deterministic.
-__device__ double block_scan_inclusive(double v, double *warp_tot /* [8] shared */, double *total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// In-order inclusive scan over the warp's lanes.
+__device__ __forceinline__ double warp_scan_inclusive(double v) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        double t = __shfl_up_sync(0xffffffffu, v, o);
+        const double t = __shfl_up_sync(0xffffffffu, v, o);
         if (lane >= o) v += t;
     }
+    return v;
+}
+
+// In-order inclusive scan over the block's threads (thread i holds element i).  Deterministic; *total is the last thread's sum.
+__device__ __forceinline__ double block_scan_inclusive(double v, double *warp_tot /* [32] shared */, double *total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    v = warp_scan_inclusive(v);
     __syncthreads();  // protect warp_tot from a previous use
     if (lane == 31) warp_tot[warp] = v;
     __syncthreads();
-    double pre = 0.0, tot = 0.0;
-    for (int w = 0; w < kAccThreads / 32; ++w) {
-        if (w < warp) pre += warp_tot[w];
-        tot += warp_tot[w];
-    }
-    *total = tot;
-    return v + pre;
+    const double t = warp_scan_inclusive(warp_tot[lane]);
+    const double pre = __shfl_sync(0xffffffffu, t, warp ? warp - 1 : 0);
+    *total = __shfl_sync(0xffffffffu, t, kAccWarps - 1);
+    return warp ? v + pre : v;
 }
 
 // Max and sum of exponentials of one 4096-token chunk of one logit row.
-__device__ void stats_item(const AcceptParams &p, int b, int r, int c) {
-    __shared__ float smax[kAccThreads / 32];
-    __shared__ double ssum[kAccThreads / 32];
+__device__ __forceinline__ void stats_item(const AcceptParams &p, int b, int r, int c) {
+    __shared__ float smax[kAccWarps];
+    __shared__ double ssum[kAccWarps];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     __syncthreads();   // the shared arrays may still be read by the previous item
     const float *row = logit_row(p, b, r);
     float v[kAccPerThread];
-    float m = -INFINITY;
-    if ((c + 1) * kAccChunk <= p.V && (((uintptr_t)row) & 15) == 0 && (p.V & 3) == 0) {
-        // full chunk, 16-byte aligned: four float4 loads per thread
-#pragma unroll
-        for (int e4 = 0; e4 < kAccPerThread / 4; ++e4) {
-            const float4 t = __ldg(reinterpret_cast<const float4 *>(row + c * kAccChunk) + e4 * kAccThreads + tid);
-            v[4 * e4] = t.x; v[4 * e4 + 1] = t.y; v[4 * e4 + 2] = t.z; v[4 * e4 + 3] = t.w;
-        }
+    if ((c + 1) * kAccChunk <= p.V && (((uintptr_t)row) & 15) == 0 && (p.V & 3) == 0) {      // full chunk, 16-byte aligned
+        const float4 t = __ldg(reinterpret_cast<const float4 *>(row + c * kAccChunk) + tid);
+        v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
     } else {
 #pragma unroll
         for (int e = 0; e < kAccPerThread; ++e) {
@@ -97,24 +102,27 @@ __device__ void stats_item(const AcceptParams &p, int b, int r, int c) {
             v[e] = t < p.V ? row[t] : -INFINITY;
         }
     }
+    float m = fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3]));
 #pragma unroll
-    for (int e = 0; e < kAccPerThread; ++e) m = fmaxf(m, v[e]);
     for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (lane == 0) smax[warp] = m;
     __syncthreads();
-    m = smax[0];
-    for (int w = 1; w < kAccThreads / 32; ++w) m = fmaxf(m, smax[w]);
+    m = smax[lane];
+#pragma unroll
+    for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     double s = 0.0;
 #pragma unroll
     for (int e = 0; e < kAccPerThread; ++e)
         if (v[e] != -INFINITY) s += exp((double)v[e] - (double)m);
+#pragma unroll
     for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) ssum[warp] = s;
     __syncthreads();
-    if (tid == 0) {
-        double tot = 0.0;
-        for (int w = 0; w < kAccThreads / 32; ++w) tot += ssum[w];
-        p.stats[((size_t)b * (2 * p.gamma + 1) + r) * p.n_chunks + c] = make_double2((double)m, tot);
+    if (warp == 0) {
+        s = ssum[lane];
+#pragma unroll
+        for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) p.stats[((size_t)b * (2 * p.gamma + 1) + r) * p.n_chunks + c] = make_double2((double)m, s);
     }
 }
 
@@ -137,7 +145,7 @@ __device__ __forceinline__ double draw_weight(const float *trow, const float *dr
     return weight_of(trow[t], use_target_only ? 0.f : drow[t], ri, use_target_only);
 }
 
-// Thread-local weights of one chunk (16 consecutive tokens per thread) and their in-order sum.
+// Thread-local weights of one chunk (four consecutive tokens per thread) and their in-order sum.
 __device__ __forceinline__ double chunk_local(const float *trow, const float *drow, int c, int V, const RowInfo &ri,
                                               bool target_only, double *w) {
     double s = 0.0;
@@ -145,14 +153,11 @@ __device__ __forceinline__ double chunk_local(const float *trow, const float *dr
     float tv[kAccPerThread], dv[kAccPerThread];
     const bool vec = t0 + kAccPerThread <= V && (((uintptr_t)(trow + t0) | (target_only ? 0 : (uintptr_t)(drow + t0))) & 15) == 0;
     if (vec) {
-#pragma unroll
-        for (int e4 = 0; e4 < kAccPerThread / 4; ++e4) {
-            const float4 a = __ldg(reinterpret_cast<const float4 *>(trow + t0) + e4);
-            tv[4 * e4] = a.x; tv[4 * e4 + 1] = a.y; tv[4 * e4 + 2] = a.z; tv[4 * e4 + 3] = a.w;
-            float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (!target_only) d = __ldg(reinterpret_cast<const float4 *>(drow + t0) + e4);
-            dv[4 * e4] = d.x; dv[4 * e4 + 1] = d.y; dv[4 * e4 + 2] = d.z; dv[4 * e4 + 3] = d.w;
-        }
+        const float4 a = __ldg(reinterpret_cast<const float4 *>(trow + t0));
+        float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (!target_only) d = __ldg(reinterpret_cast<const float4 *>(drow + t0));
+        tv[0] = a.x; tv[1] = a.y; tv[2] = a.z; tv[3] = a.w;
+        dv[0] = d.x; dv[1] = d.y; dv[2] = d.z; dv[3] = d.w;
     } else {
 #pragma unroll
         for (int e = 0; e < kAccPerThread; ++e) {
@@ -171,10 +176,19 @@ __device__ __forceinline__ double chunk_local(const float *trow, const float *dr
 
 // Merge of the chunk statistics of every logit row of sequence b and the sequential accept tests.  Run by all
 // threads of a block; the result is identical in every block of the sequence (same data, same order).
-__device__ RowInfo decide_rows(const AcceptParams &p, int b, double *rowstat /* shared [2*gamma+1][2] */, int *s_n) {
+__device__ __forceinline__ RowInfo decide_rows(const AcceptParams &p, int b, double *rowstat /* shared [2*gamma+1][3] */, int *s_n) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n_rows = 2 * p.gamma + 1;
-    for (int r = warp; r < n_rows; r += kAccThreads / 32) {
+    // the first 32 draft tokens' logits are on their way while the statistics are merged
+    const int32_t *x = p.x + (size_t)b * p.gamma;
+    int tok0 = -1;
+    float tl0 = 0.f, dl0 = 0.f, u0 = 0.f;
+    if (warp == 0 && lane < p.gamma) {
+        tok0 = x[lane];
+        u0 = p.ua[(size_t)b * p.gamma + lane];
+        if ((unsigned)tok0 < (unsigned)p.V) { tl0 = logit_row(p, b, lane)[tok0]; dl0 = logit_row(p, b, p.gamma + 1 + lane)[tok0]; }
+    }
+    for (int r = warp; r < n_rows; r += kAccWarps) {
         const double2 *st = p.stats + ((size_t)b * n_rows + r) * p.n_chunks;
         double M = -INFINITY;
         for (int c = lane; c < p.n_chunks; c += 32) M = fmax(M, st[c].x);
@@ -183,24 +197,24 @@ __device__ RowInfo decide_rows(const AcceptParams &p, int b, double *rowstat /* 
         for (int c = lane; c < p.n_chunks; c += 32)
             if (st[c].x != -INFINITY) Z += st[c].y * exp(st[c].x - M);
         for (int o = 16; o; o >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, o);
-        if (lane == 0) { rowstat[2 * r] = M; rowstat[2 * r + 1] = Z; }
+        if (lane == 0) { rowstat[3 * r] = M; rowstat[3 * r + 1] = Z; rowstat[3 * r + 2] = 1.0 / Z; }
     }
     __syncthreads();
     if (warp == 0) {
         // lane j tests draft token j (all loads independent), then the first failing lane is n
-        const int32_t *x = p.x + (size_t)b * p.gamma;
         int n = p.gamma;
         for (int j0 = 0; j0 < p.gamma; j0 += 32) {
             const int j = j0 + lane;
             bool accept = true;
             if (j < p.gamma) {
-                const int rq = p.gamma + 1 + j, tok = x[j];
+                const int rq = p.gamma + 1 + j, tok = j0 ? x[j] : tok0;
                 // a token id outside the vocabulary (a fault upstream) is never looked up: it counts as rejected
                 accept = false;
                 if ((unsigned)tok < (unsigned)p.V) {
-                    const double P = exp((double)logit_row(p, b, j)[tok] - rowstat[2 * j]) / rowstat[2 * j + 1];
-                    const double Q = exp((double)logit_row(p, b, rq)[tok] - rowstat[2 * rq]) / rowstat[2 * rq + 1];
-                    const double u = (double)p.ua[(size_t)b * p.gamma + j];
+                    const float tl = j0 ? logit_row(p, b, j)[tok] : tl0, dl = j0 ? logit_row(p, b, rq)[tok] : dl0;
+                    const double P = exp((double)tl - rowstat[3 * j]) / rowstat[3 * j + 1];
+                    const double Q = exp((double)dl - rowstat[3 * rq]) / rowstat[3 * rq + 1];
+                    const double u = (double)(j0 ? p.ua[(size_t)b * p.gamma + j] : u0);
                     accept = u * Q < P;
                 }
             }
@@ -213,8 +227,8 @@ __device__ RowInfo decide_rows(const AcceptParams &p, int b, double *rowstat /* 
     RowInfo ri;
     ri.n = *s_n;
     ri.bonus = (ri.n == p.gamma);
-    ri.Mp = rowstat[2 * ri.n]; ri.Zp = 1.0 / rowstat[2 * ri.n + 1];
-    if (ri.n < p.gamma) { ri.Mq = rowstat[2 * (p.gamma + 1 + ri.n)]; ri.Zq = 1.0 / rowstat[2 * (p.gamma + 1 + ri.n) + 1]; }
+    ri.Mp = rowstat[3 * ri.n]; ri.Zp = rowstat[3 * ri.n + 2];
+    if (ri.n < p.gamma) { ri.Mq = rowstat[3 * (p.gamma + 1 + ri.n)]; ri.Zq = rowstat[3 * (p.gamma + 1 + ri.n) + 2]; }
     else { ri.Mq = 0.0; ri.Zq = 1.0; }
     ri.pad[0] = ri.pad[1] = 0;
     return ri;
@@ -222,9 +236,9 @@ __device__ RowInfo decide_rows(const AcceptParams &p, int b, double *rowstat /* 
 
 // Residual (or bonus) weights of one chunk of sequence b, scanned in token order.  Every caller re-derives the row
 // normalisers and the accept decisions of the sequence (same data, same order: identical everywhere).
-__device__ void weigh_item(const AcceptParams &p, int b, int c) {
-    __shared__ double rowstat[2 * kAccMaxRows];
-    __shared__ double warp_tot[kAccThreads / 32];
+__device__ __forceinline__ void weigh_item(const AcceptParams &p, int b, int c) {
+    __shared__ double rowstat[3 * kAccMaxRows];
+    __shared__ double warp_tot[kAccWarps];
     __shared__ int s_n;
     const int tid = threadIdx.x;
     __syncthreads();   // the shared arrays may still be read by the previous item
@@ -242,8 +256,10 @@ __device__ void weigh_item(const AcceptParams &p, int b, int c) {
     double w[kAccPerThread], total;
     double s = chunk_local(trow, drow, c, p.V, ri, ri.bonus != 0, w);
     const double incl = block_scan_inclusive(s, warp_tot, &total);
-    p.tscan[((size_t)b * p.n_chunks + c) * kAccThreads + tid] = incl;
-    if (tid == 0) p.wsum[(size_t)b * p.n_chunks + c] = total;
+    constexpr int kPerGroup = kAccGroup / kAccPerThread;     // threads that share a group
+    if (tid % kPerGroup == kPerGroup - 1) p.tscan[((size_t)b * p.n_chunks + c) * kAccGroups + tid / kPerGroup] = incl;
+    if (tid == kAccThreads - 1) total = incl;                // the chunk's sum and the last group's are the same number
+    if (tid == kAccThreads - 1) p.wsum[(size_t)b * p.n_chunks + c] = total;
 }
 
 __global__ void __launch_bounds__(kAccThreads) accept_weigh_kernel(const AcceptParams p) {
@@ -253,91 +269,82 @@ __global__ void __launch_bounds__(kAccThreads) accept_weigh_kernel(const AcceptP
 }
 
 // The emitted token of sequence b: chunk, 16-token group and token where the CDF crosses u * total.  ws: n_chunks doubles of
-// shared memory.
-__device__ void pick_item(const AcceptParams &p, int b, double *ws) {
-    __shared__ double warp_tot[kAccThreads / 32];
+// shared memory.  The chunks and the group's tokens are looked at by the lanes of one warp.
+__device__ __forceinline__ void pick_item(const AcceptParams &p, int b, double *ws) {
+    __shared__ double warp_tot[kAccWarps];
     __shared__ double s_prefix, s_target;
-    __shared__ int s_chunk, s_tok, s_target_only;
-    const int tid = threadIdx.x;
+    __shared__ int s_chunk, s_tok, s_first;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     __syncthreads();   // the shared arrays may still be read by the previous item
     const RowInfo ri = p.info[b];
     const float *trow = logit_row(p, b, ri.n);
     const float *drow = ri.bonus ? nullptr : logit_row(p, b, p.gamma + 1 + ri.n);
-    double *wsum = p.wsum + (size_t)b * p.n_chunks;
-    double w[kAccPerThread], total;
+    const double *wsum = p.wsum + (size_t)b * p.n_chunks;
+    const double u = (double)p.ur[b];
     for (int c = tid; c < p.n_chunks; c += kAccThreads) ws[c] = wsum[c];
+    if (tid == 0) { s_chunk = -1; s_tok = 0x7fffffff; s_first = 0x7fffffff; }
     __syncthreads();
-    if (tid == 0) {
+    // chunk whose running sum first exceeds u * total, by every warp for itself up to the sum, then by the first
+    auto total_weight = [&]() {
         double Z = 0.0;
-        for (int c = 0; c < p.n_chunks; ++c) Z += ws[c];
-        s_target_only = ri.bonus || !(Z > 0.0);
-    }
-    __syncthreads();
-    const bool target_only = s_target_only != 0;
+        for (int c0 = 0; c0 < p.n_chunks; c0 += 32) Z += __shfl_sync(0xffffffffu, warp_scan_inclusive(c0 + lane < p.n_chunks ? ws[c0 + lane] : 0.0), 31);
+        return Z;
+    };
+    double Z = total_weight(), w[kAccPerThread], total;
+    const bool target_only = ri.bonus || !(Z > 0.0);
     if (target_only && !ri.bonus) {
         // residual is identically zero (P_n == Q_n): fall back to P_n; recompute the chunk totals
+        __syncthreads();
         for (int c = 0; c < p.n_chunks; ++c) {
-            double s = chunk_local(trow, drow, c, p.V, ri, true, w);
-            block_scan_inclusive(s, warp_tot, &total);
-            if (tid == 0) ws[c] = total;
+            const double s = chunk_local(trow, drow, c, p.V, ri, true, w);
+            const double incl = block_scan_inclusive(s, warp_tot, &total);
+            if (tid == kAccThreads - 1) ws[c] = incl;
         }
         __syncthreads();
+        Z = total_weight();
     }
-    if (tid == 0) {
-        double Z = 0.0;
-        for (int c = 0; c < p.n_chunks; ++c) Z += ws[c];
-        const double target = (double)p.ur[b] * Z;
+    if (warp == 0) {
+        const double target = u * Z;
         double cum = 0.0;
-        int chunk = -1;
-        for (int c = 0; c < p.n_chunks; ++c) {
-            if (cum + ws[c] > target) { chunk = c; break; }
-            cum += ws[c];
+        for (int c0 = 0; c0 < p.n_chunks; c0 += 32) {
+            const double v = c0 + lane < p.n_chunks ? ws[c0 + lane] : 0.0, incl = warp_scan_inclusive(v);
+            double before = __shfl_up_sync(0xffffffffu, incl, 1);
+            before = cum + (lane ? before : 0.0);
+            const unsigned over = __ballot_sync(0xffffffffu, c0 + lane < p.n_chunks && before + v > target);
+            if (over) {
+                if (lane == __ffs(over) - 1) { s_chunk = c0 + lane; s_prefix = before; }
+                break;
+            }
+            cum += __shfl_sync(0xffffffffu, incl, 31);
         }
-        s_chunk = chunk; s_prefix = cum; s_target = target; s_tok = 0x7fffffff;
+        if (lane == 0) s_target = target;
     }
     __syncthreads();
     int tok = -1;
-    if (s_chunk >= 0 && !(target_only && !ri.bonus)) {
-        // the 16-token group: first thread of the chunk whose stored running sum exceeds the target
-        const int c = s_chunk;
-        const double incl = p.tscan[((size_t)b * p.n_chunks + c) * kAccThreads + tid];
-        const bool over = s_prefix + incl > s_target;
-        const unsigned bal = __ballot_sync(0xffffffffu, over);
-        __shared__ int s_first[kAccThreads / 32];
-        if ((tid & 31) == 0) s_first[tid >> 5] = bal ? (tid & ~31) + __ffs(bal) - 1 : 0x7fffffff;
-        __syncthreads();
-        int first = 0x7fffffff;
-        for (int w8 = 0; w8 < kAccThreads / 32; ++w8) first = min(first, s_first[w8]);
-        if (first != 0x7fffffff && tid == first) {
-            // this thread's tokens alone, in order, from the running sum before them
-            const int t0 = c * kAccChunk + tid * kAccPerThread;
-            double run = s_prefix + incl, back = 0.0;
-            double wt[kAccPerThread];
-#pragma unroll
-            for (int e = 0; e < kAccPerThread; ++e) {
-                wt[e] = t0 + e < p.V ? draw_weight(trow, drow, t0 + e, ri, target_only) : 0.0;
-                back += wt[e];
-            }
-            run -= back;
-            int mine = -1;
-#pragma unroll
-            for (int e = 0; e < kAccPerThread; ++e) {
-                run += wt[e];
-                if (mine < 0 && run > s_target) mine = t0 + e;
-            }
-            // rounding may leave the crossing just past the group's end: then its last positive weight
-            if (mine < 0) {
-#pragma unroll
-                for (int e = 0; e < kAccPerThread; ++e) if (wt[e] > 0.0) mine = t0 + e;
-            }
-            s_tok = mine < 0 ? 0x7fffffff : mine;
+    const int c = s_chunk;
+    if (c >= 0 && !(target_only && !ri.bonus)) {
+        // the 16-token group: the first of the chunk whose stored running sum exceeds the target
+        const double *scan = p.tscan + ((size_t)b * p.n_chunks + c) * kAccGroups;
+        if (tid < kAccGroups) {
+            const unsigned over = __ballot_sync(0xffffffffu, s_prefix + scan[tid] > s_target);
+            if (over && lane == __ffs(over) - 1) atomicMin(&s_first, tid);
         }
         __syncthreads();
-        if (s_tok != 0x7fffffff) tok = s_tok;
-    } else if (s_chunk >= 0) {
-        const int c = s_chunk;
-        double s = chunk_local(trow, drow, c, p.V, ri, target_only, w);
-        double incl = block_scan_inclusive(s, warp_tot, &total);
+        const int first = s_first;
+        if (warp == 0 && first != 0x7fffffff) {
+            // its tokens, a lane each, in order from the running sum before them
+            const int t = c * kAccChunk + first * kAccGroup + lane;
+            const bool in = lane < kAccGroup && t < p.V;
+            const double wt = in ? draw_weight(trow, drow, t, ri, target_only) : 0.0;
+            const double run = s_prefix + (first ? scan[first - 1] : 0.0) + warp_scan_inclusive(wt);
+            const unsigned over = __ballot_sync(0xffffffffu, in && run > s_target), positive = __ballot_sync(0xffffffffu, in && wt > 0.0);
+            // rounding may leave the crossing just past the group's end: then its last positive weight
+            const int at = over ? __ffs(over) - 1 : positive ? 31 - __clz(positive) : -1;
+            if (at >= 0) tok = c * kAccChunk + first * kAccGroup + at;
+        }
+    } else if (c >= 0) {
+        const double s = chunk_local(trow, drow, c, p.V, ri, target_only, w);
+        const double incl = block_scan_inclusive(s, warp_tot, &total);
         double run = s_prefix + (incl - s);  // CDF just before this thread's first token
         int mine = 0x7fffffff;
 #pragma unroll
@@ -421,7 +428,7 @@ static AcceptWs accept_ws(int B, int gamma, int V) {
     w.wsum_off = w.stats_off + align_up((size_t)B * (2 * gamma + 1) * w.n_chunks * sizeof(double2), 256);
     w.info_off = w.wsum_off + align_up((size_t)B * w.n_chunks * sizeof(double), 256);
     w.tscan_off = w.info_off + align_up((size_t)B * sizeof(RowInfo), 256);
-    w.total = w.tscan_off + align_up((size_t)B * w.n_chunks * kAccThreads * sizeof(double), 256);
+    w.total = w.tscan_off + align_up((size_t)B * w.n_chunks * kAccGroups * sizeof(double), 256);
     return w;
 }
 
@@ -430,8 +437,8 @@ static AcceptWs accept_ws(int B, int gamma, int V) {
 //   argmax  per (sequence, target row, chunk): maximum and its first position -> stats[b][row][chunk] = (max, index)
 //   greedy  per sequence: merge the chunks of every row, compare with the draft tokens, write the outputs
 __global__ void __launch_bounds__(kAccThreads) accept_argmax_kernel(const AcceptParams p) {
-    __shared__ float smax[kAccThreads / 32];
-    __shared__ int sidx[kAccThreads / 32];
+    __shared__ float smax[kAccWarps];
+    __shared__ int sidx[kAccWarps];
     pdl_wait();
     pdl_trigger();
     const int c = blockIdx.x, r = blockIdx.y, b = blockIdx.z, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -451,10 +458,14 @@ __global__ void __launch_bounds__(kAccThreads) accept_argmax_kernel(const Accept
     }
     if (lane == 0) { smax[warp] = m; sidx[warp] = mi; }
     __syncthreads();
-    if (tid == 0) {
-        for (int w = 1; w < kAccThreads / 32; ++w)
-            if (smax[w] > m || (smax[w] == m && sidx[w] < mi)) { m = smax[w]; mi = sidx[w]; }
-        p.stats[((size_t)b * (2 * p.gamma + 1) + r) * p.n_chunks + c] = make_double2((double)m, (double)mi);
+    if (warp == 0) {
+        m = smax[lane]; mi = sidx[lane];
+        for (int o = 16; o; o >>= 1) {
+            const float om = __shfl_xor_sync(0xffffffffu, m, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, mi, o);
+            if (om > m || (om == m && oi < mi)) { m = om; mi = oi; }
+        }
+        if (lane == 0) p.stats[((size_t)b * (2 * p.gamma + 1) + r) * p.n_chunks + c] = make_double2((double)m, (double)mi);
     }
 }
 
@@ -464,7 +475,7 @@ __global__ void __launch_bounds__(kAccThreads) accept_greedy_kernel(const Accept
     pdl_trigger();
     const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n_rows = 2 * p.gamma + 1;
-    for (int r = warp; r <= p.gamma; r += kAccThreads / 32) {
+    for (int r = warp; r <= p.gamma; r += kAccWarps) {
         const double2 *st = p.stats + ((size_t)b * n_rows + r) * p.n_chunks;
         double m = -INFINITY, mi = 2147483647.0;
         for (int c = lane; c < p.n_chunks; c += 32)
