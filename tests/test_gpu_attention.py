@@ -237,6 +237,29 @@ def test_short_cache_path(hb, D, q_len, Hq, Hkv, lens):
             assert np.all(got[b] == 0) and np.all(np.isneginf(lse[b]))
 
 
+# (dtype, head size, q_len, query heads, kv heads, lengths, splits): head sizes outside the tensor-core kernels, one key, clusters of
+# 1 to 16, two tiles per CTA, more splits than a cluster (partial slots), rows that only leave room for 16-key tiles
+GENERIC = [("fp32", 32, 1, 2, 2, [1], 0), ("fp32", 96, 3, 6, 2, [33, 3, 2, 64], 0), ("fp32", 64, 5, 4, 1, [513], 0), ("fp32", 128, 2, 4, 2, [1024], 0),
+           ("fp32", 128, 2, 4, 2, [1025], 0), ("fp32", 64, 1, 2, 1, [1500], 40), ("fp32", 256, 4, 8, 2, [300], 5), ("bf16", 160, 2, 6, 3, [700, 90], 0),
+           ("fp32", 192, 14, 16, 2, [200], 0), ("bf16", 256, 3, 4, 1, [3000], 0)]
+
+
+@pytest.mark.parametrize("dtype,D,q_len,Hq,Hkv,lens,splits", GENERIC)
+def test_cuda_core_path(hb, dtype, D, q_len, Hq, Hkv, lens, splits):
+    rng = np.random.default_rng(D + q_len + sum(lens))
+    B = len(lens)
+    q = W.round_to_storage(rng.standard_normal((B, q_len, Hq, D)).astype(np.float32), dtype)
+    k = W.round_to_storage(rng.standard_normal((B, max(lens), Hkv, D)).astype(np.float32), dtype)
+    v = W.round_to_storage(rng.standard_normal((B, max(lens), Hkv, D)).astype(np.float32), dtype)
+    live = [b for b in range(B) if lens[b] >= q_len]
+    got, lse = run_case(hb, hb.hippo_verify_attention, q, k, v, lens, dtype, shuffle_seed=4, num_splits=splits, fill=np.nan)
+    ref, ref_lse = oracle.attention(q[live], k[live], v[live], [lens[b] for b in live])
+    assert_close(got[live], ref, TOL[dtype], "CUDA-core path")
+    assert_close(lse[live], ref_lse, TOL[dtype] if dtype == "fp32" else 2e-3, "CUDA-core path lse")
+    for b in set(range(B)) - set(live):
+        assert np.all(got[b] == 0) and np.all(np.isneginf(lse[b]))
+
+
 @pytest.mark.parametrize("dtype,q_len,kvl", [("bf16", 6, 700), ("bf16", 1, 500), ("fp32", 3, 200)])
 def test_lengths_known_on_the_host(hb, dtype, q_len, kvl):
     """kv_len = NULL: every sequence has max_kv_len keys; same result as with the length array."""
