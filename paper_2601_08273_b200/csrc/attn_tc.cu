@@ -1462,16 +1462,20 @@ static int32_t launch_tc_layers(AttnParams p, int n_layers, const void *const *q
     if (max_ctas > 0 && sms > max_ctas) sms = max_ctas;    // the caller leaves the other SMs to concurrent kernels
     if (sms < 1) sms = 1;
     p.num_splits = 0;
-    // Short caches: with fewer than about seven pages per CTA and layer a CTA spends longer merging (every output row
-    // gathers one partial per contributing CTA) than streaming, so the grid shrinks with the work, to a whole number of
-    // CTAs per unit where it can.  Measured at 6,400 keys, 4 kv heads, 42 packed rows, per layer: 19.1 us on 148 CTAs,
-    // 17.3 on 72, 15.0 on 64, 14.6 on 56, 17.1 on 48.
+    // Short caches: a CTA that gathers many partials per row spends longer merging than streaming, one with many pages
+    // streams longer than the fixed part of a layer takes.  About fifteen CTAs per unit with two to seven pages each, a whole
+    // number per unit where that works.  Measured per layer at 42 packed rows, 4 kv heads, pages per CTA 2 / 3 / 5 / 7: 1,700
+    // keys 11.0 / 12.6 / 17.1 / 24.2 us, 3,000 keys 8.7 / 10.3 / 12.7 / 15.4, 5,000 keys 10.7 / 10.6 / 10.4 / 12.2, 8,000 keys
+    // 10.9 / 10.9 / 10.7 / 10.9; at 6,400 keys 148 CTAs (2.7 pages, 37 partials per row) took 19.1 us before the merge warp
+    // had all its loads in flight.
     {
         int longest;
         long long total_pages;
         plan_pages(p, longest, total_pages);
-        long long by_work = total_pages / 7;
         const int units_all = p.batch * p.n_kv_heads;
+        long long pages_per_cta = total_pages / units_all / 15;
+        pages_per_cta = pages_per_cta < 2 ? 2 : pages_per_cta > 7 ? 7 : pages_per_cta;
+        long long by_work = total_pages / pages_per_cta;
         if (by_work > units_all) by_work -= by_work % units_all;
         if (by_work < sms) sms = (int)(by_work < 1 ? 1 : by_work);
     }

@@ -244,3 +244,13 @@ def test_host_lengths_only_plan_the_launch(hb):
         out = hb.hippo_verify_attention(qd, kv, kvl, max(lens), kv_len_host=hl)
         torch.cuda.synchronize()
         assert_close(host(out), ref, TOL["bf16"], "host lengths %s" % (hl is not None))
+
+
+@pytest.mark.parametrize("kv", [130, 961, 1921, 2881])
+def test_short_caches_spread_over_many_ctas(hb, kv):
+    """Two and three pages per CTA, at and just past the lengths where the number of CTAs per unit changes."""
+    rng = np.random.default_rng(kv)
+    lens = [kv, max(kv - 70, 6)]
+    q, k, v = layer_inputs(rng, 3, 2, 6, 14, 2, 128, lens, "bf16")
+    check_layers(hb, q, k, v, lens, "bf16", fill=np.nan)
+    check_layers(hb, q, k, v, lens, "bf16", host_lens=True)
