@@ -750,9 +750,9 @@ int32_t hippo_select_tokens_policy(int32_t batch, const int32_t *n_visual, int32
         count_launches(1);
     }
     const bool need_emb = scored && (score_mask & (HIPPO_SCORE_TEMP | HIPPO_SCORE_SPA)) != 0;
-    // bf16: the integer tensor path, except where its fixed cost (set-up, merge and scores of a tile, about 17 us) outweighs the
+    // bf16: the integer tensor path, except where its fixed cost (set-up, merge and scores of a tile, about 14 us) outweighs the
     // shorter loop.  Whole selection, integer path against fp64 kernels: 2,000 tokens of 2,048 44.9 / 37.6 us, 1,000 of 3,584
-    // 45.9 / 45.4, 512 of 8,192 56 / 70, 3,000 of 4,096 59 / 68, 32,768 of 4,096 201 / 289, 65,536 of 8,192 544 / 917.
+    // 45.9 / 45.4, 512 of 8,192 54 / 70, 3,000 of 4,096 55 / 68, 32,768 of 4,096 190 / 289, 65,536 of 8,192 521 / 917.
     const bool gram = dtype == HIPPO_DTYPE_BF16 && embed_dim <= kGramMaxDim && (embed_dim >= 4096 || tok * embed_dim >= 5000000);
     if (need_emb && gram) {
         const int32_t rc = launch_select_gram(p, (WsHeader *)workspace, s);

@@ -25,7 +25,7 @@
 // cluster split the embedding dimension and add their blocks through distributed shared memory.
 // Bound: the shared-memory and L1 data path (per step of 64 dimensions 64 KB loaded, stored and passed through L1, 72 KB read by
 // the MMAs, 1,270 clocks of the 1,700 that a step takes) beside the conversion (about 150 instructions per thread and step, 940
-// clocks with neither loads nor MMAs).  65,536 tokens of 8,192: 470 us; 890 us for the fp64 kernels.  Measured and not better: MMA
+// clocks with neither loads nor MMAs).  65,536 tokens of 8,192: 440 us; 890 us for the fp64 kernels.  Measured and not better: MMA
 // issue by one of the converting warps (+25 %), L2 prefetch ahead of the loads (+6 %), generic instead of shared stores (+10 %).
 #include <cuda_fp16.h>
 #include <math.h>
@@ -70,6 +70,8 @@ struct GramShared {
     volatile int abort;
     int n_list;
     int scale_exp[kGramRows];        // biased exponent E of the scale's upper bound 2^(E - 127); s = 2^(E - 127 - 14)
+    int token[kGramRows];            // the rows' tokens (-1: none) and first rows of their crops
+    int first[kGramRows];
     double inv_root[kGramRows];      // 1 / root of the scaled norm
     uint32_t list[kGramList];        // row << 16 | dimension
 };
@@ -281,7 +283,11 @@ __global__ void __launch_bounds__(kGramThreads, 1) select_gram_kernel(const Sele
         mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
         mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
         const int e = mx ? (int)(mx >> 7) + 3 : 127;
-        if ((tid & 3) == 0) sh->scale_exp[r] = e < 20 ? 20 : e > 250 ? 250 : e;
+        if ((tid & 3) == 0) {
+            sh->scale_exp[r] = e < 20 ? 20 : e > 250 ? 250 : e;
+            sh->token[r] = tk;
+            sh->first[r] = r / m * m;
+        }
     }
     fence_proxy_async();
     tc_fence_before();
@@ -326,7 +332,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) select_gram_kernel(const Sele
         const int s_full = p.d / kGramStep;                          // steps whose every piece exists
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-            const int r = row0 + 64 * i, tk = token(r);
+            const int r = row0 + 64 * i, tk = sh->token[r];
             // a row without a token reads the sequence's first one, scaled by 0; nobody looks at its sums
             src[i] = reinterpret_cast<const uint4 *>(E + (size_t)(tk >= 0 ? tk : p.seq_off[b]) * p.d + piece * 8) + (size_t)s0 * (kGramStep / 8);
             const uint32_t inv = tk >= 0 ? (uint32_t)(268 - sh->scale_exp[r]) << 23 : 0u;         // 2^(14 - (E - 127))
@@ -380,7 +386,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) select_gram_kernel(const Sele
         //      <x_i, x_j> / (s_i s_j) = P_ij + P_ji
         if (!sh->abort) {
             tc_fence_after();
-            const int r = (warp & 3) * 32 + lane, col0 = r / m * m;
+            const int r = (warp & 3) * 32 + lane, col0 = sh->first[r];
             const uint32_t base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
 #pragma unroll 1
             for (int h = 0; h < 2; ++h) {
@@ -393,12 +399,11 @@ __global__ void __launch_bounds__(kGramThreads, 1) select_gram_kernel(const Sele
                 for (int e = 0; e < 16; ++e) {
                     const int col = cb + e, rel = col - col0;
                     const bool in_crop = rel >= 0 && rel < m, next = col == r + m, prev = col == r - m;
-                    if (in_crop || next || prev) {
-                        const double v = fma(32768.0, int_to_double(acc[0][e]), fma(256.0, int_to_double(acc[1][e]), 0.5 * (int_to_double(acc[2][e]) + (double)acc[3][e])));
-                        if (in_crop) P[r * kGramPStride + rel] = v;
-                        if (next) t_next[r] = v;
-                        if (prev) t_prev[r] = v;
-                    }
+                    // formed for every column: a branch per column would put their chains one behind the other (3.2 us)
+                    const double v = fma(32768.0, int_to_double(acc[0][e]), fma(256.0, int_to_double(acc[1][e]), 0.5 * (int_to_double(acc[2][e]) + (double)acc[3][e])));
+                    if (in_crop) P[r * kGramPStride + rel] = v;
+                    if (next) t_next[r] = v;
+                    if (prev) t_prev[r] = v;
                 }
             }
             tc_fence_before();
@@ -416,13 +421,13 @@ __global__ void __launch_bounds__(kGramThreads, 1) select_gram_kernel(const Sele
     if (n_list > 0) {
         const int k_begin = s0 * kGramStep, k_end = min(p.d, s1 * kGramStep);
         for (int r = warp; r < kGramRows; r += kGramThreads / 32) {
-            const int ti = token(r);
+            const int ti = sh->token[r];
             if (ti < 0) continue;
-            const int fr = r / m * m;
+            const int fr = sh->first[r];
             // lanes: the row's crop, then (lanes 0, 1 of a second round) its neighbours in time
             for (int turn = 0; turn < 2; ++turn) {
                 const int rj = turn == 0 ? (lane < m ? fr + lane : -1) : (lane == 0 ? r + m : lane == 1 ? r - m : -1);
-                const int tj = rj >= 0 && rj < kGramRows ? token(rj) : -1;
+                const int tj = rj >= 0 && rj < kGramRows ? sh->token[rj] : -1;
                 if (tj < 0) continue;
                 double *dst = turn == 0 ? P + r * kGramPStride + lane : lane == 0 ? t_next + r : t_prev + r;
                 const double si = scalbn(1.0, 141 - sh->scale_exp[r]), sj = scalbn(1.0, 141 - sh->scale_exp[rj]);
@@ -470,22 +475,23 @@ __global__ void __launch_bounds__(kGramThreads, 1) select_gram_kernel(const Sele
     if (gp.part == 2 && gp.splits == 1) asm volatile("griddepcontrol.wait;" ::: "memory");
     if (!good) return;
     __syncthreads();
-    // ---- scores: norms, cosines, their variance per row
+    // ---- scores: norms, cosines, their variance per row (the shared frame's belong to the next tile)
+    const int own_rows = (own_end - f0) * m;
     if (tid < kGramRows) {
-        const int a = tid - tid / m * m;
+        const int a = tid - sh->first[tid];
         const double n2 = 2.0 * P[tid * kGramPStride + a];
         sh->inv_root[tid] = n2 == 0.0 ? 0.0 : rsqrt(n2);             // NaN stays; a cosine with a zero vector is 0
-        const int tk = token(tid), f = f0 + tid / m;
-        if (tk >= 0 && f < own_end) {
+        const int tk = sh->token[tid];
+        if (tk >= 0 && tid < own_rows) {
             const double s = scalbn(1.0, sh->scale_exp[tid] - 141);
             p.norm2[tk] = n2 * s * s;
             const int nx = tid + m;
-            if (nx < kGramRows && token(nx) >= 0) p.tdot[tk] = (t_next[tid] + t_prev[nx]) * s * scalbn(1.0, sh->scale_exp[nx] - 141);
+            if (nx < kGramRows && sh->token[nx] >= 0) p.tdot[tk] = (t_next[tid] + t_prev[nx]) * s * scalbn(1.0, sh->scale_exp[nx] - 141);
         }
     }
     __syncthreads();
     for (int i = tid; i < kGramRows * kMaxCrop; i += kGramThreads) {
-        const int r = i / kMaxCrop, cj = i % kMaxCrop, fr = r / m * m, a = r - fr;
+        const int r = i / kMaxCrop, cj = i % kMaxCrop, fr = sh->first[r], a = r - fr;
         if (cj >= m || cj <= a || fr + cj >= kGramRows) continue;
         const double cs = (P[r * kGramPStride + cj] + P[(fr + cj) * kGramPStride + a]) * (sh->inv_root[r] * sh->inv_root[fr + cj]);
         P[r * kGramPStride + cj] = cs;
@@ -493,9 +499,9 @@ __global__ void __launch_bounds__(kGramThreads, 1) select_gram_kernel(const Sele
     }
     __syncthreads();
     if (tid < 4 * kGramRows) {                                        // four threads per row
-        const int r = tid >> 2, tk = token(r), f = f0 + r / m, fr = r / m * m, a = r - fr;
+        const int r = tid >> 2, tk = sh->token[r], fr = sh->first[r], a = r - fr;
         int M = m;                                                    // a partial frame holds the first cells of a crop
-        while (M > 1 && token(fr + M - 1) < 0) --M;
+        while (M > 1 && (fr + M > kGramRows || sh->token[fr + M - 1] < 0)) --M;
         const double *row = P + r * kGramPStride;
         double mu = 0.0, var = 0.0;
         for (int j = tid & 3; j < M; j += 4) mu += j == a ? 1.0 : row[j];
@@ -508,7 +514,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) select_gram_kernel(const Sele
         }
         var += __shfl_xor_sync(0xffffffffu, var, 1);
         var += __shfl_xor_sync(0xffffffffu, var, 2);
-        if ((tid & 3) == 0 && tk >= 0 && f < own_end) p.s_spa[tk] = var / M;
+        if ((tid & 3) == 0 && tk >= 0 && r < own_rows) p.s_spa[tk] = var / M;
     }
 }
 
