@@ -1433,9 +1433,9 @@ AttnLayersWsLayout attn_layers_ws_layout(int n_layers, int batch, int q_len, int
     return L;
 }
 
-// Bounded multi-layer grids are launched as clusters of eight, up to a grid of which all clusters are sure to be resident
-// together (a GPC of 16 - 20 SMs holds two: 12 clusters need six of the eight GPCs).
-constexpr int kPackCtas = 8, kPackMaxCtas = 96;
+// Bounded multi-layer grids are launched as clusters of eight, up to a grid of which all clusters are resident together beside
+// two clusters of a draft call (fifteen fit at one CTA per SM; with 14 the draft calls ran one cluster at a time).
+constexpr int kPackCtas = 8, kPackMaxCtas = 104;
 
 template <int D>
 static int32_t launch_tc_layers(AttnParams p, int n_layers, const void *const *q, const hippo_kv_cache_t *kv, void *const *out,

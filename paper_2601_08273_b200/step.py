@@ -130,14 +130,15 @@ class HippoStep:
         self.stream_v = torch.cuda.Stream(device=self.device)
         if verify_max_ctas == 0 and multi_layer_verify:
             # Default sharing, from the two legs' sizes.  A draft call (latency-bound, about 4.5 us) finds no SM beside a
-            # verification pass on all of them, so the legs add up; on 96 SMs verification (bandwidth-bound) is 1.3 times as
-            # long and the draft calls run beside it.  Measured on B200, 32k tokens, 96 against all SMs: 7 draft tokens
-            # 1.57 ms / 2.12, 3 draft tokens (the draft leg 0.44 of the verification leg) 1.41 / 1.56; 64k tokens with 80
-            # target layers (0.24) 6.11 / 5.39.
+            # verification pass on all of them, so the legs add up; on 104 SMs verification (bandwidth-bound) is 1.25 times as
+            # long and the draft calls run beside it.  Measured on B200, 32k tokens, 96 / 104 SMs: 3 draft tokens (the draft leg
+            # 0.4 of the verification leg) 1.27 / 1.19 ms, 5 draft tokens 1.34 / 1.25, 7 draft tokens (legs of one length)
+            # 1.43 / 1.45.  All SMs against 96: 7 draft tokens 2.12 ms / 1.57, 3 draft tokens 1.56 / 1.41; 64k tokens with 80
+            # target layers (0.24) 5.39 / 6.11.
             verify_s = self.verify_kv_bytes_per_layer() * self.Lt / 5.4e12
             draft_s = g * self.Ld * 4.5e-6
             if draft_s > 0.33 * verify_s:
-                self.verify_max_ctas = 96
+                self.verify_max_ctas = 104 if draft_s < 0.9 * verify_s else 96
         if self.verify_max_ctas:
             self.draft_num_splits = 8
 
@@ -271,7 +272,7 @@ class HippoStep:
 
         The verification leg reads neither the selection nor the pruned cache.  With `verify_beside_select` it is forked
         first and runs beside select and gather too; otherwise it starts once the selection has finished (the selection's
-        fp64 kernels want every SM for themselves) and runs beside the draft calls only."""
+        kernels take every SM) and runs beside the draft calls only."""
         main = torch.cuda.current_stream(self.device)
         if self.verify_beside_select:
             self.stream_v.wait_stream(main)

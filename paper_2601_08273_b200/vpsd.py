@@ -39,7 +39,7 @@ class VpsdLoop:
         if draft_num_splits is None:
             # alone on the GPU: automatic; beside a bounded verification pass: clusters of eight while whole GPCs stay free,
             # else the kernel that takes scattered SMs
-            draft_num_splits = 0 if verify_max_ctas == 0 else 8 if verify_max_ctas <= 96 else 16
+            draft_num_splits = 0 if verify_max_ctas == 0 else 8 if verify_max_ctas <= 104 else 16
         self.st.draft_num_splits = draft_num_splits
         st, g = self.st, cfg.gamma
         self.dev = st.device
