@@ -23,8 +23,8 @@
 
 namespace hippo {
 
-// The steps are bound by the latency of fp64 exponentials, so a chunk goes to many threads with few tokens each (and a short
-// code path: the unrolled exponentials are most of it).
+// The steps are bound by the latency of fp64 exponentials until there is a wave of chunks: a chunk goes to 1,024 threads of four
+// tokens, or to fewer with more (see the launches).
 constexpr int kAccThreads = 1024;
 constexpr int kAccWarps = kAccThreads / 32;
 constexpr int kAccPerThread = 4;
@@ -72,64 +72,73 @@ __device__ __forceinline__ double warp_scan_inclusive(double v) {
 }
 
 // In-order inclusive scan over the block's threads (thread i holds element i).  Deterministic; *total is the last thread's sum.
+template <int T>
 __device__ __forceinline__ double block_scan_inclusive(double v, double *warp_tot /* [32] shared */, double *total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     v = warp_scan_inclusive(v);
     __syncthreads();  // protect warp_tot from a previous use
     if (lane == 31) warp_tot[warp] = v;
     __syncthreads();
-    const double t = warp_scan_inclusive(warp_tot[lane]);
+    const double t = warp_scan_inclusive(lane < T / 32 ? warp_tot[lane] : 0.0);
     const double pre = __shfl_sync(0xffffffffu, t, warp ? warp - 1 : 0);
-    *total = __shfl_sync(0xffffffffu, t, kAccWarps - 1);
+    *total = __shfl_sync(0xffffffffu, t, T / 32 - 1);
     return warp ? v + pre : v;
 }
 
-// Max and sum of exponentials of one 4096-token chunk of one logit row.
+// Max and sum of exponentials of one 4096-token chunk of one logit row, by T threads.
+template <int T>
 __device__ __forceinline__ void stats_item(const AcceptParams &p, int b, int r, int c) {
-    __shared__ float smax[kAccWarps];
-    __shared__ double ssum[kAccWarps];
+    constexpr int kPer = kAccChunk / T, kWarps = T / 32;
+    __shared__ float smax[kWarps];
+    __shared__ double ssum[kWarps];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     __syncthreads();   // the shared arrays may still be read by the previous item
     const float *row = logit_row(p, b, r);
-    float v[kAccPerThread];
+    float v[kPer];
     if ((c + 1) * kAccChunk <= p.V && (((uintptr_t)row) & 15) == 0 && (p.V & 3) == 0) {      // full chunk, 16-byte aligned
-        const float4 t = __ldg(reinterpret_cast<const float4 *>(row + c * kAccChunk) + tid);
-        v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+#pragma unroll
+        for (int e = 0; e < kPer; e += 4) {
+            const float4 t = __ldg(reinterpret_cast<const float4 *>(row + c * kAccChunk) + (e / 4) * T + tid);
+            v[e] = t.x; v[e + 1] = t.y; v[e + 2] = t.z; v[e + 3] = t.w;
+        }
     } else {
 #pragma unroll
-        for (int e = 0; e < kAccPerThread; ++e) {
-            const int t = c * kAccChunk + e * kAccThreads + tid;
+        for (int e = 0; e < kPer; ++e) {
+            const int t = c * kAccChunk + e * T + tid;
             v[e] = t < p.V ? row[t] : -INFINITY;
         }
     }
-    float m = fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3]));
+    float m = v[0];
+#pragma unroll
+    for (int e = 1; e < kPer; ++e) m = fmaxf(m, v[e]);
 #pragma unroll
     for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (lane == 0) smax[warp] = m;
     __syncthreads();
-    m = smax[lane];
+    m = smax[lane % kWarps];
 #pragma unroll
     for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     double s = 0.0;
 #pragma unroll
-    for (int e = 0; e < kAccPerThread; ++e)
+    for (int e = 0; e < kPer; ++e)
         if (v[e] != -INFINITY) s += exp((double)v[e] - (double)m);
 #pragma unroll
     for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) ssum[warp] = s;
     __syncthreads();
     if (warp == 0) {
-        s = ssum[lane];
+        s = lane < kWarps ? ssum[lane] : 0.0;
 #pragma unroll
         for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (lane == 0) p.stats[((size_t)b * (2 * p.gamma + 1) + r) * p.n_chunks + c] = make_double2((double)m, s);
     }
 }
 
-__global__ void __launch_bounds__(kAccThreads) accept_stats_kernel(const AcceptParams p) {
+template <int T>
+__global__ void __launch_bounds__(T) accept_stats_kernel(const AcceptParams p) {
     pdl_wait();
     pdl_trigger();
-    stats_item(p, blockIdx.z, blockIdx.y, blockIdx.x);
+    stats_item<T>(p, blockIdx.z, blockIdx.y, blockIdx.x);
 }
 
 // Weight of token t in the distribution the emitted token is drawn from.  use_target_only: bonus row, or the
@@ -145,29 +154,34 @@ __device__ __forceinline__ double draw_weight(const float *trow, const float *dr
     return weight_of(trow[t], use_target_only ? 0.f : drow[t], ri, use_target_only);
 }
 
-// Thread-local weights of one chunk (four consecutive tokens per thread) and their in-order sum.
+// Thread-local weights of one chunk (4096 / T consecutive tokens per thread) and their in-order sum.
+template <int T>
 __device__ __forceinline__ double chunk_local(const float *trow, const float *drow, int c, int V, const RowInfo &ri,
                                               bool target_only, double *w) {
+    constexpr int kPer = kAccChunk / T;
     double s = 0.0;
-    const int t0 = c * kAccChunk + threadIdx.x * kAccPerThread;
-    float tv[kAccPerThread], dv[kAccPerThread];
-    const bool vec = t0 + kAccPerThread <= V && (((uintptr_t)(trow + t0) | (target_only ? 0 : (uintptr_t)(drow + t0))) & 15) == 0;
+    const int t0 = c * kAccChunk + threadIdx.x * kPer;
+    float tv[kPer], dv[kPer];
+    const bool vec = t0 + kPer <= V && (((uintptr_t)(trow + t0) | (target_only ? 0 : (uintptr_t)(drow + t0))) & 15) == 0;
     if (vec) {
-        const float4 a = __ldg(reinterpret_cast<const float4 *>(trow + t0));
-        float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (!target_only) d = __ldg(reinterpret_cast<const float4 *>(drow + t0));
-        tv[0] = a.x; tv[1] = a.y; tv[2] = a.z; tv[3] = a.w;
-        dv[0] = d.x; dv[1] = d.y; dv[2] = d.z; dv[3] = d.w;
+#pragma unroll
+        for (int e = 0; e < kPer; e += 4) {
+            const float4 a = __ldg(reinterpret_cast<const float4 *>(trow + t0 + e));
+            float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (!target_only) d = __ldg(reinterpret_cast<const float4 *>(drow + t0 + e));
+            tv[e] = a.x; tv[e + 1] = a.y; tv[e + 2] = a.z; tv[e + 3] = a.w;
+            dv[e] = d.x; dv[e + 1] = d.y; dv[e + 2] = d.z; dv[e + 3] = d.w;
+        }
     } else {
 #pragma unroll
-        for (int e = 0; e < kAccPerThread; ++e) {
+        for (int e = 0; e < kPer; ++e) {
             const int t = t0 + e;
             tv[e] = t < V ? trow[t] : 0.f;
             dv[e] = (t < V && !target_only) ? drow[t] : 0.f;
         }
     }
 #pragma unroll
-    for (int e = 0; e < kAccPerThread; ++e) {
+    for (int e = 0; e < kPer; ++e) {
         w[e] = t0 + e < V ? weight_of(tv[e], dv[e], ri, target_only) : 0.0;
         s += w[e];
     }
@@ -176,6 +190,7 @@ __device__ __forceinline__ double chunk_local(const float *trow, const float *dr
 
 // Merge of the chunk statistics of every logit row of sequence b and the sequential accept tests.  Run by all
 // threads of a block; the result is identical in every block of the sequence (same data, same order).
+template <int T>
 __device__ __forceinline__ RowInfo decide_rows(const AcceptParams &p, int b, double *rowstat /* shared [2*gamma+1][3] */, int *s_n) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n_rows = 2 * p.gamma + 1;
@@ -188,7 +203,7 @@ __device__ __forceinline__ RowInfo decide_rows(const AcceptParams &p, int b, dou
         u0 = p.ua[(size_t)b * p.gamma + lane];
         if ((unsigned)tok0 < (unsigned)p.V) { tl0 = logit_row(p, b, lane)[tok0]; dl0 = logit_row(p, b, p.gamma + 1 + lane)[tok0]; }
     }
-    for (int r = warp; r < n_rows; r += kAccWarps) {
+    for (int r = warp; r < n_rows; r += T / 32) {
         const double2 *st = p.stats + ((size_t)b * n_rows + r) * p.n_chunks;
         double M = -INFINITY;
         for (int c = lane; c < p.n_chunks; c += 32) M = fmax(M, st[c].x);
@@ -236,13 +251,14 @@ __device__ __forceinline__ RowInfo decide_rows(const AcceptParams &p, int b, dou
 
 // Residual (or bonus) weights of one chunk of sequence b, scanned in token order.  Every caller re-derives the row
 // normalisers and the accept decisions of the sequence (same data, same order: identical everywhere).
+template <int T>
 __device__ __forceinline__ void weigh_item(const AcceptParams &p, int b, int c) {
     __shared__ double rowstat[3 * kAccMaxRows];
     __shared__ double warp_tot[kAccWarps];
     __shared__ int s_n;
     const int tid = threadIdx.x;
     __syncthreads();   // the shared arrays may still be read by the previous item
-    const RowInfo ri = decide_rows(p, b, rowstat, &s_n);
+    const RowInfo ri = decide_rows<T>(p, b, rowstat, &s_n);
     if (c == 0 && tid == 0) {
         const int32_t *x = p.x + (size_t)b * p.gamma;
         int32_t *out = p.out + (size_t)b * (p.gamma + 1);
@@ -253,19 +269,19 @@ __device__ __forceinline__ void weigh_item(const AcceptParams &p, int b, int c) 
     }
     const float *trow = logit_row(p, b, ri.n);
     const float *drow = ri.bonus ? nullptr : logit_row(p, b, p.gamma + 1 + ri.n);
-    double w[kAccPerThread], total;
-    double s = chunk_local(trow, drow, c, p.V, ri, ri.bonus != 0, w);
-    const double incl = block_scan_inclusive(s, warp_tot, &total);
-    constexpr int kPerGroup = kAccGroup / kAccPerThread;     // threads that share a group
+    constexpr int kPer = kAccChunk / T, kPerGroup = kAccGroup / kPer;     // tokens per thread, threads that share a group
+    double w[kPer], total;
+    const double s = chunk_local<T>(trow, drow, c, p.V, ri, ri.bonus != 0, w);
+    const double incl = block_scan_inclusive<T>(s, warp_tot, &total);
     if (tid % kPerGroup == kPerGroup - 1) p.tscan[((size_t)b * p.n_chunks + c) * kAccGroups + tid / kPerGroup] = incl;
-    if (tid == kAccThreads - 1) total = incl;                // the chunk's sum and the last group's are the same number
-    if (tid == kAccThreads - 1) p.wsum[(size_t)b * p.n_chunks + c] = total;
+    if (tid == T - 1) p.wsum[(size_t)b * p.n_chunks + c] = incl;          // the chunk's sum and the last group's are the same number
 }
 
-__global__ void __launch_bounds__(kAccThreads) accept_weigh_kernel(const AcceptParams p) {
+template <int T>
+__global__ void __launch_bounds__(T) accept_weigh_kernel(const AcceptParams p) {
     pdl_wait();
     pdl_trigger();
-    weigh_item(p, blockIdx.y, blockIdx.x);
+    weigh_item<T>(p, blockIdx.y, blockIdx.x);
 }
 
 // The emitted token of sequence b: chunk, 16-token group and token where the CDF crosses u * total.  ws: n_chunks doubles of
@@ -296,8 +312,8 @@ __device__ __forceinline__ void pick_item(const AcceptParams &p, int b, double *
         // residual is identically zero (P_n == Q_n): fall back to P_n; recompute the chunk totals
         __syncthreads();
         for (int c = 0; c < p.n_chunks; ++c) {
-            const double s = chunk_local(trow, drow, c, p.V, ri, true, w);
-            const double incl = block_scan_inclusive(s, warp_tot, &total);
+            const double s = chunk_local<kAccThreads>(trow, drow, c, p.V, ri, true, w);
+            const double incl = block_scan_inclusive<kAccThreads>(s, warp_tot, &total);
             if (tid == kAccThreads - 1) ws[c] = incl;
         }
         __syncthreads();
@@ -343,8 +359,8 @@ __device__ __forceinline__ void pick_item(const AcceptParams &p, int b, double *
             if (at >= 0) tok = c * kAccChunk + first * kAccGroup + at;
         }
     } else if (c >= 0) {
-        const double s = chunk_local(trow, drow, c, p.V, ri, target_only, w);
-        const double incl = block_scan_inclusive(s, warp_tot, &total);
+        const double s = chunk_local<kAccThreads>(trow, drow, c, p.V, ri, target_only, w);
+        const double incl = block_scan_inclusive<kAccThreads>(s, warp_tot, &total);
         double run = s_prefix + (incl - s);  // CDF just before this thread's first token
         int mine = 0x7fffffff;
 #pragma unroll
@@ -413,9 +429,9 @@ __global__ void __launch_bounds__(kAccThreads) accept_fused_kernel(const AcceptP
     pdl_trigger();
     const int rows = 2 * p.gamma + 1;
     for (int i = blockIdx.x; i < p.B * rows * p.n_chunks; i += gridDim.x)
-        stats_item(p, i / (rows * p.n_chunks), (i / p.n_chunks) % rows, i % p.n_chunks);
+        stats_item<kAccThreads>(p, i / (rows * p.n_chunks), (i / p.n_chunks) % rows, i % p.n_chunks);
     if (!accept_grid_barrier(hdr, 0)) return;
-    for (int i = blockIdx.x; i < p.B * p.n_chunks; i += gridDim.x) weigh_item(p, i / p.n_chunks, i % p.n_chunks);
+    for (int i = blockIdx.x; i < p.B * p.n_chunks; i += gridDim.x) weigh_item<kAccThreads>(p, i / p.n_chunks, i % p.n_chunks);
     if (!accept_grid_barrier(hdr, 1)) return;
     for (int b = blockIdx.x; b < p.B; b += gridDim.x) pick_item(p, b, ws);
 }
@@ -436,9 +452,10 @@ static AcceptWs accept_ws(int B, int gamma, int V) {
 // arg-max of the target row, then emit the target's arg-max (lowest token id on ties).
 //   argmax  per (sequence, target row, chunk): maximum and its first position -> stats[b][row][chunk] = (max, index)
 //   greedy  per sequence: merge the chunks of every row, compare with the draft tokens, write the outputs
-__global__ void __launch_bounds__(kAccThreads) accept_argmax_kernel(const AcceptParams p) {
-    __shared__ float smax[kAccWarps];
-    __shared__ int sidx[kAccWarps];
+template <int T>
+__global__ void __launch_bounds__(T) accept_argmax_kernel(const AcceptParams p) {
+    __shared__ float smax[T / 32];
+    __shared__ int sidx[T / 32];
     pdl_wait();
     pdl_trigger();
     const int c = blockIdx.x, r = blockIdx.y, b = blockIdx.z, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -446,8 +463,8 @@ __global__ void __launch_bounds__(kAccThreads) accept_argmax_kernel(const Accept
     float m = -INFINITY;
     int mi = 0x7fffffff;
 #pragma unroll
-    for (int e = 0; e < kAccPerThread; ++e) {
-        const int t = c * kAccChunk + e * kAccThreads + tid;     // ascending in e: a strict '>' keeps the first maximum
+    for (int e = 0; e < kAccChunk / T; ++e) {
+        const int t = c * kAccChunk + e * T + tid;     // ascending in e: a strict '>' keeps the first maximum
         const float v = t < p.V ? row[t] : -INFINITY;
         if (v > m || (v == m && t < mi && t < p.V)) { m = v; mi = t; }
     }
@@ -459,7 +476,7 @@ __global__ void __launch_bounds__(kAccThreads) accept_argmax_kernel(const Accept
     if (lane == 0) { smax[warp] = m; sidx[warp] = mi; }
     __syncthreads();
     if (warp == 0) {
-        m = smax[lane]; mi = sidx[lane];
+        m = smax[lane % (T / 32)]; mi = sidx[lane % (T / 32)];
         for (int o = 16; o; o >>= 1) {
             const float om = __shfl_xor_sync(0xffffffffu, m, o);
             const int oi = __shfl_xor_sync(0xffffffffu, mi, o);
@@ -508,7 +525,14 @@ static int32_t launch_accept_greedy(const AcceptParams &p, cudaStream_t s) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     cfg.gridDim = dim3((unsigned)p.n_chunks, (unsigned)(p.gamma + 1), (unsigned)p.B);
-    HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, accept_argmax_kernel, p));
+    if ((long long)p.n_chunks * (p.gamma + 1) * p.B <= 320) {        // as in the sampling mode
+        cfg.blockDim = dim3(512);
+        HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, accept_argmax_kernel<512>, p));
+    } else {
+        cfg.blockDim = dim3(256);
+        HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, accept_argmax_kernel<256>, p));
+    }
+    cfg.blockDim = dim3(kAccThreads);
     cfg.gridDim = dim3((unsigned)p.B);
     HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, accept_greedy_kernel, p));
     count_launches(2);
@@ -526,9 +550,26 @@ static int32_t launch_accept_chain(const AcceptParams &p, cudaStream_t s) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     cfg.gridDim = dim3((unsigned)p.n_chunks, (unsigned)(2 * p.gamma + 1), (unsigned)p.B);
-    HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, accept_stats_kernel, p));
+    // Threads per chunk: many while the chunks leave SMs idle (latency), few once there is a wave of them or more (the block's
+    // meetings then cost more than they hide).  Vocabulary 152,064, us with 1,024 / 512 / 256 threads for the statistics: batch 1
+    // 23.8 / 22.8 / 23.2, batch 2 27.2 / 25.7 / 24.7, batch 8 61.6 / 53.8 / 52.4; for the weights: batch 1 22.8 / 23.6 / 32.5,
+    // batch 4 29.5 / 30.0 / 32.5, batch 8 55.2 / 52.4 / 51.6.
+    if ((long long)p.n_chunks * (2 * p.gamma + 1) * p.B <= 640) {
+        cfg.blockDim = dim3(512);
+        HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, accept_stats_kernel<512>, p));
+    } else {
+        cfg.blockDim = dim3(256);
+        HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, accept_stats_kernel<256>, p));
+    }
     cfg.gridDim = dim3((unsigned)p.n_chunks, (unsigned)p.B);
-    HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, accept_weigh_kernel, p));
+    if ((long long)p.n_chunks * p.B <= kNumSMs) {
+        cfg.blockDim = dim3(1024);
+        HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, accept_weigh_kernel<1024>, p));
+    } else {
+        cfg.blockDim = dim3(256);
+        HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, accept_weigh_kernel<256>, p));
+    }
+    cfg.blockDim = dim3(kAccThreads);
     cfg.gridDim = dim3((unsigned)p.B);
     cfg.dynamicSmemBytes = (size_t)p.n_chunks * sizeof(double);
     HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, accept_pick_kernel, p));
