@@ -158,7 +158,8 @@ int32_t hippo_attention_mass(int32_t batch, const int32_t *n_visual, int32_t l_t
  *             offset kept_offsets[b]; kept_offsets (host int32 [batch]) may be NULL, meaning sum(k[0..b)).  Explicit
  *             offsets let the caller interleave other entries (e.g. always-kept text positions) in the same list.
  *   fused_score out fp32 [sum n_visual]
- * Scores are accumulated in fp64.  embed_dim must be a multiple of 8; crop_h*crop_w <= 32.
+ * Scores have the accuracy of fp64 sums (bf16: exact integer sums of 8-bit digits plus a remainder, on the tensor cores; fp32:
+ * fp64).  embed_dim must be a multiple of 8; crop_h*crop_w <= 32.
  */
 size_t hippo_select_workspace_bytes(int32_t batch, const int32_t *n_visual, int32_t grid_h, int32_t grid_w,
                                     int32_t crop_h, int32_t crop_w);
@@ -273,7 +274,7 @@ int32_t hippo_draft_attention(int32_t batch, int32_t q_len, int32_t n_q_heads, c
  *                          shared memory) from the first layer to the last, so a caller that wants kernels of another
  *                          stream to run beside it - the draft model's, Section 5.2 - leaves them some SMs this way
  * The host arrays are read before the call returns.  The call enqueues one memset of its counters and one kernel
- * per 64 layers.  The workspace is larger than a single-layer one (three sets of partial-result slots and per-layer
+ * per 64 layers.  The workspace is larger than a single-layer one (six sets of partial-result slots and per-layer
  * counters): size it with hippo_verify_attention_layers_workspace_bytes.  bf16 with head_dim 64 or 128 and at most
  * 256 (sequence, kv head) units use the multi-layer kernel; every other shape is run layer by layer on the
  * single-layer paths, with the same results.  Because the CTAs of the launch wait for one another's partial results,
