@@ -40,6 +40,8 @@ __global__ void __launch_bounds__(kGatherThreads) gather_kv_kernel(const GatherP
     if (x >= per_plane) return;
     const uint32_t c = x % (uint32_t)p.row_chunks, y = x / (uint32_t)p.row_chunks;
     const int i = (int)(y % (uint32_t)p.total_keep), h = (int)(y / (uint32_t)p.total_keep);
+    asm volatile("griddepcontrol.wait;" ::: "memory");           // the launch overlaps the end of its predecessor in the stream
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // sequence of flat keep index i: largest b with keep_offsets[b] <= i
     int lo = 0, hi = p.batch;
     while (hi - lo > 1) {
@@ -145,8 +147,16 @@ extern "C" int32_t hippo_gather_kv(int32_t n_layers, const hippo_kv_cache_t *src
     if (p.planes_per_group > kGatherUnroll) p.planes_per_group = kGatherUnroll;
     gy = (2 * n_layers + p.planes_per_group - 1) / p.planes_per_group;
     if (bx > 0x7fffffffLL || gy > 65535) return fail(HIPPO_ERR_UNSUPPORTED_SHAPE, "hippo_gather_kv: grid too large");
-    gather_kv_kernel<<<dim3((unsigned)bx, (unsigned)gy), kGatherThreads, 0, (cudaStream_t)stream>>>(p);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)bx, (unsigned)gy);
+    cfg.blockDim = dim3(kGatherThreads);
+    cfg.stream = (cudaStream_t)stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, gather_kv_kernel, p));
     count_launches(1);
-    HIPPO_CUDA_TRY(cudaGetLastError());
     return HIPPO_OK;
 }
