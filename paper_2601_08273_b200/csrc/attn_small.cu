@@ -20,7 +20,7 @@
 //
 // Bound by latency: two dependent round trips to memory (lengths and page ids, then keys and values; one for an
 // identity-mapped cache), the softmax and the merge.  Measured per call in a chain of 28 layers: 758 keys (0.39 MB) 3.5 us, 5.8 us
-// with the CUDA-core kernel that stood here before; 3,537 keys (1.8 MB, from HBM) 4.7 us, 10.5 us through tensor memory.
+// with the CUDA-core kernel that stood here before; 3,537 keys (1.8 MB, from HBM) 4.3 us, 10.5 us through tensor memory.
 //
 // The warps of a CTA merge through shared memory.  Row r of the unit is merged by CTA r mod cluster size: every CTA
 // pushes its (m, l, O[r]) into that CTA's shared memory with remote stores, and after a cluster barrier the owners
@@ -51,6 +51,12 @@ __device__ __forceinline__ uint4 sm_ldg(const __nv_bfloat16 *p) { return __ldg(r
 __device__ __forceinline__ uint4 sm_ldg_hint(const __nv_bfloat16 *p, uint64_t pol) {
     uint4 v;
     asm("ld.global.nc.L2::cache_hint.v4.b32 {%0, %1, %2, %3}, [%4], %5;" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(pol));
+    return v;
+}
+// a word that another kernel may be writing: from L2, so that no old line stays in L1
+__device__ __forceinline__ int sm_peek(const int32_t *p) {
+    int v;
+    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
 __device__ __forceinline__ void sm_mma(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
@@ -123,6 +129,31 @@ __device__ __noinline__ void attn_small_redo(const AttnParams &p, int b, int hk,
     }
 }
 
+// Ahead of the wait for the predecessor in the stream: asks L2 for what the warp is going to read.  These are hints and nothing else: a
+// line that the predecessor writes later is current in L2 all the same, and the values used here (length, page ids) are looked up again
+// after the wait.  They may be stale or not yet written, so they count only inside their bounds.  us per call in a chain of 28, cold
+// caches: 758 keys 4.0 -> 3.9, 3,537 keys 4.9 -> 4.3, 33,000 keys 13.7 -> 11.7, eight sequences of 2,000 keys 8.1 -> 6.6.
+template <int D>
+__device__ __forceinline__ void sm_prefetch(const AttnParams &p, int b, int hk, int first, int stride, bool queries, int max_blocks, uint64_t pol) {
+    const int lane = threadIdx.x & 31;
+    if (queries && lane < p.q_len) {
+        const __nv_bfloat16 *q = (const __nv_bfloat16 *)p.q + (((size_t)b * p.q_len + lane) * p.n_q_heads + hk * p.group) * D;
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(q), "r"((uint32_t)(p.group * D * 2)) : "memory");
+    }
+    // the first step's blocks; later ones, and those behind a page table, only as far as the length is known to reach
+    const int blk = first + (lane >> 1) * stride;
+    if (blk >= max_blocks) return;
+    int pid = b * p.max_pages_per_seq + blk / (kPageSize / kSmBlock);
+    if (p.page_table || blk != first) {
+        if (p.kv_len && blk * kSmBlock >= sm_peek(p.kv_len + b)) return;
+        if (p.page_table) pid = sm_peek(p.page_table + (size_t)b * p.max_pages_per_seq + blk / (kPageSize / kSmBlock));
+    }
+    if ((unsigned)pid >= (unsigned)p.n_pages) return;
+    const __nv_bfloat16 *src = (const __nv_bfloat16 *)(lane & 1 ? p.v_pages : p.k_pages) +
+                               (((size_t)pid * p.n_kv_heads + hk) * kPageSize + (blk % (kPageSize / kSmBlock)) * kSmBlock) * D;
+    asm volatile("cp.async.bulk.prefetch.L2.global.L2::cache_hint [%0], %1, %2;" ::"l"(src), "r"((uint32_t)(kSmBlock * D * 2)), "l"(pol) : "memory");
+}
+
 template <int D, int NT>   // head size; groups of eight packed rows
 __global__ void __launch_bounds__(D == 64 ? 512 : 256) attn_small_kernel(const __grid_constant__ AttnParams p, const int cluster_size) {
     using S = SmallSmem<D, NT>;
@@ -138,27 +169,30 @@ __global__ void __launch_bounds__(D == 64 ? 512 : 256) attn_small_kernel(const _
     const int stride = W * cluster_size;                        // blocks of 32 keys from one step of this warp to the next
     const int first = warp * cluster_size + rank;
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");     // this CTA runs: its peers may push into its memory
+    const int max_blocks = (p.max_kv_len + kSmBlock - 1) / kSmBlock;
+    // the draft's pruned cache is read again by every token: kept in L2 beside a verification pass that streams through it (28 layers
+    // hold 13 - 25 MB of 126; beside 104 SMs of verification the 32k step takes 1,425 us with either policy)
+    const uint64_t pol = p.kv_resident ? l2_policy_evict_last() : l2_policy_evict_first();
+    const __nv_bfloat16 *q_rows[NT];                            // this lane's part of its query rows
+#pragma unroll
+    for (int n = 0; n < NT; ++n) {
+        const int r = g + 8 * n, tq = r / G, gq = r - tq * G;
+        q_rows[n] = (const __nv_bfloat16 *)p.q + (((size_t)b * p.q_len + tq) * p.n_q_heads + hk * G + gq) * D + t * 8;
+    }
+    sm_prefetch<D>(p, b, hk, first, stride, rank == 0 && warp == 0, max_blocks, pol);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     int kvl = p.kv_len ? __ldg(p.kv_len + b) : p.max_kv_len;    // no length array: every sequence has max_kv_len keys
     if (kvl < p.q_len) kvl = 0;                                 // skipped: its row of the page table may hold anything
-    const int max_blocks = (p.max_kv_len + kSmBlock - 1) / kSmBlock;
 
     // query rows as A operand; the contraction order is the one of the keys' loads
     uint4 qr[NT][kKV4];
 #pragma unroll
-    for (int n = 0; n < NT; ++n) {
-        const int r = g + 8 * n, tq = r / G, gq = r - tq * G;
+    for (int n = 0; n < NT; ++n)
 #pragma unroll
-        for (int j = 0; j < kKV4; ++j)
-            qr[n][j] = r < R ? sm_ldg((const __nv_bfloat16 *)p.q + (((size_t)b * p.q_len + tq) * p.n_q_heads + hk * G + gq) * D + j * 32 + t * 8)
-                             : make_uint4(0, 0, 0, 0);
-    }
+        for (int j = 0; j < kKV4; ++j) qr[n][j] = g + 8 * n < R ? sm_ldg(q_rows[n] + j * 32) : make_uint4(0, 0, 0, 0);
     const float sl2 = p.scale * kSmLog2e;
-    // the draft's pruned cache is read again by every token: kept in L2 beside a verification pass that streams through it (28 layers
-    // hold 13 - 25 MB of 126; beside 104 SMs of verification the 32k step takes 1,425 us with either policy)
-    const uint64_t pol = p.kv_resident ? l2_policy_evict_last() : l2_policy_evict_first();
 
     float o[NT][kDT][4], m[NT], l[NT];
 #pragma unroll
