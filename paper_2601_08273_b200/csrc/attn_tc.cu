@@ -49,6 +49,9 @@
 #include <stddef.h>
 #include <string.h>
 
+#include <algorithm>
+#include <utility>
+
 #include "common.cuh"
 #include "tc_ptx.cuh"
 
@@ -282,7 +285,7 @@ attn_tc_kernel(const AttnParams p, const __grid_constant__ LayerSetT<NL> set, co
     // ---- set-up: barriers, tile prefix, CTA split, tensor memory
     const int U = B * Hkv;
     const bool clustered = cluster_size > 1;                  // one cluster per unit, merge through shared memory
-    const bool aligned = !clustered && U <= (int)gridDim.x && U <= kMaxAlignedUnits;
+    const bool aligned = cluster_size == 0 && U <= (int)gridDim.x && U <= kMaxAlignedUnits;
     const bool small_problem = U <= 32;                       // tile prefix and CTA split by warp 0 alone, no block barriers
     {
         // one barrier per thread of warps 1..: [0, n_slots) full, [n_slots, 2 n_slots) empty, then the fixed ones
@@ -353,7 +356,8 @@ attn_tc_kernel(const AttnParams p, const __grid_constant__ LayerSetT<NL> set, co
 
     Partition part;
     part.total = (long long)sh->tile_prefix[B] * Hkv;
-    part.grid = gridDim.x;
+    // the flat split: no CTA without a tile between two that share a unit (the merge counts the CTAs from the first to the last)
+    part.grid = clustered || aligned || part.total >= (long long)gridDim.x ? (int)gridDim.x : part.total > 0 ? (int)part.total : 1;
     int2 *unit_info = reinterpret_cast<int2 *>(p.counters);   // per unit: first slot, number of contributing CTAs
     if (aligned && !small_problem) {
         // CTAs per unit: one each, the others in proportion to the tile counts (largest remainders first)
@@ -415,7 +419,7 @@ attn_tc_kernel(const AttnParams p, const __grid_constant__ LayerSetT<NL> set, co
                 t_begin = unit_start + T * i / nc;
                 t_end = unit_start + T * (i + 1) / nc;
             }
-        } else if (part.total > 0) {
+        } else if (part.total > 0 && c < part.grid) {
             t_begin = part.start_of(c);
             t_end = part.start_of(c + 1);
         }
@@ -1232,6 +1236,88 @@ __global__ void __launch_bounds__(kCombineThreads) attn_tc_combine_kernel(const 
     }
 }
 
+// The same merge where a unit has a handful of contributors: a warp per row, eight rows per CTA.  Up to eight contributors' values of a
+// row are in flight together (lane j fetches (m, l) of contributor j, every lane its output columns of all of them), so a row is one
+// round trip, and the whole grid is resident while the main kernel runs (the kernel above, a CTA per row with five of its warps idle, is
+// more than one wave of CTAs from 1,184 rows on: eight ragged sequences of 10,406 keys, 1,344 rows, 46.4 us a call, 41.8 with this one).
+template <int D>
+__global__ void __launch_bounds__(kCombineThreads) attn_tc_combine_rows_kernel(const AttnParams p, const int main_grid, const int n_rows) {
+    constexpr int V = D / 32, kBatch = 8;
+    __shared__ int2 s_info[32];
+    const int R = p.rows, G = p.group, Hkv = p.n_kv_heads;
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    if (main_grid > 0) {                              // as above
+        if (w == 0) {
+            const int U = p.batch * Hkv;
+            const int kvl = lane < p.batch ? (p.kv_len ? __ldcg(p.kv_len + lane) : p.max_kv_len) : 0;
+            const int nt = lane < p.batch ? seq_tiles(kvl, p.q_len) : 0;
+            int sum = nt;
+#pragma unroll
+            for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            const int my_tiles = __shfl_sync(0xffffffffu, nt, lane < U ? lane / Hkv : 0);
+            int all;
+            s_info[lane] = aligned_split_warp(lane, U, main_grid, lane < U ? my_tiles : 0, (long long)sum * Hkv, all);
+        }
+        __syncthreads();
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int row = blockIdx.x * (kCombineThreads / 32) + w;
+    if (row >= n_rows) return;
+    const int h = row % p.n_q_heads, t = (row / p.n_q_heads) % p.q_len, b = row / (p.n_q_heads * p.q_len);
+    const int unit = b * Hkv + h / G, r = t * G + (h % G);
+    const int2 info = main_grid > 0 ? s_info[unit] : reinterpret_cast<const int2 *>(p.counters)[unit];   // first slot, contributors
+    const int n = info.y;
+    if (n == 1) return;
+    const size_t slot_floats = slot_float_count(R, D);
+    const int Rp = slot_rows_padded(R);
+    const float *base = p.partials + (size_t)info.x * slot_floats;
+    float M = -INFINITY, L = 0.f, acc[V];
+#pragma unroll
+    for (int x = 0; x < V; ++x) acc[x] = 0.f;
+    for (int c0 = 0; c0 < n; c0 += kBatch) {
+        const bool mine = lane < kBatch && c0 + lane < n;
+        const float *ml = base + (size_t)(mine ? c0 + lane : 0) * slot_floats + r;
+        const float m = mine ? ml[0] : -INFINITY, l = mine ? ml[Rp] : 0.f;
+        float v[kBatch][V];
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+            const float *src = base + (size_t)min(c0 + j, n - 1) * slot_floats + 2 * Rp + (size_t)r * D + lane * V;   // clamped: not used
+            if (V == 4) {
+                const float4 t4 = *reinterpret_cast<const float4 *>(src);
+                v[j][0] = t4.x; v[j][1] = t4.y; v[j][V - 2] = t4.z; v[j][V - 1] = t4.w;
+            } else {
+                const float2 t2 = *reinterpret_cast<const float2 *>(src);
+                v[j][0] = t2.x; v[j][1] = t2.y;
+            }
+        }
+        float top = m;
+#pragma unroll
+        for (int o = kBatch / 2; o; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+        const float m_new = fmaxf(M, __shfl_sync(0xffffffffu, top, 0));
+        const float f_old = M == -INFINITY ? 0.f : expf(M - m_new), f_mine = m == -INFINITY ? 0.f : expf(m - m_new);
+        const unsigned seen = __ballot_sync(0xffffffffu, m != -INFINITY);      // a contributor without a visible key adds nothing
+        L *= f_old;
+#pragma unroll
+        for (int x = 0; x < V; ++x) acc[x] *= f_old;
+#pragma unroll
+        for (int j = 0; j < kBatch; ++j) {
+            if (!(seen >> j & 1u)) continue;
+            const float f = __shfl_sync(0xffffffffu, f_mine, j);
+            L += __shfl_sync(0xffffffffu, l, j) * f;
+#pragma unroll
+            for (int x = 0; x < V; ++x) acc[x] += v[j][x] * f;
+        }
+        M = m_new;
+    }
+    // a sequence shorter than q_len is skipped (n = 0): its outputs are defined as zero
+    __nv_bfloat16 *out = (__nv_bfloat16 *)p.out + (size_t)row * D + lane * V;
+#pragma unroll
+    for (int x = 0; x < V; x += 2)
+        *reinterpret_cast<__nv_bfloat162 *>(out + x) = __floats2bfloat162_rn(L > 0.f ? acc[x] / L : 0.f, L > 0.f ? acc[x + 1] / L : 0.f);
+    if (p.lse && lane == 0) p.lse[row] = L > 0.f ? M + logf(L) : -INFINITY;
+}
+
 // ---- host side -----------------------------------------------------------------------------------------------------
 EncodeTiledFn tensor_map_encoder() {
     static EncodeTiledFn fn = nullptr;
@@ -1263,24 +1349,6 @@ bool attn_tc_supported(const AttnParams &p, int dtype) {
            p.rows <= kMaxRows;
 }
 
-// Cluster size for the one-cluster-per-unit mode, or 0 for the split modes.  `pages` = pages of the longest unit,
-// `total_pages` = pages of all units (exact when the caller passed the lengths on the host, else units * pages);
-// max_active[cs] = clusters of cs CTAs of this kernel that the device keeps resident at once.  The cluster mode
-// needs no second kernel, but all clusters must be resident together, a unit gets at most 16 SMs and the longest
-// unit sets the time, so long caches with few units and ragged batches stay on the split path.
-static int choose_cluster_size(int units, int pages, long long total_pages, int total_rows, const int *max_active) {
-    // costs in pages per CTA (ranges are cut on page boundaries); the second kernel of the split modes is worth ten, and
-    // one more for every 128 output rows it merges (measured: 8 ragged sequences of 168 rows, 35 pages per CTA in the split
-    // mode against 50 in the cluster mode, 46.4 us against 43.7 us)
-    int best = 0, best_cost = (int)((total_pages + kNumSMs - 1) / kNumSMs) + 10 + total_rows / 128;
-    for (int cs = 2; cs <= 16 && 2 * cs <= pages + 1; ++cs) {
-        if (units > max_active[cs]) continue;
-        const int cost = ceil_div(pages, cs);
-        if (cost < best_cost || (cost == best_cost && best == 0)) { best = cs; best_cost = cost; }
-    }
-    return best;
-}
-
 // Pages of the longest unit and of all units together, from the host copy of the lengths when there is one.
 static void plan_pages(const AttnParams &p, int &longest, long long &total) {
     const int bound = ceil_div(p.max_kv_len, kPageSize);
@@ -1298,6 +1366,79 @@ static void plan_pages(const AttnParams &p, int &longest, long long &total) {
         }
         if (longest < 1) longest = 1;
     }
+}
+
+// Grid of the split modes: one CTA per SM, never more CTAs than pages (bound from the host-side length bound; the
+// kernel derives the exact partition from kv_len on the device).
+static int split_grid(const AttnParams &p, int sms) {
+    const long long max_tiles = (long long)p.batch * p.n_kv_heads * ceil_div(p.max_kv_len, kPageSize);
+    long long grid = p.num_splits > 0 ? (long long)p.num_splits * p.batch * p.n_kv_heads : sms;
+    if (grid > max_tiles) grid = max_tiles;
+    if (grid > kExtraSlots) grid = kExtraSlots;
+    if (grid < 1) grid = 1;
+    return (int)grid;
+}
+
+// Pages of the longest CTA range of the unit-aligned split, as aligned_split_warp deals the CTAs out (0: more units than CTAs).
+static int aligned_longest(const AttnParams &p, int grid) {
+    const int U = p.batch * p.n_kv_heads;
+    if (U > grid || U > kMaxAlignedUnits) return 0;
+    auto pages = [&](int b) {
+        const int kvl = p.kv_len_host ? (p.kv_len_host[b] < p.max_kv_len ? p.kv_len_host[b] : p.max_kv_len) : p.max_kv_len;
+        return kvl < p.q_len ? 0 : ceil_div(kvl, kPageSize);
+    };
+    long long total = 0;
+    int live = 0, given = 0;
+    for (int b = 0; b < p.batch; ++b) { total += (long long)pages(b) * p.n_kv_heads; live += pages(b) > 0 ? p.n_kv_heads : 0; }
+    if (total == 0) return 1;
+    const int spare = grid - live;
+    std::pair<long long, int> rest[kMaxAlignedUnits];          // remainder of a sequence's units, sequence
+    for (int b = 0; b < p.batch; ++b) {
+        const long long num = (long long)spare * pages(b);
+        given += (int)(num / total) * p.n_kv_heads;
+        rest[b] = {num % total, b};
+    }
+    std::sort(rest, rest + p.batch, [](const auto &x, const auto &y) { return x.first > y.first || (x.first == y.first && x.second < y.second); });
+    int longest = 1, left = spare - given;
+    for (int i = 0; i < p.batch; ++i) {                        // a sequence's units have the same remainder: some or all get one more
+        const int t = pages(rest[i].second), n = 1 + (int)((long long)spare * t / total);
+        if (t == 0) continue;
+        const int with = left < p.n_kv_heads ? (left < 0 ? 0 : left) : p.n_kv_heads;
+        left -= with;
+        const int share = ceil_div(t, with == p.n_kv_heads ? n + 1 : n);
+        if (share > longest) longest = share;
+    }
+    return longest;
+}
+
+// How a single-layer call is split: > 1 one cluster of so many CTAs per unit, kAligned or kFlat.  Times in us of a call in a chain of
+// them, by the pages of the longest CTA (up to 32 packed rows / each 16 rows more): clusters 12 + 0.53 per page / 1.3 and 0.09, then 0.055 (128
+// CTAs saturate HBM as well as 148), aligned 14.5 + 0.645 / 0.055, flat 15.5 + 0.667 / 0.055 (1.5 besides) with the average in place of the
+// longest.  Measured, clusters / aligned / flat, head size 128: eight ragged sequences of 10,406 keys, 4 kv heads, 42 rows 45.8 / 41.8 / 43.8;
+// of 12,000, 8 kv heads, 24 rows 70.0 / 79.9 / 70.7; of 9,000, 8 kv heads, 48 rows 65.0 / 66.4 / 59.6; four of 13,000, 8 kv heads, 24 rows
+// 42.6 / 46.5 / 44.4, of 3,000 with 72 rows 26.8 / 25.1 / 29.6; one of 3,000, 48 rows 14.0 / 15.7 / 18.5, of 8,000 20.2 / 19.1 / 21.5.  Head
+// size 64, eight of 10,406, 42 rows: 38.5 / 35.2 / 36.2.
+constexpr int kAligned = 0, kFlat = -1;
+static int choose_split(const AttnParams &p, int rows_padded, const int *max_active) {
+    const int units = p.batch * p.n_kv_heads, groups = rows_padded / 16;
+    int pages;
+    long long total_pages;
+    plan_pages(p, pages, total_pages);
+    const float more = groups <= 2 ? 0.f : groups - 2.f;                                  // groups of rows beyond 32
+    const int even = aligned_longest(p, split_grid(p, kNumSMs));
+    int best = kFlat;
+    float best_us = 15.5f + 1.5f * (groups > 2) + (0.667f + 0.055f * more) * (float)((total_pages + kNumSMs - 1) / kNumSMs);
+    if (even > 0) {
+        const float us = 14.5f + (0.645f + 0.055f * more) * even;
+        if (us < best_us) { best = kAligned; best_us = us; }
+    }
+    // a cluster of more than eight needs most of a GPC, and only six of them can be counted on to hold one
+    for (int cs = 2; cs <= (units <= 6 ? 16 : 8) && 2 * cs <= pages + 1; ++cs) {
+        if (units > max_active[cs]) continue;
+        const float us = 12.f + 1.3f * more + (0.53f + 0.09f * (more > 0.f) + 0.055f * (more > 1.f ? more - 1.f : 0.f)) * ceil_div(pages, cs);
+        if (us < best_us) { best = cs; best_us = us; }
+    }
+    return best;
 }
 
 struct TcLaunchShape { int Rp, spare_cols, tmem_cols; TcSmemPlan plan; };
@@ -1353,10 +1494,7 @@ static int32_t launch_tc(const AttnParams &p, int grid, cudaStream_t stream) {
         }
         have_active[plan.slots].store(true, std::memory_order_release);
     }
-    int longest;
-    long long total_pages;
-    plan_pages(p, longest, total_pages);
-    const int cs = p.num_splits > 0 ? 0 : choose_cluster_size(units, longest, total_pages, p.batch * p.q_len * p.n_q_heads, max_active[plan.slots]);
+    const int split = p.num_splits > 0 ? kAligned : choose_split(p, sh.Rp, max_active[plan.slots]);
     // Both kernels are launched with programmatic stream serialization and wait (griddepcontrol.wait) before they
     // touch memory, so stream order is kept while launch latency overlaps the previous kernel's tail.
     cudaLaunchAttribute attr[2];
@@ -1367,16 +1505,16 @@ static int32_t launch_tc(const AttnParams &p, int grid, cudaStream_t stream) {
     cfg.dynamicSmemBytes = (size_t)plan.total;
     cfg.stream = stream;
     cfg.attrs = attr;
-    if (cs > 1) {
+    if (split > 1) {
         // one cluster per unit; the partial of a CTA (m, l, O) must fit in its ring memory
         attr[1].id = cudaLaunchAttributeClusterDimension;
-        attr[1].val.clusterDim.x = (unsigned)cs;
+        attr[1].val.clusterDim.x = (unsigned)split;
         attr[1].val.clusterDim.y = 1;
         attr[1].val.clusterDim.z = 1;
         cfg.numAttrs = 2;
-        cfg.gridDim = dim3((unsigned)(units * cs));
+        cfg.gridDim = dim3((unsigned)(units * split));
         if (slot_float_count(p.rows, D) * sizeof(float) <= (size_t)plan.slots * kBlockN * D * 2 &&
-            cudaLaunchKernelEx(&cfg, attn_tc_kernel<D, 1>, p, set, mc, sh.Rp, plan.slots, sh.tmem_cols, cs, sh.spare_cols) == cudaSuccess) {
+            cudaLaunchKernelEx(&cfg, attn_tc_kernel<D, 1>, p, set, mc, sh.Rp, plan.slots, sh.tmem_cols, split, sh.spare_cols) == cudaSuccess) {
             count_launches(1);
             return HIPPO_OK;
         }
@@ -1384,27 +1522,23 @@ static int32_t launch_tc(const AttnParams &p, int grid, cudaStream_t stream) {
     }
     cfg.numAttrs = 1;
     cfg.gridDim = dim3((unsigned)grid);
-    HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_kernel<D, 1>, p, set, mc, sh.Rp, plan.slots, sh.tmem_cols, 0, sh.spare_cols));
+    const int mode = split == kFlat ? kFlat : kAligned;
+    HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_kernel<D, 1>, p, set, mc, sh.Rp, plan.slots, sh.tmem_cols, mode, sh.spare_cols));
     count_launches(1);
-    cfg.gridDim = dim3((unsigned)(p.batch * p.q_len * p.n_q_heads));
+    const int n_rows = p.batch * p.q_len * p.n_q_heads;
     cfg.blockDim = dim3(kCombineThreads);
     cfg.dynamicSmemBytes = 0;
     // unit-aligned split by one warp (see the kernel): the combine kernel derives the slot table itself
-    const int derive = (units <= grid && units <= 32) ? grid : 0;
-    HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_combine_kernel<D>, p, derive));
+    const int derive = (mode == kAligned && units <= grid && units <= 32) ? grid : 0;
+    if (grid <= 8 * units) {             // one round trip per row
+        cfg.gridDim = dim3((unsigned)ceil_div(n_rows, kCombineThreads / 32));
+        HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_combine_rows_kernel<D>, p, derive, n_rows));
+    } else {
+        cfg.gridDim = dim3((unsigned)n_rows);
+        HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_combine_kernel<D>, p, derive));
+    }
     count_launches(1);
     return HIPPO_OK;
-}
-
-// Grid of the split modes: one CTA per SM, never more CTAs than pages (bound from the host-side length bound; the
-// kernel derives the exact partition from kv_len on the device).
-static int split_grid(const AttnParams &p, int sms) {
-    const long long max_tiles = (long long)p.batch * p.n_kv_heads * ceil_div(p.max_kv_len, kPageSize);
-    long long grid = p.num_splits > 0 ? (long long)p.num_splits * p.batch * p.n_kv_heads : sms;
-    if (grid > max_tiles) grid = max_tiles;
-    if (grid > kExtraSlots) grid = kExtraSlots;
-    if (grid < 1) grid = 1;
-    return (int)grid;
 }
 
 int32_t launch_attn_tc(const AttnParams &p, cudaStream_t stream) {
