@@ -50,10 +50,11 @@ template <> __device__ __forceinline__ void load8<float>(const float *p, double 
 }
 
 // One warp per token; a lane takes 8 consecutive elements per step (embed_dim is a multiple of 8).
+constexpr int kDotsThreads = 256;
 template <typename T>
-__global__ void __launch_bounds__(256) select_dots_kernel(const SelectParams p) {
+__device__ __forceinline__ void select_dots(const SelectParams &p, int block) {
     const int total = p.seq_off[p.batch];
-    const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int j = block * (kDotsThreads / 32) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (j >= total) return;
     const int b = find_seq(p.seq_off, p.batch, j);
@@ -75,6 +76,12 @@ __global__ void __launch_bounds__(256) select_dots_kernel(const SelectParams p) 
     n2 = warp_sum(n2);
     td = warp_sum(td);
     if (lane == 0) { p.norm2[j] = n2; p.tdot[j] = td; }
+}
+template <typename T>
+__global__ void __launch_bounds__(kDotsThreads) select_dots_kernel(const SelectParams p) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    select_dots<T>(p, (int)blockIdx.x);
 }
 
 // ---- spatial score on the fp64 tensor path: one CTA per crop ---------------------------------------------------------
@@ -128,16 +135,25 @@ __device__ __forceinline__ void load_frag4(const float *p, double *v) {
     v[0] = (double)a.x; v[1] = (double)a.y; v[2] = (double)a.z; v[3] = (double)a.w;
 }
 
+// The blocks behind the crops' form the norms and the products with the next frame, which need nothing of the crops: one launch for
+// both (whole selection of 2,048 tokens of 1,024, bf16: 29.3 us with two, 27.4).
 template <typename T>
 __global__ void __launch_bounds__(kMmaThreads, 3) select_spatial_mma_kernel(const SelectParams p) {
+    static_assert(kMmaThreads == kDotsThreads, "one launch for both");
     using Sh = MmaShape<T>;
     extern __shared__ __align__(16) uint8_t mma_smem[];   // ring of staged chunks; reused for the warps' partial tiles
     __shared__ int tok[kMaxCrop];
     __shared__ double S[kMaxCrop][kMaxCrop + 1];
-    __shared__ double nrm2[kMaxCrop];
+    __shared__ double root[kMaxCrop];
     __shared__ double tail_red[kMmaWarps][kMaxCrop + 1];
     __shared__ int s_M;
-    const int crops_per_frame = p.crops_y * p.crops_x;
+    const int crops_per_frame = p.crops_y * p.crops_x, n_crops = p.frame_off[p.batch] * crops_per_frame;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if ((int)blockIdx.x >= n_crops) {
+        select_dots<T>(p, (int)blockIdx.x - n_crops);
+        return;
+    }
     const int gframe = blockIdx.x / crops_per_frame, cr = blockIdx.x % crops_per_frame;
     const int b = find_seq(p.frame_off, p.batch, gframe);
     const int f = gframe - p.frame_off[b];
@@ -289,13 +305,13 @@ __global__ void __launch_bounds__(kMmaThreads, 3) select_spatial_mma_kernel(cons
             S[a][c] = g;
         }
         __syncthreads();
-        if (tid < M) nrm2[tid] = S[tid][tid];
+        if (tid < M) root[tid] = S[tid][tid] > 0.0 ? sqrt(S[tid][tid]) : 0.0;
         __syncthreads();
         for (int x = tid; x < M * M; x += kMmaThreads) {
             const int a = x / M, c = x % M;
             if (a >= c) continue;
-            const double na = nrm2[a], nc = nrm2[c];
-            const double cs = (na > 0.0 && nc > 0.0) ? S[a][c] / (sqrt(na) * sqrt(nc)) : 0.0;
+            const double na = root[a], nc = root[c];
+            const double cs = (na > 0.0 && nc > 0.0) ? S[a][c] / (na * nc) : 0.0;
             S[a][c] = cs;
             S[c][a] = cs;
         }
@@ -303,15 +319,20 @@ __global__ void __launch_bounds__(kMmaThreads, 3) select_spatial_mma_kernel(cons
     }
     if (tid < M) S[tid][tid] = 1.0;
     __syncthreads();
-    if (tid < M) {
-        const int a = tid;
-        double mu = 0.0;
-        for (int c = 0; c < M; ++c) mu += S[a][c];
-        mu /= M;
-        double var = 0.0;
-        for (int c = 0; c < M; ++c) var += (S[a][c] - mu) * (S[a][c] - mu);
-        p.s_spa[tok[a]] = var / M;
-    }
+    // eight threads per row
+    static_assert(kMmaThreads == 8 * kMaxCrop, "a row of the matrix per eight threads");
+    const int a = tid >> 3;
+    double mu = 0.0, var = 0.0;
+    if (a < M)
+        for (int c = tid & 7; c < M; c += 8) mu += S[a][c];
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) mu += __shfl_xor_sync(0xffffffffu, mu, o);
+    mu /= M;
+    if (a < M)
+        for (int c = tid & 7; c < M; c += 8) var += (S[a][c] - mu) * (S[a][c] - mu);
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) var += __shfl_xor_sync(0xffffffffu, var, o);
+    if (a < M && (tid & 7) == 0) p.s_spa[tok[a]] = var / M;
 }
 
 // ---- per-frame standardisation and fusion: one CTA per frame ---------------------------------------------------
@@ -352,20 +373,15 @@ __global__ void __launch_bounds__(1024) select_fuse_kernel(const SelectParams p)
         if (p.mask & HIPPO_SCORE_ATTN) x[0] = (double)p.attn_mass[j];
         if (p.mask & HIPPO_SCORE_SPA) x[1] = p.s_spa[j];
         if (p.mask & HIPPO_SCORE_TEMP) {
-            double sum = 0.0;
-            int cnt = 0;
-            const double nj = p.norm2[j];
-            if (f > 0) {  // previous frame always holds every cell
-                const double nk = p.norm2[j - p.tpf];
-                sum += (nj > 0.0 && nk > 0.0) ? p.tdot[j - p.tpf] / (sqrt(nj) * sqrt(nk)) : 0.0;
-                ++cnt;
+            // the previous frame always holds every cell
+            const bool back = f > 0, on = f + 1 < n_frames && c < min(p.tpf, n_v - (f + 1) * p.tpf);
+            double cb = back ? p.tdot[j - p.tpf] : 0.0, co = on ? p.tdot[j] : 0.0;
+            if (!p.cosines) {
+                const double nj = p.norm2[j], nb = back ? p.norm2[j - p.tpf] : 0.0, no = on ? p.norm2[j + p.tpf] : 0.0;
+                cb = nj > 0.0 && nb > 0.0 ? cb / (sqrt(nj) * sqrt(nb)) : 0.0;
+                co = nj > 0.0 && no > 0.0 ? co / (sqrt(nj) * sqrt(no)) : 0.0;
             }
-            if (f + 1 < n_frames && c < min(p.tpf, n_v - (f + 1) * p.tpf)) {
-                const double nk = p.norm2[j + p.tpf];
-                sum += (nj > 0.0 && nk > 0.0) ? p.tdot[j] / (sqrt(nj) * sqrt(nk)) : 0.0;
-                ++cnt;
-            }
-            x[2] = 1.0 - (cnt ? sum / cnt : 0.0);
+            x[2] = 1.0 - (back && on ? 0.5 * (cb + co) : cb + co);
         }
     }
     double mu[3] = {x[0], x[1], x[2]}, dv[3], var[3];
@@ -397,9 +413,10 @@ __device__ __forceinline__ uint32_t order_key(float x) {  // larger float -> lar
 // A sequence's keys are dealt to the CTAs of a cluster in contiguous shares, to a CTA's threads in groups of eight neighbours
 // (a share of more than one round is read again per pass).  The key T of the k-th largest element comes from three histogram
 // passes over its digits (11, 11 and 10 bits, top first): every CTA counts its own keys that agree with T so far, reads the
-// others' counts through distributed shared memory and finds the digit by a scan of its own.  Then one scan of the pairs
-// (keys > T, keys == T) gives every thread its first output position: the kept ones among the equal are those with the lowest
-// indices, so position = (larger ones before) + min(equal ones before, equal ones to keep).
+// others' counts through distributed shared memory and finds the digit by a scan of its own, which also adds up what the
+// shares in front of its own hold above the digit and on it.  Then one scan of the pairs (keys > T, keys == T) gives every thread its
+// first output position: the kept ones among the equal are those with the lowest indices, so position = (larger ones before) +
+// min(equal ones before, equal ones to keep).
 // Bound: latency (three passes of count, exchange, scan).  65,536 tokens 20 us, 160 us with one CTA and two bits per step (three
 // block barriers each, keys beyond 32 per thread in shared memory); 28 us with the remote counts loaded one after the other.
 constexpr int kTopThreads = 1024, kTopPerThread = 8, kTopTile = kTopThreads * kTopPerThread, kTopBins = 2048;
@@ -411,13 +428,14 @@ __global__ void __launch_bounds__(kTopThreads, 1) select_topk_kernel(const Selec
     __shared__ uint32_t hist1[kTopBins], hist2[kTopBins / 2];
     uint32_t *hist0 = copies;
     __shared__ uint32_t wsum[32], s_digit, s_above;
-    __shared__ unsigned long long w64[32];
-    __shared__ unsigned long long share_total;   // this CTA's (keys > T) << 32 | (keys == T)
+    __shared__ uint32_t wlow[32];
+    __shared__ unsigned long long w64[32], s_lower;
     const int b = blockIdx.x / cluster, rank = blockIdx.x % cluster, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = p.seq_off[b + 1] - p.seq_off[b], k = p.k[b];
     for (int i = tid; i < kTopBins; i += kTopThreads) { reinterpret_cast<uint4 *>(hist0)[i] = make_uint4(0, 0, 0, 0); hist1[i] = 0; }
     hist2[tid] = 0;
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const float *score = p.fused + p.seq_off[b];
     int32_t *out = p.kept + p.k_off[b];
     if (k <= 0) return;                           // the same for the whole cluster
@@ -435,6 +453,7 @@ __global__ void __launch_bounds__(kTopThreads, 1) select_topk_kernel(const Selec
     load(0);
     __syncthreads();
     uint32_t T = 0, mask = 0;
+    unsigned long long base = 0;                  // (larger than T) << 32 | (equal to T) in the shares in front of this CTA's
     int need = k;                                 // the wanted element is the need-th largest among the keys that agree with T so far
     auto find_digit = [&](auto pass_tag) {
         constexpr int pass = decltype(pass_tag)::value, shift = pass == 0 ? 21 : pass == 1 ? 10 : 0;
@@ -458,7 +477,7 @@ __global__ void __launch_bounds__(kTopThreads, 1) select_topk_kernel(const Selec
         if (cluster > 1) cluster_sync_all(); else __syncthreads();
         // counts over the cluster and their sums from the top: thread t owns the bins 2 t, 2 t + 1 counted from the top
         constexpr int kBins = pass == 2 ? kTopBins / 2 : kTopBins;
-        uint32_t c[2], w[2][7];
+        uint32_t c[2], low[2] = {0, 0}, w[2][7];   // low: in the shares in front of this CTA's
 #pragma unroll
         for (int h = 0; h < 2; ++h) {             // every remote load is in flight before the first is used
             const int bin = kBins - 1 - (2 * tid + h);
@@ -473,77 +492,69 @@ __global__ void __launch_bounds__(kTopThreads, 1) select_topk_kernel(const Selec
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int q = 0; q < 7; ++q) c[h] += w[h][q];
-        uint32_t inc = c[0] + c[1];
+            for (int q = 0; q < 7; ++q) {
+                c[h] += w[h][q];
+                low[h] += (rank ^ (q + 1)) < rank ? w[h][q] : 0u;
+            }
+        // keys in higher bins, of all shares and (in a cluster) of those in front
+        auto scan = [&](uint32_t mine, uint32_t *sums) {
+            uint32_t inc = mine;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += v; }
-        if (lane == 31) wsum[warp] = inc;
+            for (int o = 1; o < 32; o <<= 1) { const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += v; }
+            if (lane == 31) sums[warp] = inc;
+            return inc - mine;
+        };
+        auto in_front = [&](const uint32_t *sums) { return __reduce_add_sync(0xffffffffu, lane < warp ? sums[lane] : 0u); };
+        uint32_t before = scan(c[0] + c[1], wsum), lower = cluster > 1 ? scan(low[0] + low[1], wlow) : 0u;
         __syncthreads();
-        if (warp == 0) {
-            uint32_t v = wsum[lane];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) { const uint32_t w = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += w; }
-            wsum[lane] = v;
-        }
-        __syncthreads();
-        uint32_t before = (warp ? wsum[warp - 1] : 0u) + inc - c[0] - c[1];      // keys in higher bins
+        before += in_front(wsum);
+        if (cluster > 1) lower += in_front(wlow);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            if (before < (uint32_t)need && (uint32_t)need <= before + c[h]) { s_digit = (uint32_t)(kBins - 1 - (2 * tid + h)); s_above = before; }
+            if (before < (uint32_t)need && (uint32_t)need <= before + c[h]) {
+                s_digit = (uint32_t)(kBins - 1 - (2 * tid + h));
+                s_above = before;
+                s_lower = (unsigned long long)lower << 32 | low[h];
+            }
             before += c[h];
+            lower += low[h];
         }
         __syncthreads();
         T |= s_digit << shift;
         mask |= digits << shift;
         need -= (int)s_above;                     // after the last pass: elements equal to T to keep
+        // what the shares in front of this one have above the digit, and, should it be the last one, on it
+        base = (base & 0xffffffff00000000ull) + s_lower;
     };
     find_digit(std::integral_constant<int, 0>{});
     find_digit(std::integral_constant<int, 1>{});
     find_digit(std::integral_constant<int, 2>{});
-    unsigned long long base = 0;                  // (larger, equal) in front of this CTA's share
-    for (int ph = cluster > 1 ? 0 : 1; ph < 2; ++ph) {
-        // first the share's totals (only where there are other shares), then the output
-        unsigned long long run = ph ? base : 0;
-        for (int r = 0; r < rounds; ++r) {
-            if (rounds > 1) load(r);
-            unsigned long long mine = 0;
+    unsigned long long run = base;
+    for (int r = 0; r < rounds; ++r) {
+        if (rounds > 1) load(r);
+        unsigned long long mine = 0;
 #pragma unroll
-            for (int e = 0; e < kTopPerThread; ++e)
-                if (live(r, e)) mine += key[e] > T ? 1ull << 32 : key[e] == T ? 1ull : 0ull;
-            unsigned long long inc = mine;
+        for (int e = 0; e < kTopPerThread; ++e)
+            if (live(r, e)) mine += key[e] > T ? 1ull << 32 : key[e] == T ? 1ull : 0ull;
+        unsigned long long inc = mine;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) { const unsigned long long v = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += v; }
-            __syncthreads();                      // w64 of the round before has been read
-            if (lane == 31) w64[warp] = inc;
-            __syncthreads();
-            unsigned long long sums = w64[lane];
+        for (int o = 1; o < 32; o <<= 1) { const unsigned long long v = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += v; }
+        __syncthreads();                          // w64 of the round before has been read
+        if (lane == 31) w64[warp] = inc;
+        __syncthreads();
+        unsigned long long sums = w64[lane];
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) { const unsigned long long v = __shfl_up_sync(0xffffffffu, sums, o); if (lane >= o) sums += v; }
-            const unsigned long long in_front = __shfl_sync(0xffffffffu, sums, warp ? warp - 1 : 0);
-            const unsigned long long at = run + (warp ? in_front : 0ull) + inc - mine;
-            run += __shfl_sync(0xffffffffu, sums, 31);
-            if (ph) {
-                uint32_t gt = (uint32_t)(at >> 32), eq = (uint32_t)at;
+        for (int o = 1; o < 32; o <<= 1) { const unsigned long long v = __shfl_up_sync(0xffffffffu, sums, o); if (lane >= o) sums += v; }
+        const unsigned long long in_front = __shfl_sync(0xffffffffu, sums, warp ? warp - 1 : 0);
+        const unsigned long long at = run + (warp ? in_front : 0ull) + inc - mine;
+        run += __shfl_sync(0xffffffffu, sums, 31);
+        uint32_t gt = (uint32_t)(at >> 32), eq = (uint32_t)at;
 #pragma unroll
-                for (int e = 0; e < kTopPerThread; ++e) {
-                    if (!live(r, e)) continue;
-                    const bool g = key[e] > T, q = key[e] == T;
-                    if (g || (q && eq < (uint32_t)need)) out[gt + min(eq, (uint32_t)need)] = begin + r * kTopTile + tid * kTopPerThread + e;
-                    gt += g; eq += q;
-                }
-            }
-        }
-        if (!ph) {
-            if (tid == 0) share_total = run;
-            cluster_sync_all();
-            unsigned long long v[7];
-#pragma unroll
-            for (int q = 0; q < 7; ++q) {
-                v[q] = 0;
-                if (q < rank) asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v[q]) : "r"(cluster_map(smem_u32(&share_total), (uint32_t)q)) : "memory");
-            }
-#pragma unroll
-            for (int q = 0; q < 7; ++q) base += v[q];
+        for (int e = 0; e < kTopPerThread; ++e) {
+            if (!live(r, e)) continue;
+            const bool g = key[e] > T, q = key[e] == T;
+            if (g || (q && eq < (uint32_t)need)) out[gt + min(eq, (uint32_t)need)] = begin + r * kTopTile + tid * kTopPerThread + e;
+            gt += g; eq += q;
         }
     }
     if (cluster > 1) cluster_sync_all();          // nobody leaves while its shared memory may be read
@@ -626,7 +637,7 @@ __global__ void select_copy_keys_kernel(const float *keys, float *fused, int n) 
 
 // A kernel that begins with griddepcontrol.wait: its launch overlaps the end of its predecessor in the stream.
 template <typename... Args>
-static cudaError_t launch_dependent(void (*kernel)(Args...), int grid, int threads, int cluster, cudaStream_t s, Args... args) {
+static cudaError_t launch_dependent(void (*kernel)(Args...), long long grid, int threads, int cluster, size_t smem, cudaStream_t s, Args... args) {
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -637,6 +648,7 @@ static cudaError_t launch_dependent(void (*kernel)(Args...), int grid, int threa
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = cluster > 1 ? 2 : 1;
@@ -774,32 +786,34 @@ int32_t hippo_select_tokens_policy(int32_t batch, const int32_t *n_visual, int32
         const double chain_us = area > 1 ? 1e-3 * ns_per_dim[(area + 6) / 8] * embed_dim : 0.0, rate_us = 2.2e-6 * tok * embed_dim;
         gram = tiles_us < 10.0 + (chain_us > rate_us ? chain_us + 0.5 * rate_us : rate_us + 0.5 * chain_us);
     }
+    p.cosines = need_emb && gram ? 1 : 0;
     if (need_emb && gram) {
         const int32_t rc = launch_select_gram(p, (WsHeader *)workspace, s);
         if (rc != HIPPO_OK) return rc;
     } else if (need_emb) {
-        const int warps = 8;
-        dim3 g1((unsigned)((tok + warps - 1) / warps));
-        if (dtype == HIPPO_DTYPE_FP32) select_dots_kernel<float><<<g1, warps * 32, 0, s>>>(p);
-        else select_dots_kernel<__nv_bfloat16><<<g1, warps * 32, 0, s>>>(p);
-        count_launches(1);
-    }
-    if (scored && (score_mask & HIPPO_SCORE_SPA) && !gram) {
-        dim3 g2((unsigned)(frames * p.crops_y * p.crops_x));
-        static PerDeviceOnce spa_attr;
-        int dev;
-        if (spa_attr.needed(dev)) {
-            HIPPO_CUDA_TRY(cudaFuncSetAttribute(select_spatial_mma_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MmaShape<float>::kSmemBytes));
-            HIPPO_CUDA_TRY(cudaFuncSetAttribute(select_spatial_mma_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MmaShape<__nv_bfloat16>::kSmemBytes));
-            spa_attr.mark(dev);
+        // norms and next-frame products, and in front of them the crops where the mask has the spatial term
+        const bool spa = (score_mask & HIPPO_SCORE_SPA) != 0, fp32 = dtype == HIPPO_DTYPE_FP32;
+        const int dots = ceil_div((int)tok, kDotsThreads / 32);
+        if (spa) {
+            static PerDeviceOnce spa_attr;
+            int dev;
+            if (spa_attr.needed(dev)) {
+                HIPPO_CUDA_TRY(cudaFuncSetAttribute(select_spatial_mma_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MmaShape<float>::kSmemBytes));
+                HIPPO_CUDA_TRY(cudaFuncSetAttribute(select_spatial_mma_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MmaShape<__nv_bfloat16>::kSmemBytes));
+                spa_attr.mark(dev);
+            }
+            const long long grid = frames * p.crops_y * p.crops_x + dots;
+            HIPPO_CUDA_TRY(fp32 ? launch_dependent(select_spatial_mma_kernel<float>, grid, kMmaThreads, 1, MmaShape<float>::kSmemBytes, s, p)
+                                : launch_dependent(select_spatial_mma_kernel<__nv_bfloat16>, grid, kMmaThreads, 1, MmaShape<__nv_bfloat16>::kSmemBytes, s, p));
+        } else {
+            HIPPO_CUDA_TRY(fp32 ? launch_dependent(select_dots_kernel<float>, dots, kDotsThreads, 1, 0, s, p)
+                                : launch_dependent(select_dots_kernel<__nv_bfloat16>, dots, kDotsThreads, 1, 0, s, p));
         }
-        if (dtype == HIPPO_DTYPE_FP32) select_spatial_mma_kernel<float><<<g2, kMmaThreads, MmaShape<float>::kSmemBytes, s>>>(p);
-        else select_spatial_mma_kernel<__nv_bfloat16><<<g2, kMmaThreads, MmaShape<__nv_bfloat16>::kSmemBytes, s>>>(p);
         count_launches(1);
     }
     const int fuse_threads = ((p.tpf + 31) / 32) * 32;
     if (scored) {
-        HIPPO_CUDA_TRY(launch_dependent(select_fuse_kernel, (int)frames, fuse_threads, 1, s, p));
+        HIPPO_CUDA_TRY(launch_dependent(select_fuse_kernel, frames, fuse_threads, 1, 0, s, p));
         count_launches(1);
     }
     if (ksum > 0 && policy == HIPPO_SELECT_UNIFORM_PER_FRAME) {
@@ -812,7 +826,7 @@ int32_t hippo_select_tokens_policy(int32_t batch, const int32_t *n_visual, int32
         for (int b = 0; b < batch; ++b) longest = n_visual[b] > longest ? n_visual[b] : longest;
         int cluster = 1;
         while (cluster < 8 && longest > cluster * kTopTile / 2) cluster *= 2;
-        HIPPO_CUDA_TRY(launch_dependent(select_topk_kernel, batch * cluster, kTopThreads, cluster, s, p, cluster));
+        HIPPO_CUDA_TRY(launch_dependent(select_topk_kernel, batch * cluster, kTopThreads, cluster, 0, s, p, cluster));
         count_launches(1);
     }
     HIPPO_CUDA_TRY(cudaGetLastError());

@@ -14,7 +14,8 @@ struct SelectParams {
     const float *attn_mass;
     float *fused;
     int32_t *kept;
-    double *norm2, *tdot, *s_spa;   // [total tokens]: squared norm, product with the next frame's (integer path: 1 or 0, the cosine), Eq. 5-6
+    double *norm2, *tdot, *s_spa;   // [total tokens]: squared norm, product with the next frame's, Eq. 5-6
+    int cosines;                    // 1: tdot holds the cosine itself (the integer path), norm2 nothing
     int batch, grid_h, grid_w, crop_h, crop_w, d, tpf, crops_y, crops_x;
     unsigned mask;
     int seq_off[kSelMaxBatch + 1];    // token offset of each sequence

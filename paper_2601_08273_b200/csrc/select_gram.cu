@@ -711,7 +711,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) select_gram_kernel(const Sele
     if (gp.part == 2 && gp.splits == 1) asm volatile("griddepcontrol.wait;" ::: "memory");
     const int own_rows = (own_end - f0) * m;
     if (!good) {                                                      // a wait gave up: scores that cannot be taken for any
-        if (tid < own_rows && sh->token[tid] >= 0) p.s_spa[sh->token[tid]] = p.norm2[sh->token[tid]] = p.tdot[sh->token[tid]] = __longlong_as_double(0x7ff8000000000000ll);
+        if (tid < own_rows && sh->token[tid] >= 0) p.s_spa[sh->token[tid]] = p.tdot[sh->token[tid]] = __longlong_as_double(0x7ff8000000000000ll);
         return;
     }
     __syncthreads();
@@ -723,12 +723,11 @@ __global__ void __launch_bounds__(kGramThreads, 1) select_gram_kernel(const Sele
     }
     __syncthreads();
     if (tid < own_rows && sh->token[tid] >= 0) {
-        // The fusion gets the cosine with the next frame itself, and a norm of 1 or 0 with it.  All three sums of a cosine are then this
+        // The fusion gets the cosine with the next frame itself.  All three sums of a cosine are then this
         // tile's: another tile may have added up other parts of the dimensions, and where frames are equal (a cosine of 1, a variance
         // of 0) the difference of their roundings would be standardised to scores of several sigma.
         const int tk = sh->token[tid], nx = tid + m;
         const double in = sh->inv_root[tid], ix = nx < kGramRows && sh->token[nx] >= 0 ? sh->inv_root[nx] : -1.0;
-        p.norm2[tk] = in >= 0.0 ? 1.0 : 0.0;
         if (nx < kGramRows && sh->token[nx] >= 0) p.tdot[tk] = in >= 0.0 && ix >= 0.0 ? (t_next[tid] + t_prev[nx]) * (in * ix) : 0.0;
     }
     for (int i = tid; i < kGramRows * kMaxCrop; i += kGramThreads) {
