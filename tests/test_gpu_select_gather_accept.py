@@ -402,6 +402,20 @@ def test_topk_sizes_and_ties(hb, lens):
                 at += k
 
 
+@pytest.mark.parametrize("lens", [[255], [256], [257], [256, 5000, 31, 33], [4096, 256]])
+def test_topk_by_counting(hb, lens):
+    """Up to 256 keys are ranked by counting, alone and beside sequences whose digits a cluster looks for; few different keys."""
+    rng = np.random.default_rng(sum(lens))
+    for values in (3, 200):
+        keys = [(rng.integers(0, values, n) / values - 0.5).astype(np.float32) for n in lens]
+        for ks in ([1] * len(lens), [n // 2 for n in lens], list(lens)):
+            kept, _ = hb.hippo_select_tokens(None, None, lens, ks, 8, 8, policy=hb.HIPPO_SELECT_RANDOM, random_keys=dev(np.concatenate(keys)))
+            got, at = host(kept), 0
+            for x, k in zip(keys, ks):
+                np.testing.assert_array_equal(got[at:at + k], np.sort(np.argsort(-x, kind="stable")[:k]))
+                at += k
+
+
 def test_select_random_and_frames_need_no_embeddings(hb):
     cfg = W.CONFIGS[2]
     n, tpf = W.visual_lengths(cfg)[0], cfg.tokens_per_frame
@@ -657,3 +671,23 @@ def test_a_vocabulary_chunk_of_nan_stays_out_of_its_rows_sum(hb, batch):
             res.append((host(n).tolist(), host(out).tolist()))
     assert all(r == res[-1] for r in res)
     assert max(res[-1][0]) >= 2                          # the row with the NaN was tested and passed somewhere
+
+
+@pytest.mark.parametrize("batch,vocab", [(1, 1), (1, 1023), (1, 1024), (1, 1025), (1, 4097), (2, 5000), (1, 152063), (2, 152065)])
+@pytest.mark.parametrize("eps", [0.0, 0.5])
+def test_accept_pieces_of_a_quarter_chunk(hb, batch, vocab, eps):
+    """Few sequences: the weights go to pieces of 1,024 tokens.  Token ids and counts equal the oracle's."""
+    check_accept(hb, W.accept_inputs(W.CONFIGS[0], batch=batch, gamma=5, vocab=vocab, corr_eps=eps), "V=%d" % vocab)
+
+
+@pytest.mark.parametrize("offset", [0, 1e6, 3e10])
+def test_accept_logits_far_below_the_maximum(hb, offset):
+    """Exponentials from 1 down to below the smallest double, and their sum: the tail of one row lies 0 to 800 below its maximum; masked
+    entries (-inf); logits so large that their neighbours are 1,000 apart."""
+    inp = W.accept_inputs(W.CONFIGS[0], batch=2, gamma=3, vocab=9000, corr_eps=0.3)
+    for x in (inp["target_logits"], inp["draft_logits"]):
+        x[:, 1] = x[:, 1].max(axis=-1, keepdims=True) - np.linspace(0, 800, 9000, dtype=np.float32)
+        x[:, 2, 100::3] = -np.inf
+        x += np.float32(offset)
+    inp["draft_tokens"][:, 1:] = 99
+    check_accept(hb, inp, "far below")
