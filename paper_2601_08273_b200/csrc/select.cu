@@ -419,6 +419,7 @@ __device__ __forceinline__ uint32_t order_key(float x) {  // larger float -> lar
 // min(equal ones before, equal ones to keep).
 // Bound: latency (three passes of count, exchange, scan).  65,536 tokens 20 us, 160 us with one CTA and two bits per step (three
 // block barriers each, keys beyond 32 per thread in shared memory); 28 us with the remote counts loaded one after the other.
+constexpr int kTopByRank = 256;     // keys that are ranked by counting
 constexpr int kTopThreads = 1024, kTopPerThread = 8, kTopTile = kTopThreads * kTopPerThread, kTopBins = 2048;
 
 __global__ void __launch_bounds__(kTopThreads, 1) select_topk_kernel(const SelectParams p, const int cluster) {
@@ -439,6 +440,30 @@ __global__ void __launch_bounds__(kTopThreads, 1) select_topk_kernel(const Selec
     const float *score = p.fused + p.seq_off[b];
     int32_t *out = p.kept + p.k_off[b];
     if (k <= 0) return;                           // the same for the whole cluster
+    if (n <= kTopByRank) {
+        // A key's rank is the number of better ones; several threads per key look at every kParts-th of the others.  Two barriers where
+        // the digits take a dozen.
+        if (rank > 0) return;
+        constexpr int kParts = kTopThreads / kTopByRank;
+        uint32_t *keys = hist2, *kept = hist1;
+        if (tid < n) keys[tid] = order_key(score[tid]);
+        __syncthreads();
+        const int i = tid / kParts;
+        const uint32_t mine = i < n ? keys[i] : 0u;
+        int better = 0, j = tid % kParts;
+        for (; j < min(i, n); j += kParts) better += keys[j] >= mine ? 1 : 0;           // an equal key in front is better
+        if (j == i) j += kParts;
+        for (; j < n; j += kParts) better += keys[j] > mine ? 1 : 0;
+#pragma unroll
+        for (int o = 1; o < kParts; o <<= 1) better += __shfl_xor_sync(0xffffffffu, better, o);
+        const bool keep = i < n && better < k;
+        const unsigned bits = __ballot_sync(0xffffffffu, keep && tid % kParts == 0);
+        if (lane == 0) kept[warp] = __popc(bits);
+        __syncthreads();
+        const int before = (int)__reduce_add_sync(0xffffffffu, lane < warp ? kept[lane] : 0u) + __popc(bits & ((1u << lane) - 1));
+        if (keep && tid % kParts == 0) out[before] = i;
+        return;
+    }
     const int begin = (int)((long long)n * rank / cluster), end = (int)((long long)n * (rank + 1) / cluster);
     const int rounds = (end - begin + kTopTile - 1) / kTopTile;
     uint32_t key[kTopPerThread];
