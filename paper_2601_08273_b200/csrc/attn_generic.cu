@@ -41,8 +41,24 @@ __global__ void __launch_bounds__(kGenThreads) attn_generic_kernel(const AttnPar
     float *ms = Ps + (size_t)R * tile_keys, *ls = ms + R, *fs = ls + R;
     const int split = blockIdx.x, hk = blockIdx.y, b = blockIdx.z;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int n_splits = cluster ? cluster : p.num_splits;      // split s takes the tiles s, s + n_splits, ...
+    const int D4 = D / 4;
+    const T *kp = (const T *)p.k_pages, *vp = (const T *)p.v_pages;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // An identity-mapped cache is addressable up to max_kv_len: the first tile need not wait for the length.
+    constexpr int kEarly = 2;
+    float4 k_early[kEarly], v_early[kEarly];
+    const bool early = !p.page_table && tile_keys * D4 <= kEarly * kGenThreads && split * tile_keys < p.max_kv_len;
+    if (early) {
+        const int tok0 = split * tile_keys;
+        const size_t base = (((size_t)(b * p.max_pages_per_seq + tok0 / kPageSize) * p.n_kv_heads + hk) * kPageSize + tok0 % kPageSize) * D;
+#pragma unroll
+        for (int e = 0; e < kEarly; ++e) {
+            const int i = tid + e * kGenThreads;
+            if (i < tile_keys * D4) { k_early[e] = load_kv4(kp + base + (size_t)i * 4); v_early[e] = load_kv4(vp + base + (size_t)i * 4); }
+        }
+    }
     const int kvl = p.kv_len ? p.kv_len[b] : p.max_kv_len;
     const bool skipped = kvl < p.q_len;                     // zeros; the combine kernel writes them where there is one
     if (skipped && !cluster) return;
@@ -55,23 +71,27 @@ __global__ void __launch_bounds__(kGenThreads) attn_generic_kernel(const AttnPar
     }
     for (int r = tid; r < R; r += kGenThreads) { ms[r] = -INFINITY; ls[r] = 0.f; }
 
-    const int n_splits = cluster ? cluster : p.num_splits;
     const int n_tiles = skipped ? 0 : (kvl + tile_keys - 1) / tile_keys;
-    const int per = (n_tiles + n_splits - 1) / n_splits;
-    const int t0 = split * per, t1 = min(n_tiles, t0 + per);
-    const T *kp = (const T *)p.k_pages, *vp = (const T *)p.v_pages;
-    const int D4 = D / 4;
 
-    for (int tile = t0; tile < t1; ++tile) {
+    for (int tile = split; tile < n_tiles; tile += n_splits) {
         const int tok0 = tile * tile_keys;
-        const int pid = page_of(p.page_table, p.max_pages_per_seq, b, tok0 / kPageSize);
-        const size_t base = (((size_t)pid * p.n_kv_heads + hk) * kPageSize + (tok0 % kPageSize)) * D;
-        for (int i = tid; i < tile_keys * D4; i += kGenThreads) {
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        auto stage = [&](int i, auto k_of, auto v_of) {
             const int j = i / D4, d = (i % D4) * 4;
             const bool ok = tok0 + j < kvl;
-            const float4 z = make_float4(0.f, 0.f, 0.f, 0.f), k = ok ? load_kv4(kp + base + (size_t)j * D + d) : z, v = ok ? load_kv4(vp + base + (size_t)j * D + d) : z;
+            const float4 k = ok ? k_of() : z, v = ok ? v_of() : z;
             *reinterpret_cast<float4 *>(Ks + j * KS + d) = k;
             *reinterpret_cast<float4 *>(Vs + j * KS + d) = v;
+        };
+        if (early && tile == split) {
+#pragma unroll
+            for (int e = 0; e < kEarly; ++e)
+                if (tid + e * kGenThreads < tile_keys * D4) stage(tid + e * kGenThreads, [&] { return k_early[e]; }, [&] { return v_early[e]; });
+        } else {
+            const int pid = page_of(p.page_table, p.max_pages_per_seq, b, tok0 / kPageSize);
+            const size_t base = (((size_t)pid * p.n_kv_heads + hk) * kPageSize + (tok0 % kPageSize)) * D;
+            for (int i = tid; i < tile_keys * D4; i += kGenThreads)
+                stage(i, [&] { return load_kv4(kp + base + (size_t)i * 4); }, [&] { return load_kv4(vp + base + (size_t)i * 4); });
         }
         __syncthreads();
         // ---- scores
