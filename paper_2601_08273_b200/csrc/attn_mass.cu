@@ -36,10 +36,10 @@ constexpr int kMassSlices = 4;            // column slices of an accumulator til
 constexpr int kMassSliceCols = 32;
 constexpr int kMassConsumers = 128 * kMassSlices;
 constexpr int kMassThreads = 64 + kMassConsumers;
-constexpr int kMassSlots = 3;            // ring of streamed tiles
+constexpr int kMassSlots = 4;            // ring of streamed tiles
+constexpr int kMassAcc = 4;              // accumulator tiles that tensor memory holds
 constexpr int kMassTile = 128;           // rows and keys per accumulator tile
 constexpr int kMassMaxBatch = 64;        // per-sequence lengths travel in the kernel parameters
-constexpr int kMassMaxSplits = 64;
 constexpr int kMassMaxRows = 3072;       // l_txt * group: the pass-2 table of a KV head lives in shared memory
 constexpr float kMassLog2e = 1.4426950408889634f;
 constexpr unsigned long long kMassWaitLimitNs = 2000000000ull;
@@ -50,8 +50,9 @@ struct MassParams {
     int rows_per_block;    // T * G
     int n_row_blocks;      // ceil(l_txt / T)
     int r_tot;             // l_txt * G packed rows per KV head
-    int splits;            // key splits of this launch
-    int stat_splits;       // key splits of pass 1 (layout of `stats`)
+    int grid;              // CTAs of this launch (tensor-core path)
+    int stat_grid;         // CTAs of pass 1
+    int stat_slots;        // partial results that a row block can have from pass 1 (layout of `stats`)
     int sum_nv;            // total visual tokens
     int max_pages_per_seq;
     float sl2;             // softmax scale * log2(e)
@@ -60,7 +61,7 @@ struct MassParams {
     const int32_t *page_table;
     const void *q;
     const void *k_pages;
-    float2 *stats;         // [batch * n_kv_heads][stat_splits][r_tot]: (max in the log2 domain, sum of 2^(x - max))
+    float2 *stats;         // [batch * n_kv_heads][stat_slots][r_tot]: (max in the log2 domain, sum of 2^(x - max))
     float2 *table;         // CUDA-core path: [batch * n_kv_heads][r_tot] (-max, 1 / sum), natural-log domain
     float *table_log2;     // tensor-core path, same memory: [batch * n_kv_heads][r_tot] -(max + log2 sum), log2 domain
     float *colsum;         // [n_kv_heads][sum_nv]
@@ -68,10 +69,62 @@ struct MassParams {
     WsHeader *header;
     int n_visual[kMassMaxBatch];
     int offset[kMassMaxBatch];   // first token of each sequence in the concatenated mass array
+    int tile_off[kMassMaxBatch + 1];   // key tiles of the sequences before this one
 };
 
+// The work of both passes is one flat list, cut into equal ranges for the CTAs of one wave whatever sequence, head or row block
+// they end in.  Pass 1: (sequence, KV head, row block, key tile); pass 2: (sequence, KV head, key tile).  Before, every (head, row block)
+// was split into the same number of key ranges, 64 x 4 of them for 296 places and 8 x 18 for 148 (32,768 tokens, 32 heads, 256 text rows:
+// 216 us, 210 with the flat list).
+struct MassRange {
+    long long total;
+    int grid;
+    __host__ __device__ long long start(int c) const { return total * c / grid; }
+    __host__ __device__ int cta_of(long long t) const { return (int)(((t + 1) * grid - 1) / total); }   // whose range t is in
+};
+struct MassCursor {
+    int b, hk, rb, kt, n_kt;     // sequence, KV head, row block (pass 1), key tile, the sequence's key tiles
+};
+template <int PASS>              // 0: pass 1, 1: pass 2
+__device__ __forceinline__ MassCursor mass_locate(const MassParams &p, long long t) {
+    const int per = p.n_kv_heads * (PASS == 0 ? p.n_row_blocks : 1);
+    MassCursor c;
+    c.b = 0;
+    while (c.b + 1 < p.batch && (long long)p.tile_off[c.b + 1] * per <= t) ++c.b;
+    c.n_kt = p.tile_off[c.b + 1] - p.tile_off[c.b];
+    const long long in = t - (long long)p.tile_off[c.b] * per;
+    const int row = (int)(in / c.n_kt);
+    c.kt = (int)(in % c.n_kt);
+    c.hk = PASS == 0 ? row / p.n_row_blocks : row;
+    c.rb = PASS == 0 ? row % p.n_row_blocks : 0;
+    return c;
+}
+// A resident tile and what is streamed past it.  Pass 1: a row block, up to `left` key tiles; pass 2: a key tile, all row blocks.
+// Returns how many entries of the flat list that is.
+template <int PASS>
+__device__ __forceinline__ int mass_segment(const MassParams &p, const MassCursor &c, long long left, int &i0, int &i1) {
+    if (PASS == 1) { i0 = 0; i1 = p.n_row_blocks; return 1; }
+    const int n = (int)(left < c.n_kt - c.kt ? left : c.n_kt - c.kt);
+    i0 = c.kt;
+    i1 = c.kt + n;
+    return n;
+}
+// On by n entries; at the end of a row (pass 1: row block, pass 2: head) to the next one, past sequences without keys.
+template <int PASS>
+__device__ __forceinline__ void mass_advance(const MassParams &p, MassCursor &c, int n) {
+    c.kt += n;
+    if (c.kt < c.n_kt) return;
+    c.kt = 0;
+    if (PASS == 0 && ++c.rb < p.n_row_blocks) return;
+    c.rb = 0;
+    if (++c.hk < p.n_kv_heads) return;
+    c.hk = 0;
+    do ++c.b; while (c.b < p.batch && p.tile_off[c.b + 1] == p.tile_off[c.b]);
+    c.n_kt = c.b < p.batch ? p.tile_off[c.b + 1] - p.tile_off[c.b] : 1;
+}
+
 struct MassShared {
-    unsigned long long full[kMassSlots], empty[kMassSlots], res_full[2], res_free[2], s_full[2], s_free[2], drain;
+    unsigned long long full[kMassSlots], empty[kMassSlots], res_full[2], res_free[2], s_full[kMassAcc], s_free[kMassAcc], drain;
     long long wait_limit;   // the header's wait limit (0: the built-in one), read once
     uint32_t tmem_base;
     volatile int abort;
@@ -111,6 +164,7 @@ template <int PASS> struct MassBuffers {
     static constexpr int kRes = PASS == 0 ? 1 : 2;
     static constexpr int kSlots = PASS == 0 ? 2 : kMassSlots;
     static constexpr int kCtasPerSm = PASS == 0 ? 2 : 1;
+    static constexpr int kAcc = kMassAcc / kCtasPerSm;       // consumer warps may drift apart by that many tiles
 };
 
 template <int D, int PASS>
@@ -120,7 +174,7 @@ mass_tc_kernel(const MassParams p, const __grid_constant__ CUtensorMap k_map, co
     constexpr int kChunkBytes = kMassTile * 128;          // one chunk of a 128-row tile
     constexpr int kTileBytes = kChunks * kChunkBytes;
     constexpr int kPageChunkBytes = kPageSize * 128;      // one chunk of one page
-    constexpr int kRes = MassBuffers<PASS>::kRes, kSlots = MassBuffers<PASS>::kSlots;
+    constexpr int kRes = MassBuffers<PASS>::kRes, kSlots = MassBuffers<PASS>::kSlots, kAcc = MassBuffers<PASS>::kAcc;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t *res = base;                                  // [2] resident tiles: [chunk][128 rows][128 B], 128-byte swizzle
@@ -132,48 +186,37 @@ mass_tc_kernel(const MassParams p, const __grid_constant__ CUtensorMap k_map, co
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int G = p.group, Hkv = p.n_kv_heads, T = p.t_per_block, TG = p.rows_per_block;
-    int bid = blockIdx.x;
-    const int split = bid % p.splits; bid /= p.splits;
-    int rb = 0;
-    if (PASS == 0) { rb = bid % p.n_row_blocks; bid /= p.n_row_blocks; }
-    const int hk = bid % Hkv, b = bid / Hkv;
-    const int unit = b * Hkv + hk;
-    const int nv = p.n_visual[b];
-    const int nkt = (nv + kMassTile - 1) / kMassTile;
-    const int kt0 = (int)((long long)split * nkt / p.splits), kt1 = (int)((long long)(split + 1) * nkt / p.splits);
     // outer loop: resident tiles; inner loop: streamed tiles
-    const int o0 = PASS == 0 ? rb : kt0, o1 = PASS == 0 ? rb + 1 : kt1;
-    const int i0 = PASS == 0 ? kt0 : 0, i1 = PASS == 0 ? kt1 : p.n_row_blocks;
-
-    if (o1 <= o0 || i1 <= i0) {
-        // nothing to stream: a pass-0 CTA still owes its rows an empty partial
-        if (PASS == 0 && tid < TG && rb * TG + tid < p.r_tot)
-            p.stats[((size_t)unit * p.stat_splits + split) * p.r_tot + rb * TG + tid] = make_float2(-INFINITY, 0.f);
-        return;
-    }
+    const MassRange range{(long long)p.tile_off[p.batch] * Hkv * (PASS == 0 ? p.n_row_blocks : 1), p.grid};
+    const long long t0 = range.start(blockIdx.x), t1 = range.start(blockIdx.x + 1);      // never empty: the grid is not above the total
+    const MassCursor first = mass_locate<PASS>(p, t0);
 
     // ---- set-up
     if (tid >= 32 && tid < 32 + kSlots) mbar_init(smem_u32(&sh->full[tid - 32]), 1);
     else if (tid >= 40 && tid < 40 + kSlots) mbar_init(smem_u32(&sh->empty[tid - 40]), 1);
     else if (tid >= 48 && tid < 50) mbar_init(smem_u32(&sh->res_full[tid - 48]), 1);
     else if (tid >= 50 && tid < 52) mbar_init(smem_u32(&sh->res_free[tid - 50]), 1);
-    else if (tid >= 52 && tid < 54) mbar_init(smem_u32(&sh->s_full[tid - 52]), 1);
-    else if (tid >= 54 && tid < 56) mbar_init(smem_u32(&sh->s_free[tid - 54]), kMassConsumers);
-    else if (tid == 56) mbar_init(smem_u32(&sh->drain), 1);
-    else if (tid == 57) { sh->abort = 0; sh->wait_limit = p.header->wait_limit_ns; }
+    else if (tid >= 52 && tid < 52 + kAcc) mbar_init(smem_u32(&sh->s_full[tid - 52]), 1);
+    else if (tid >= 56 && tid < 56 + kAcc) mbar_init(smem_u32(&sh->s_free[tid - 56]), kMassConsumers);
+    else if (tid == 60) mbar_init(smem_u32(&sh->drain), 1);
+    else if (tid == 61) sh->abort = 0;
     if (tid == 0) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(&k_map) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&q_map) : "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh->tmem_base)), "r"(256) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh->tmem_base)), "r"(kAcc * kMassTile) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     // Rows of a tile that no load ever writes (the last 128 - T*G rows of a Q block, a missing second page) must hold
     // finite numbers: clear all tile buffers once.
     for (int x = tid; x < (kRes + kSlots) * kTileBytes / 16; x += kMassThreads) reinterpret_cast<uint4 *>(res)[x] = make_uint4(0, 0, 0, 0);
+    // what follows reads memory that kernels before this one write
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (tid == 61) sh->wait_limit = p.header->wait_limit_ns;
     if (PASS == 1) {
-        const float *src = p.table_log2 + (size_t)unit * p.r_tot;
+        const float *src = p.table_log2 + (size_t)(first.b * Hkv + first.hk) * p.r_tot;
         for (int x = tid; x < tab_entries; x += kMassThreads) tab[x] = x < p.r_tot ? src[x] : -INFINITY;
     }
     fence_proxy_async();
@@ -186,31 +229,34 @@ mass_tc_kernel(const MassParams p, const __grid_constant__ CUtensorMap k_map, co
     if (warp == 0) {
         // ================= TMA producer =================
         if (lane == 0) {
+            MassCursor c = first;
             auto load_keys = [&](uint8_t *dst, int kt, uint32_t bar) {
-                const int pages_b = (nv + kPageSize - 1) / kPageSize;
+                const int b = c.b, hk = c.hk, pages_b = (p.n_visual[b] + kPageSize - 1) / kPageSize;
                 const int np = min(2, pages_b - 2 * kt);
                 mbar_expect_tx(bar, np * kChunks * kPageChunkBytes);
                 for (int q = 0; q < np; ++q) {
                     const int row = (page_of(p.page_table, p.max_pages_per_seq, b, 2 * kt + q) * Hkv + hk) * kPageSize;
 #pragma unroll
-                    for (int c = 0; c < kChunks; ++c)
-                        tma_load_2d(smem_u32(dst) + c * kChunkBytes + q * kPageChunkBytes, &k_map, c * 64, row, bar);
+                    for (int ch = 0; ch < kChunks; ++ch)
+                        tma_load_2d(smem_u32(dst) + ch * kChunkBytes + q * kPageChunkBytes, &k_map, ch * 64, row, bar);
                 }
             };
             auto load_rows = [&](uint8_t *dst, int blk, uint32_t bar) {
                 mbar_expect_tx(bar, kChunks * TG * 128);
 #pragma unroll
-                for (int c = 0; c < kChunks; ++c) tma_load_4d(smem_u32(dst) + c * kChunkBytes, &q_map, c * 64, hk * G, blk * T, b, bar);
+                for (int ch = 0; ch < kChunks; ++ch) tma_load_4d(smem_u32(dst) + ch * kChunkBytes, &q_map, ch * 64, c.hk * G, blk * T, c.b, bar);
             };
             RingPos rp{0, 0};
             uint32_t issued = 0, res_issued = 0;
             bool ok = true;
-            for (int o = o0; o < o1 && ok; ++o) {
-                const int rbuf = (o - o0) % kRes;
-                ok = mass_wait(sh, hdr, &sh->res_free[rbuf], ((((o - o0) / kRes) & 1) ^ 1), 1);
+            int i0, i1;
+            for (long long t = t0; t < t1 && ok;) {
+                const int n = mass_segment<PASS>(p, c, t1 - t, i0, i1);
+                const int rbuf = (int)(res_issued % kRes);
+                ok = mass_wait(sh, hdr, &sh->res_free[rbuf], (((res_issued / kRes) & 1) ^ 1), 1);
                 if (!ok) break;
-                if (PASS == 0) load_rows(res + rbuf * kTileBytes, o, smem_u32(&sh->res_full[rbuf]));
-                else load_keys(res + rbuf * kTileBytes, o, smem_u32(&sh->res_full[rbuf]));
+                if (PASS == 0) load_rows(res + rbuf * kTileBytes, c.rb, smem_u32(&sh->res_full[rbuf]));
+                else load_keys(res + rbuf * kTileBytes, c.kt, smem_u32(&sh->res_full[rbuf]));
                 ++res_issued;
                 for (int i = i0; i < i1; ++i, rp.advance(kSlots), ++issued) {
                     ok = mass_wait(sh, hdr, &sh->empty[rp.slot], rp.phase ^ 1, 2);
@@ -218,6 +264,8 @@ mass_tc_kernel(const MassParams p, const __grid_constant__ CUtensorMap k_map, co
                     if (PASS == 0) load_keys(ring + rp.slot * kTileBytes, i, smem_u32(&sh->full[rp.slot]));
                     else load_rows(ring + rp.slot * kTileBytes, i, smem_u32(&sh->full[rp.slot]));
                 }
+                t += n;
+                mass_advance<PASS>(p, c, n);
             }
             // every load that was issued must have landed before the CTA may exit
             const int back = issued < (uint32_t)kSlots ? (int)issued : kSlots;
@@ -235,30 +283,35 @@ mass_tc_kernel(const MassParams p, const __grid_constant__ CUtensorMap k_map, co
             const uint64_t adesc0 = smem_desc(smem_u32(res), 16, 1024, 2);
             const uint64_t bdesc0 = smem_desc(smem_u32(ring), 16, 1024, 2);
             RingPos rp{0, 0};
-            uint32_t it = 0;
+            uint32_t it = 0, o = 0;
             bool ok = true;
-            for (int o = o0; o < o1 && ok; ++o) {
-                const int rbuf = (o - o0) % kRes;
-                ok = mass_wait(sh, hdr, &sh->res_full[rbuf], ((o - o0) / kRes) & 1, 5);
+            MassCursor c = first;
+            int i0, i1;
+            for (long long t = t0; t < t1 && ok; ++o) {
+                const int n = mass_segment<PASS>(p, c, t1 - t, i0, i1);
+                const int rbuf = (int)(o % kRes);
+                ok = mass_wait(sh, hdr, &sh->res_full[rbuf], (o / kRes) & 1, 5);
                 for (int i = i0; i < i1 && ok; ++i, ++it, rp.advance(kSlots)) {
-                    const int j = it & 1;
+                    const int j = it % kAcc;
                     ok = mass_wait(sh, hdr, &sh->full[rp.slot], rp.phase, 6);
                     if (!ok) break;
-                    if (it >= 2) { ok = mass_wait(sh, hdr, &sh->s_free[j], ((it - 2) >> 1) & 1, 7); if (!ok) break; }
+                    if (it >= (uint32_t)kAcc) { ok = mass_wait(sh, hdr, &sh->s_free[j], (it / kAcc - 1) & 1, 7); if (!ok) break; }
                     tc_fence_after();
                     const uint64_t ad = adesc0 + (uint64_t)((uint32_t)(rbuf * kTileBytes) >> 4);
                     const uint64_t bd = bdesc0 + (uint64_t)((uint32_t)(rp.slot * kTileBytes) >> 4);
 #pragma unroll
-                    for (int c = 0; c < kChunks; ++c)
+                    for (int ch = 0; ch < kChunks; ++ch)
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks) {
-                            const uint64_t off = (uint64_t)((c * kChunkBytes + ks * 32) >> 4);
-                            tc_mma(tmem + j * kMassTile, ad + off, bd + off, idesc, (c | ks) ? 1u : 0u);
+                            const uint64_t off = (uint64_t)((ch * kChunkBytes + ks * 32) >> 4);
+                            tc_mma(tmem + j * kMassTile, ad + off, bd + off, idesc, (ch | ks) ? 1u : 0u);
                         }
                     tc_commit(smem_u32(&sh->s_full[j]));
                     tc_commit(smem_u32(&sh->empty[rp.slot]));
                 }
                 if (ok) tc_commit(smem_u32(&sh->res_free[rbuf]));
+                t += n;
+                mass_advance<PASS>(p, c, n);
             }
             // all tensor-core work of this CTA must be complete before tensor memory is released
             tc_commit(smem_u32(&sh->drain));
@@ -274,13 +327,16 @@ mass_tc_kernel(const MassParams p, const __grid_constant__ CUtensorMap k_map, co
         const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
         const float sl2 = p.sl2;
         const int c0 = slice * kMassSliceCols;
-        uint32_t it = 0;
+        uint32_t it = 0, o = 0;
         bool ok = true;
-        for (int o = o0; o < o1; ++o) {
+        MassCursor c = first;
+        int i0, i1;
+        for (long long t = t0; t < t1; ++o) {
+            const int n = mass_segment<PASS>(p, c, t1 - t, i0, i1), nv = p.n_visual[c.b], unit = c.b * Hkv + c.hk;
             float m = -INFINITY, l = 0.f, acc = 0.f;
             for (int i = i0; i < i1; ++i, ++it) {
-                const int j = it & 1;
-                if (ok) ok = mass_wait(sh, hdr, &sh->s_full[j], (it >> 1) & 1, 9);
+                const int j = it % kAcc;
+                if (ok) ok = mass_wait(sh, hdr, &sh->s_full[j], (it / kAcc) & 1, 9);
                 if (!ok) continue;
                 tc_fence_after();
                 // columns: keys of tile i (pass 0) / packed rows of block i (pass 1)
@@ -362,7 +418,7 @@ mass_tc_kernel(const MassParams p, const __grid_constant__ CUtensorMap k_map, co
                 mbar_arrive(smem_u32(&sh->s_free[j]));
             }
             // the four slices of a lane meet in shared memory (double buffered over the outer steps)
-            float2 *pt = part + ((o - o0) & 1) * (kMassSlices * kMassTile);
+            float2 *pt = part + (o & 1) * (kMassSlices * kMassTile);
             pt[slice * kMassTile + L] = PASS == 0 ? make_float2(m, l) : make_float2(acc, 0.f);
             asm volatile("bar.sync 1, %0;" ::"n"(kMassConsumers) : "memory");
             if (slice == 0 && ok && !sh->abort) {
@@ -376,15 +432,24 @@ mass_tc_kernel(const MassParams p, const __grid_constant__ CUtensorMap k_map, co
                         const float2 v = pt[q * kMassTile + L];
                         if (v.y > 0.f) Ls += v.y * ex2_approx(v.x - M);
                     }
-                    if (L < TG && o * TG + L < p.r_tot)
-                        p.stats[((size_t)unit * p.stat_splits + split) * p.r_tot + o * TG + L] = make_float2(M, Ls);
+                    // the row block's partials are numbered from the first CTA that has a part of it
+                    const int slot = (int)blockIdx.x - range.cta_of(t - c.kt);
+                    if (L < TG && c.rb * TG + L < p.r_tot)
+                        p.stats[((size_t)unit * p.stat_slots + slot) * p.r_tot + c.rb * TG + L] = make_float2(M, Ls);
                 } else {
                     float sum = acc;
 #pragma unroll
                     for (int q = 1; q < kMassSlices; ++q) sum += pt[q * kMassTile + L].x;
-                    const int key = o * kMassTile + L;
-                    if (key < nv) p.colsum[(size_t)hk * p.sum_nv + p.offset[b] + key] = sum;
+                    const int key = c.kt * kMassTile + L;
+                    if (key < nv) p.colsum[(size_t)c.hk * p.sum_nv + p.offset[c.b] + key] = sum;
                 }
+            }
+            t += n;
+            mass_advance<PASS>(p, c, n);
+            if (PASS == 1 && t < t1 && c.b * Hkv + c.hk != unit) {       // another head: all are past their last look at this one's table
+                const float *src = p.table_log2 + (size_t)(c.b * Hkv + c.hk) * p.r_tot;
+                for (int x = tid - 64; x < tab_entries; x += kMassConsumers) tab[x] = x < p.r_tot ? src[x] : -INFINITY;
+                asm volatile("bar.sync 1, %0;" ::"n"(kMassConsumers) : "memory");
             }
         }
     }
@@ -392,22 +457,31 @@ mass_tc_kernel(const MassParams p, const __grid_constant__ CUtensorMap k_map, co
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kAcc * kMassTile) : "memory");
     }
 }
 
 // One thread per packed row of a KV head: merge the key splits of pass 1 into t = -(max + log2 sum).
 __global__ void mass_merge_kernel(const MassParams p) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // pass 2 sets itself up meanwhile
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long total = (long long)p.batch * p.n_kv_heads * p.r_tot;
     if (x >= total) return;
     const int r = (int)(x % p.r_tot);
     const int unit = (int)(x / p.r_tot);
-    const float2 *src = p.stats + (size_t)unit * p.stat_splits * p.r_tot + r;
+    const int b = unit / p.n_kv_heads, hk = unit % p.n_kv_heads, n_kt = p.tile_off[b + 1] - p.tile_off[b];
+    int n = 0;                                // CTAs that have a part of the row's block
+    if (n_kt > 0) {
+        const MassRange range{(long long)p.tile_off[p.batch] * p.n_kv_heads * p.n_row_blocks, p.stat_grid};
+        const long long at = ((long long)p.tile_off[b] * p.n_kv_heads + (long long)hk * n_kt) * p.n_row_blocks + (long long)(r / p.rows_per_block) * n_kt;
+        n = range.cta_of(at + n_kt - 1) - range.cta_of(at) + 1;
+    }
+    const float2 *src = p.stats + (size_t)unit * p.stat_slots * p.r_tot + r;
     float M = -INFINITY;
-    for (int s = 0; s < p.stat_splits; ++s) M = fmaxf(M, src[(size_t)s * p.r_tot].x);
+    for (int s = 0; s < n; ++s) M = fmaxf(M, src[(size_t)s * p.r_tot].x);
     float Lsum = 0.f;
-    for (int s = 0; s < p.stat_splits; ++s) {
+    for (int s = 0; s < n; ++s) {
         const float2 v = src[(size_t)s * p.r_tot];
         if (v.y > 0.f) Lsum += v.y * exp2f(v.x - M);
     }
@@ -416,6 +490,8 @@ __global__ void mass_merge_kernel(const MassParams p) {
 
 // mass += weight * (column sums of the KV heads, added in head order)
 __global__ void mass_reduce_kernel(const MassParams p) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= p.sum_nv) return;
     float s = 0.f;
@@ -478,23 +554,9 @@ __global__ void mass_generic_sum_kernel(const MassParams p) {
 // ---- host side ---------------------------------------------------------------------------------------------------------
 struct MassPlan {
     bool tc;
-    int T, TG, RB, r_tot, stat_splits, sum_splits, max_nkt;
+    int T, TG, RB, r_tot, stat_grid, sum_grid, stat_slots;
     size_t stats_off, table_off, colsum_off, total;
 };
-
-// Key splits for `items` equal work items of `tiles` key tiles each (every key tile costing `inner` accumulator
-// tiles): the CTAs run one per SM in waves, so the cost is waves x (accumulator tiles per CTA + a fixed start-up).
-static int mass_best_splits(int items, int tiles, int inner, int ctas_per_sm) {
-    int best = 1;
-    long long best_cost = -1;
-    const int room = kNumSMs * ctas_per_sm;
-    for (int s = 1; s <= tiles && s <= kMassMaxSplits; ++s) {
-        const long long waves = ((long long)items * s + room - 1) / room;
-        const long long cost = waves * ((long long)ceil_div(tiles, s) * inner + 4);
-        if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = s; }
-    }
-    return best;
-}
 
 static MassPlan mass_plan(int batch, const int32_t *n_visual, int l_txt, int n_q_heads, int n_kv_heads, int head_dim, int dtype) {
     MassPlan pl;
@@ -505,15 +567,26 @@ static MassPlan mass_plan(int batch, const int32_t *n_visual, int l_txt, int n_q
     if (pl.T > l_txt) pl.T = l_txt;
     pl.TG = pl.T * G;
     pl.RB = ceil_div(l_txt, pl.T);
-    long long sum_nv = 0;
-    int max_nv = 0;
-    for (int b = 0; b < batch; ++b) { sum_nv += n_visual[b]; if (n_visual[b] > max_nv) max_nv = n_visual[b]; }
-    pl.max_nkt = ceil_div(max_nv > 0 ? max_nv : 1, kMassTile);
+    long long sum_nv = 0, tiles = 0, longest = 0;         // key tiles of all sequences, of the longest
+    for (int b = 0; b < batch; ++b) {
+        const long long n = ceil_div(n_visual[b], kMassTile);
+        sum_nv += n_visual[b];
+        tiles += n;
+        if (n > longest) longest = n;
+    }
     const int units = batch * n_kv_heads;
-    pl.stat_splits = pl.tc ? mass_best_splits(units * pl.RB, pl.max_nkt, 1, MassBuffers<0>::kCtasPerSm) : 1;
-    pl.sum_splits = mass_best_splits(units, pl.max_nkt, pl.RB, MassBuffers<1>::kCtasPerSm);
+    // one wave, one entry of the flat list per CTA at least; a row block's entries lie in at most stat_slots CTAs' ranges
+    const long long stat_total = tiles * n_kv_heads * pl.RB, sum_total = tiles * n_kv_heads;
+    auto at_most = [](long long n, int room) { return (int)(n < 1 ? 1 : n < room ? n : room); };
+    pl.stat_grid = at_most(stat_total, kNumSMs * MassBuffers<0>::kCtasPerSm);
+    pl.sum_grid = at_most(sum_total, kNumSMs * MassBuffers<1>::kCtasPerSm);
+    pl.stat_slots = 1;
+    if (pl.tc && longest > 0) {
+        const long long least = stat_total / pl.stat_grid;            // entries of the shortest range
+        pl.stat_slots = at_most((longest + least - 1) / least + 1, pl.stat_grid);
+    }
     pl.stats_off = kWsHeaderBytes;
-    pl.table_off = align_up(pl.stats_off + (size_t)units * pl.stat_splits * pl.r_tot * sizeof(float2), 256);
+    pl.table_off = align_up(pl.stats_off + (size_t)units * pl.stat_slots * pl.r_tot * sizeof(float2), 256);
     pl.colsum_off = align_up(pl.table_off + (size_t)units * pl.r_tot * sizeof(float2), 256);
     pl.total = align_up(pl.colsum_off + (size_t)n_kv_heads * (size_t)sum_nv * sizeof(float), 256);
     return pl;
@@ -547,6 +620,23 @@ static int32_t make_k_map(CUtensorMap *m, const void *pool, long long rows, int 
     return HIPPO_OK;
 }
 
+// Each kernel of the chain begins with griddepcontrol.wait: its set-up (barriers, tensor memory, cleared tiles) overlaps the end of the
+// one before.
+template <typename... Args>
+static cudaError_t launch_mass_dependent(void (*kernel)(Args...), long long grid, int threads, size_t smem, cudaStream_t s, Args... args) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 template <int D>
 static int32_t launch_mass_tc(MassParams &p, const MassPlan &pl, long long pool_rows, cudaStream_t s) {
     CUtensorMap km, qm;
@@ -566,15 +656,12 @@ static int32_t launch_mass_tc(MassParams &p, const MassPlan &pl, long long pool_
         attr_set.mark(dev);
     }
     const int units = p.batch * p.n_kv_heads;
-    p.splits = pl.stat_splits;
-    mass_tc_kernel<D, 0><<<(unsigned)(units * pl.RB * pl.stat_splits), kMassThreads, smem0, s>>>(p, km, qm);
-    HIPPO_CUDA_TRY(cudaGetLastError());
+    p.grid = p.stat_grid;
+    HIPPO_CUDA_TRY(launch_mass_dependent(mass_tc_kernel<D, 0>, p.grid, kMassThreads, smem0, s, p, km, qm));
     const long long rows = (long long)units * p.r_tot;
-    mass_merge_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, s>>>(p);
-    HIPPO_CUDA_TRY(cudaGetLastError());
-    p.splits = pl.sum_splits;
-    mass_tc_kernel<D, 1><<<(unsigned)(units * pl.sum_splits), kMassThreads, smem1, s>>>(p, km, qm);
-    HIPPO_CUDA_TRY(cudaGetLastError());
+    HIPPO_CUDA_TRY(launch_mass_dependent(mass_merge_kernel, (rows + 255) / 256, 256, 0, s, p));
+    p.grid = pl.sum_grid;
+    HIPPO_CUDA_TRY(launch_mass_dependent(mass_tc_kernel<D, 1>, p.grid, kMassThreads, smem1, s, p, km, qm));
     count_launches(3);
     return HIPPO_OK;
 }
@@ -643,7 +730,7 @@ extern "C" int32_t hippo_attention_mass(int32_t batch, const int32_t *n_visual, 
     p.batch = batch; p.l_txt = l_txt; p.n_q_heads = n_q_heads; p.n_kv_heads = kv->n_kv_heads;
     p.group = n_q_heads / kv->n_kv_heads; p.head_dim = kv->head_dim;
     p.t_per_block = pl.T; p.rows_per_block = pl.TG; p.n_row_blocks = pl.RB; p.r_tot = pl.r_tot;
-    p.splits = 1; p.stat_splits = pl.stat_splits; p.sum_nv = (int)sum_nv; p.max_pages_per_seq = kv->max_pages_per_seq;
+    p.grid = 0; p.stat_grid = pl.stat_grid; p.stat_slots = pl.stat_slots; p.sum_nv = (int)sum_nv; p.max_pages_per_seq = kv->max_pages_per_seq;
     p.scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)kv->head_dim);
     p.sl2 = p.scale * kMassLog2e;
     p.weight = weight;
@@ -654,12 +741,15 @@ extern "C" int32_t hippo_attention_mass(int32_t batch, const int32_t *n_visual, 
     p.colsum = (float *)((char *)workspace + pl.colsum_off);
     p.mass = mass;
     p.header = (WsHeader *)workspace;
-    int off = 0;
+    int off = 0, tiles = 0;
     for (int b = 0; b < kMassMaxBatch; ++b) {
         p.n_visual[b] = b < batch ? n_visual[b] : 0;
         p.offset[b] = off;
+        p.tile_off[b] = tiles;
         off += p.n_visual[b];
+        tiles += ceil_div(p.n_visual[b], kMassTile);
     }
+    p.tile_off[kMassMaxBatch] = tiles;
     cudaStream_t s = (cudaStream_t)stream;
     int32_t rc;
     if (pl.tc) {
@@ -671,8 +761,7 @@ extern "C" int32_t hippo_attention_mass(int32_t batch, const int32_t *n_visual, 
         rc = launch_mass_generic<__nv_bfloat16>(p, max_nv, s);
     }
     if (rc != HIPPO_OK) return rc;
-    mass_reduce_kernel<<<(unsigned)((sum_nv + 255) / 256), 256, 0, s>>>(p);
-    HIPPO_CUDA_TRY(cudaGetLastError());
+    HIPPO_CUDA_TRY(launch_mass_dependent(mass_reduce_kernel, (sum_nv + 255) / 256, 256, 0, s, p));
     count_launches(1);
     return HIPPO_OK;
 }

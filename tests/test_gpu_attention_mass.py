@@ -176,3 +176,13 @@ def test_bounded_wait_runs_out_and_the_workspace_recovers(hb):
     ref = oracle.attention_mass(q[None], k[None], nv)[0][:nv[0]]
     got = host(mass)
     assert np.all(np.abs(got - ref) <= RTOL["bf16"] * ref + 1e-12)
+
+
+@pytest.mark.parametrize("nv,L,Hq,Hkv,D", [([1], 3, 2, 1, 64), ([0, 128, 129, 0, 1000], 40, 8, 4, 64), ([5000], 256, 16, 8, 64),
+                                           ([40, 3000, 700], 33, 14, 2, 128), ([2000] * 3, 256, 28, 4, 128)])
+def test_ranges_that_end_anywhere(hb, nv, L, Hq, Hkv, D):
+    """The passes' work is cut into equal ranges: ones that end inside a row block, a head or a sequence, sequences without keys, fewer
+    entries than places."""
+    qs, ks = rand_case(sum(nv) + L, len(nv), L, Hq, Hkv, D, max(max(nv), 1), "bf16")
+    got = gpu_mass(hb, qs, ks, nv, "bf16", shuffle_seed=3)
+    check(got, oracle_mass(qs, ks, nv), "bf16", "nv %s" % (nv,))
