@@ -121,7 +121,10 @@ __device__ __forceinline__ int2 aligned_split_warp(int lane, int U, int grid, in
     const int spare = grid - __popc(__ballot_sync(0xffffffffu, live));
     int base = 0;
     uint32_t r = 0;
-    if (live) {
+    if (total < (1 << 22)) {                  // the product fits 32 bits (at most kExtraSlots CTAs)
+        const uint32_t num = (uint32_t)spare * (uint32_t)my_tiles, t = (uint32_t)total;
+        if (live) { base = (int)(num / t); r = num % t; }
+    } else if (live) {
         const long long num = (long long)spare * my_tiles;
         base = (int)(num / total);
         r = (uint32_t)(num % total);
@@ -131,11 +134,13 @@ __device__ __forceinline__ int2 aligned_split_warp(int lane, int U, int grid, in
     for (int o = 16; o; o >>= 1) sum_base += __shfl_xor_sync(0xffffffffu, sum_base, o);
     const int leftover = spare - sum_base;
     int rank = 0;
-    for (int v = 0; v < U; ++v) {
-        const uint32_t rv = __shfl_sync(0xffffffffu, r, v);
-        const int lv = __shfl_sync(0xffffffffu, (int)live, v);
-        rank += (lv && (rv > r || (rv == r && v < lane))) ? 1 : 0;
-    }
+    const unsigned lives = __ballot_sync(0xffffffffu, live);
+    for (int v0 = 0; v0 < U; v0 += 4)         // lanes beyond the last unit are not live
+#pragma unroll
+        for (int v = v0; v < v0 + 4; ++v) {
+            const uint32_t rv = __shfl_sync(0xffffffffu, r, v);
+            rank += (lives >> v & 1u) && (rv > r || (rv == r && v < lane)) ? 1 : 0;
+        }
     const int n = live ? min(my_tiles, 1 + base + (rank < leftover ? 1 : 0)) : 0;
     int cinc = n;
 #pragma unroll
@@ -258,6 +263,32 @@ static TcSmemPlan tc_smem_plan(int D, int Rp) {
     return s;
 }
 
+// a word that another kernel may be writing: from L2, so that no old line stays in L1
+__device__ __forceinline__ int tc_peek(const int32_t *p) {
+    int v;
+    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// Asks L2 for the first pages of this CTA's range (warp 0, unit-aligned split, tables in place).  A page is 64 rows of a head in a row.
+// Worth it where few units have many CTAs each: one sequence of 30,000 keys, 8 kv heads, 30.6 -> 29.7 us a call, of 20,000, 4 kv heads, 21.0 ->
+// 20.5; two of 8,000, 4 kv heads, 18.7 either way; four of 8,192, 4 kv heads, 24.4 -> 24.9.  In clusters one of 4,000 14.2 -> 14.7.
+constexpr int kPrefetchPages = 4, kPrefetchUnits = 8;
+template <int D>
+__device__ __forceinline__ void prefetch_first_pages(const AttnParams &p, const TcShared *sh, int U) {
+    const int lane = threadIdx.x & 31, c = blockIdx.x, Hkv = p.n_kv_heads;
+    const unsigned mine = __ballot_sync(0xffffffffu, lane < U && c >= sh->cta_base[lane] && c < sh->cta_base[lane] + sh->n_cta[lane]);
+    if (!mine || lane >= 2 * kPrefetchPages) return;
+    const int unit = __ffs(mine) - 1, b = unit / Hkv, hk = unit % Hkv;
+    const int T = sh->tile_prefix[b + 1] - sh->tile_prefix[b], i = c - sh->cta_base[unit], n = sh->n_cta[unit];
+    const int page = (int)((long long)T * i / n) + (lane >> 1);
+    if (page >= (int)((long long)T * (i + 1) / n) || page >= p.max_pages_per_seq) return;
+    const int pid = p.page_table ? tc_peek(p.page_table + (size_t)b * p.max_pages_per_seq + page) : b * p.max_pages_per_seq + page;
+    if ((unsigned)pid >= (unsigned)p.n_pages) return;
+    const __nv_bfloat16 *src = (const __nv_bfloat16 *)(lane & 1 ? p.v_pages : p.k_pages) + ((size_t)pid * Hkv + hk) * kPageSize * D;
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"((uint32_t)(kPageSize * D * 2)) : "memory");
+}
+
 template <int D, int NL>
 __global__ void __launch_bounds__(NL == 1 ? kTcThreads : kTcThreads + 32, 1)
 attn_tc_kernel(const AttnParams p, const __grid_constant__ LayerSetT<NL> set, const MultiCtl mc,
@@ -308,18 +339,8 @@ attn_tc_kernel(const AttnParams p, const __grid_constant__ LayerSetT<NL> set, co
             asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh->tmem_base)), "r"(tmem_cols) : "memory");
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
         }
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        if (tid == kThreads - 1) sh->wait_limit = p.header->wait_limit_ns;
-        if (!small_problem) {
-            // tiles per sequence; the exclusive prefix follows the barrier
-            for (int b = tid; b < B; b += kThreads) {
-                const int kvl = p.kv_len ? p.kv_len[b] : p.max_kv_len;
-                sh->kvlen[b] = kvl;
-                sh->tile_prefix[b + 1] = seq_tiles(kvl, p.q_len);
-            }
-        } else if (warp == 0) {
-            // lane b: sequence b; lane u: unit u.  Everything by shuffles.
-            const int kvl = lane < B ? (p.kv_len ? p.kv_len[lane] : p.max_kv_len) : 0;
+        // Tables of at most 32 units, by warp 0.  Lane b: sequence b; lane u: unit u.  Everything by shuffles.
+        auto small_tables = [&](int kvl) {
             const int nt = lane < B ? seq_tiles(kvl, p.q_len) : 0;
             int incl = nt;
 #pragma unroll
@@ -336,6 +357,31 @@ attn_tc_kernel(const AttnParams p, const __grid_constant__ LayerSetT<NL> set, co
                 if (lane < U) { sh->n_cta[lane] = mine.y; sh->cta_base[lane] = mine.x; }
                 if (lane == 0) sh->cta_base[U] = all;
             }
+            __syncwarp();
+        };
+        // A single-layer call mostly becomes resident while its predecessor ends.  Warp 0 uses that time to work out the tables from the
+        // lengths as they stand (eight ragged sequences of 10,406 keys 41.4 -> 39.4 us a call, with the earlier launch that the combine kernel
+        // allows) and may ask L2 for the first pages.  The lengths are looked up again after the wait; page ids, which nothing but the
+        // prefetch uses, count only inside the pool.
+        const bool peek = !kMulti && small_problem;
+        int peeked = 0;
+        if (peek && warp == 0) {
+            if (lane < B) peeked = p.kv_len ? min(max(tc_peek(p.kv_len + lane), 0), p.max_kv_len) : p.max_kv_len;
+            small_tables(peeked);
+            if (aligned && U <= kPrefetchUnits) prefetch_first_pages<D>(p, sh, U);
+        }
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (tid == kThreads - 1) sh->wait_limit = p.header->wait_limit_ns;
+        if (!small_problem) {
+            // tiles per sequence; the exclusive prefix follows the barrier
+            for (int b = tid; b < B; b += kThreads) {
+                const int kvl = p.kv_len ? p.kv_len[b] : p.max_kv_len;
+                sh->kvlen[b] = kvl;
+                sh->tile_prefix[b + 1] = seq_tiles(kvl, p.q_len);
+            }
+        } else if (warp == 0) {
+            const int kvl = lane < B ? (p.kv_len ? __ldcg(p.kv_len + lane) : p.max_kv_len) : 0;
+            if (!peek || !__all_sync(0xffffffffu, lane >= B || kvl == peeked)) small_tables(kvl);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -1154,6 +1200,7 @@ __global__ void __launch_bounds__(kCombineThreads) attn_tc_combine_kernel(const 
     const int h = row % p.n_q_heads, t = (row / p.n_q_heads) % p.q_len, b = row / (p.n_q_heads * p.q_len);
     const int hk = h / G, r = t * G + (h % G);
     __nv_bfloat16 *out = (__nv_bfloat16 *)p.out + (size_t)row * D;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // the next call's CTAs may take the SMs that the main kernel leaves
     if (main_grid > 0) {
         // Unit-aligned split with at most 32 units: which partials belong to this row's unit follows from the lengths
         // alone.  The lengths are an input of the call, complete before the main kernel let this one be launched, so
@@ -1174,7 +1221,6 @@ __global__ void __launch_bounds__(kCombineThreads) attn_tc_combine_kernel(const 
         __syncthreads();
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int2 info = main_grid > 0 ? s_info : reinterpret_cast<const int2 *>(p.counters)[b * Hkv + hk];   // first slot, contributors
     const int n = info.y;
     if (n == 0) {   // a sequence shorter than q_len is skipped: its outputs are defined as zero
@@ -1246,6 +1292,7 @@ __global__ void __launch_bounds__(kCombineThreads) attn_tc_combine_rows_kernel(c
     __shared__ int2 s_info[32];
     const int R = p.rows, G = p.group, Hkv = p.n_kv_heads;
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (main_grid > 0) {                              // as above
         if (w == 0) {
             const int U = p.batch * Hkv;
@@ -1261,7 +1308,6 @@ __global__ void __launch_bounds__(kCombineThreads) attn_tc_combine_rows_kernel(c
         __syncthreads();
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int row = blockIdx.x * (kCombineThreads / 32) + w;
     if (row >= n_rows) return;
     const int h = row % p.n_q_heads, t = (row / p.n_q_heads) % p.q_len, b = row / (p.n_q_heads * p.q_len);
