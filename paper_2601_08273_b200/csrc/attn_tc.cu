@@ -1457,31 +1457,33 @@ static int aligned_longest(const AttnParams &p, int grid) {
     return longest;
 }
 
-// How a single-layer call is split: > 1 one cluster of so many CTAs per unit, kAligned or kFlat.  Times in us of a call in a chain of
-// them, by the pages of the longest CTA (up to 32 packed rows / each 16 rows more): clusters 12 + 0.53 per page / 1.3 and 0.09, then 0.055 (128
-// CTAs saturate HBM as well as 148), aligned 14.5 + 0.645 / 0.055, flat 15.5 + 0.667 / 0.055 (1.5 besides) with the average in place of the
-// longest.  Measured, clusters / aligned / flat, head size 128: eight ragged sequences of 10,406 keys, 4 kv heads, 42 rows 45.8 / 41.8 / 43.8;
-// of 12,000, 8 kv heads, 24 rows 70.0 / 79.9 / 70.7; of 9,000, 8 kv heads, 48 rows 65.0 / 66.4 / 59.6; four of 13,000, 8 kv heads, 24 rows
-// 42.6 / 46.5 / 44.4, of 3,000 with 72 rows 26.8 / 25.1 / 29.6; one of 3,000, 48 rows 14.0 / 15.7 / 18.5, of 8,000 20.2 / 19.1 / 21.5.  Head
-// size 64, eight of 10,406, 42 rows: 38.5 / 35.2 / 36.2.
+// How a single-layer call is split: > 1 one cluster of so many CTAs per unit, kAligned or kFlat.  The times, in us of a call in a chain of
+// them, are fitted to 75 shapes (head size 128, 1 to 64 units, 14 to 72 packed rows; 5 to 8 % off, the mean loss of the choice 1.4 %): a
+// constant, the pages of the longest CTA (the average for the flat split), the units, and the groups of 16 rows beyond 32 in each.
+// Measured, clusters / aligned / flat: eight ragged sequences of 10,406 keys, 4 kv heads, 42 rows 45.9 / 40.2 / 44.1; of 12,000, 8 kv heads,
+// 24 rows 70.3 / 80.9 / 72.5; of 9,000, 8 kv heads, 48 rows 65.2 / 67.2 / 60.5; four of 13,000, 8 kv heads, 24 rows 42.6 / 45.0 / 45.4, of 3,000
+// with 72 rows 26.4 / 24.0 / 29.8; one of 3,000, 48 rows 14.2 / 15.8 / 18.4, of 9,000, 4 kv heads, 28 rows 16.7 / 15.4 / 15.0.  Head size 64,
+// eight of 10,406, 42 rows: 38.8 / 34.2 / 37.2.
 constexpr int kAligned = 0, kFlat = -1;
 static int choose_split(const AttnParams &p, int rows_padded, const int *max_active) {
     const int units = p.batch * p.n_kv_heads, groups = rows_padded / 16;
     int pages;
     long long total_pages;
     plan_pages(p, pages, total_pages);
-    const float more = groups <= 2 ? 0.f : groups - 2.f;                                  // groups of rows beyond 32
-    const int even = aligned_longest(p, split_grid(p, kNumSMs));
+    // a page or two per CTA: one sequence of 1,500 keys, 4 kv heads, 28 rows 11.7 / 10.6 / 10.2, of 4,000, 63 rows 15.6 / 15.9 / 14.7
+    if (total_pages <= 256) return kFlat;
+    const float g = groups <= 2 ? 0.f : groups - 2.f, u16 = units < 16 ? units : 16, u32 = units < 32 ? units : 32;
+    const int grid = split_grid(p, kNumSMs), even = aligned_longest(p, grid);
     int best = kFlat;
-    float best_us = 15.5f + 1.5f * (groups > 2) + (0.667f + 0.055f * more) * (float)((total_pages + kNumSMs - 1) / kNumSMs);
+    float best_us = 10.2f + 0.385f * g + (0.703f + 0.037f * g) * (float)((total_pages + grid - 1) / grid) + (0.296f + 0.106f * g) * u16;
     if (even > 0) {
-        const float us = 14.5f + (0.645f + 0.055f * more) * even;
+        const float us = 11.6f + 1.32f * g + (0.69f + 0.034f * g) * even + (0.027f - 0.0154f * g) * u32;
         if (us < best_us) { best = kAligned; best_us = us; }
     }
     // a cluster of more than eight needs most of a GPC, and only six of them can be counted on to hold one
     for (int cs = 2; cs <= (units <= 6 ? 16 : 8) && 2 * cs <= pages + 1; ++cs) {
         if (units > max_active[cs]) continue;
-        const float us = 12.f + 1.3f * more + (0.53f + 0.09f * (more > 0.f) + 0.055f * (more > 1.f ? more - 1.f : 0.f)) * ceil_div(pages, cs);
+        const float us = 9.6f + 1.0f * g + (0.564f + 0.045f * g) * ceil_div(pages, cs) + (0.079f + 0.029f * g) * u32;
         if (us < best_us) { best = cs; best_us = us; }
     }
     return best;
