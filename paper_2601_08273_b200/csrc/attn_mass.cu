@@ -7,7 +7,7 @@
 // times on the tensor cores (bf16, head_dim 64 or 128), and never stored:
 //   pass 1 (row statistics)  S   [128 rows x 128 keys] = Q_block . K_tile^T    thread = row: running max and sum of
 //                                                                                exponentials over its CTA's key tiles
-//   merge                     the key splits of a row -> t = -(max + log2 sum)
+//   merge                     the parts of a row, one from each piece of the work that it lies in -> t = -(max + log2 sum)
 //   pass 2 (column sums)      S^T [128 keys x 128 rows] = K_tile . Q_block^T    thread = key: sum over the rows of
 //                                                                                2^(s + t_row)
 //   reduce                    mass += weight * (sum of the KV heads' column sums), in a fixed order
@@ -41,6 +41,14 @@ constexpr int kMassAcc = 4;              // accumulator tiles that tensor memory
 constexpr int kMassTile = 128;           // rows and keys per accumulator tile
 constexpr int kMassMaxBatch = 64;        // per-sequence lengths travel in the kernel parameters
 constexpr int kMassMaxRows = 3072;       // l_txt * group: the pass-2 table of a KV head lives in shared memory
+// Pass 1 reads each key tile once per row block.  All pieces of the flat list are in work at the same time, so the keys that they read
+// should stay in L2 together: above 64 MB, and where they are read often enough, the list is worked through in rounds.  65,536 tokens, 64
+// heads, 256 text rows (128 MB of keys, 16 row blocks): 715 us in one round, 708 in two, 714 in four, 725 in eight (each piece ends with a
+// partial row block); once the chip has run long enough to be limited by its power 745-765 in one round, 721-730 in two.  64 MB of keys:
+// 209 in one round, 211 in two.  Fewer row blocks, one round and two: 13 x 50,000 tokens x 64 heads 453 and 457 (13 x 65,536, hot: 623 and
+// 594), 8 x 45,000 x 32 in four sequences 276 and 279, 4 x 65,536 x 64 217 and 221.
+constexpr long long kMassRoundBytes = 64ll << 20;
+constexpr int kMassRoundBlocks = 12, kMassMaxRounds = 64;
 constexpr float kMassLog2e = 1.4426950408889634f;
 constexpr unsigned long long kMassWaitLimitNs = 2000000000ull;
 
@@ -50,8 +58,8 @@ struct MassParams {
     int rows_per_block;    // T * G
     int n_row_blocks;      // ceil(l_txt / T)
     int r_tot;             // l_txt * G packed rows per KV head
-    int grid;              // CTAs of this launch (tensor-core path)
-    int stat_grid;         // CTAs of pass 1
+    int pieces;            // of this launch's flat list (tensor-core path): CTA c takes c, c + grid, ...
+    int stat_pieces;       // of pass 1's
     int stat_slots;        // partial results that a row block can have from pass 1 (layout of `stats`)
     int sum_nv;            // total visual tokens
     int max_pages_per_seq;
@@ -72,15 +80,15 @@ struct MassParams {
     int tile_off[kMassMaxBatch + 1];   // key tiles of the sequences before this one
 };
 
-// The work of both passes is one flat list, cut into equal ranges for the CTAs of one wave whatever sequence, head or row block
-// they end in.  Pass 1: (sequence, KV head, row block, key tile); pass 2: (sequence, KV head, key tile).  Before, every (head, row block)
-// was split into the same number of key ranges, 64 x 4 of them for 296 places and 8 x 18 for 148 (32,768 tokens, 32 heads, 256 text rows:
-// 216 us, 210 with the flat list).
+// The work of both passes is one flat list, cut into equal pieces, one or (pass 1, see kMassRoundBytes) a few for each CTA of one wave,
+// whatever sequence, head or row block they end in.  Pass 1: (sequence, KV head, row block, key tile); pass 2: (sequence, KV head, key
+// tile).  Before, every (head, row block) was split into the same number of key ranges, 64 x 4 of them for 296 places and 8 x 18 for 148
+// (32,768 tokens, 32 heads, 256 text rows: 216 us, 210 with the flat list).
 struct MassRange {
     long long total;
-    int grid;
-    __host__ __device__ long long start(int c) const { return total * c / grid; }
-    __host__ __device__ int cta_of(long long t) const { return (int)(((t + 1) * grid - 1) / total); }   // whose range t is in
+    int pieces;
+    __host__ __device__ long long start(int piece) const { return total * piece / pieces; }
+    __host__ __device__ int piece_of(long long t) const { return (int)(((t + 1) * pieces - 1) / total); }   // the one that t is in
 };
 struct MassCursor {
     int b, hk, rb, kt, n_kt;     // sequence, KV head, row block (pass 1), key tile, the sequence's key tiles
@@ -102,9 +110,9 @@ __device__ __forceinline__ MassCursor mass_locate(const MassParams &p, long long
 // A resident tile and what is streamed past it.  Pass 1: a row block, up to `left` key tiles; pass 2: a key tile, all row blocks.
 // Returns how many entries of the flat list that is.
 template <int PASS>
-__device__ __forceinline__ int mass_segment(const MassParams &p, const MassCursor &c, long long left, int &i0, int &i1) {
+__device__ __forceinline__ int mass_segment(const MassParams &p, const MassCursor &c, int left, int &i0, int &i1) {
     if (PASS == 1) { i0 = 0; i1 = p.n_row_blocks; return 1; }
-    const int n = (int)(left < c.n_kt - c.kt ? left : c.n_kt - c.kt);
+    const int n = min(left, c.n_kt - c.kt);
     i0 = c.kt;
     i1 = c.kt + n;
     return n;
@@ -121,6 +129,18 @@ __device__ __forceinline__ void mass_advance(const MassParams &p, MassCursor &c,
     c.hk = 0;
     do ++c.b; while (c.b < p.batch && p.tile_off[c.b + 1] == p.tile_off[c.b]);
     c.n_kt = c.b < p.batch ? p.tile_off[c.b + 1] - p.tile_off[c.b] : 1;
+}
+
+// On by n of the `left` entries of the CTA's piece, or to its next piece.
+template <int PASS>
+__device__ __forceinline__ void mass_step(const MassParams &p, const MassRange &range, MassCursor &c, int n, int &piece, int &left) {
+    left -= n;
+    if (PASS == 1 || left > 0) { mass_advance<PASS>(p, c, n); return; }
+    piece += gridDim.x;
+    if (piece >= range.pieces) return;
+    const long long t = range.start(piece);
+    left = (int)(range.start(piece + 1) - t);
+    c = mass_locate<PASS>(p, t);
 }
 
 struct MassShared {
@@ -187,8 +207,10 @@ mass_tc_kernel(const MassParams p, const __grid_constant__ CUtensorMap k_map, co
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int G = p.group, Hkv = p.n_kv_heads, T = p.t_per_block, TG = p.rows_per_block;
     // outer loop: resident tiles; inner loop: streamed tiles
-    const MassRange range{(long long)p.tile_off[p.batch] * Hkv * (PASS == 0 ? p.n_row_blocks : 1), p.grid};
-    const long long t0 = range.start(blockIdx.x), t1 = range.start(blockIdx.x + 1);      // never empty: the grid is not above the total
+    const MassRange range{(long long)p.tile_off[p.batch] * Hkv * (PASS == 0 ? p.n_row_blocks : 1), p.pieces};
+    int piece = blockIdx.x;
+    const long long t0 = range.start(piece);
+    int left = (int)(range.start(piece + 1) - t0);          // never empty: there are no more pieces than entries
     const MassCursor first = mass_locate<PASS>(p, t0);
 
     // ---- set-up
@@ -250,8 +272,8 @@ mass_tc_kernel(const MassParams p, const __grid_constant__ CUtensorMap k_map, co
             uint32_t issued = 0, res_issued = 0;
             bool ok = true;
             int i0, i1;
-            for (long long t = t0; t < t1 && ok;) {
-                const int n = mass_segment<PASS>(p, c, t1 - t, i0, i1);
+            while (left > 0 && ok) {
+                const int n = mass_segment<PASS>(p, c, left, i0, i1);
                 const int rbuf = (int)(res_issued % kRes);
                 ok = mass_wait(sh, hdr, &sh->res_free[rbuf], (((res_issued / kRes) & 1) ^ 1), 1);
                 if (!ok) break;
@@ -264,8 +286,7 @@ mass_tc_kernel(const MassParams p, const __grid_constant__ CUtensorMap k_map, co
                     if (PASS == 0) load_keys(ring + rp.slot * kTileBytes, i, smem_u32(&sh->full[rp.slot]));
                     else load_rows(ring + rp.slot * kTileBytes, i, smem_u32(&sh->full[rp.slot]));
                 }
-                t += n;
-                mass_advance<PASS>(p, c, n);
+                mass_step<PASS>(p, range, c, n, piece, left);
             }
             // every load that was issued must have landed before the CTA may exit
             const int back = issued < (uint32_t)kSlots ? (int)issued : kSlots;
@@ -287,8 +308,8 @@ mass_tc_kernel(const MassParams p, const __grid_constant__ CUtensorMap k_map, co
             bool ok = true;
             MassCursor c = first;
             int i0, i1;
-            for (long long t = t0; t < t1 && ok; ++o) {
-                const int n = mass_segment<PASS>(p, c, t1 - t, i0, i1);
+            for (; left > 0 && ok; ++o) {
+                const int n = mass_segment<PASS>(p, c, left, i0, i1);
                 const int rbuf = (int)(o % kRes);
                 ok = mass_wait(sh, hdr, &sh->res_full[rbuf], (o / kRes) & 1, 5);
                 for (int i = i0; i < i1 && ok; ++i, ++it, rp.advance(kSlots)) {
@@ -310,8 +331,7 @@ mass_tc_kernel(const MassParams p, const __grid_constant__ CUtensorMap k_map, co
                     tc_commit(smem_u32(&sh->empty[rp.slot]));
                 }
                 if (ok) tc_commit(smem_u32(&sh->res_free[rbuf]));
-                t += n;
-                mass_advance<PASS>(p, c, n);
+                mass_step<PASS>(p, range, c, n, piece, left);
             }
             // all tensor-core work of this CTA must be complete before tensor memory is released
             tc_commit(smem_u32(&sh->drain));
@@ -331,8 +351,8 @@ mass_tc_kernel(const MassParams p, const __grid_constant__ CUtensorMap k_map, co
         bool ok = true;
         MassCursor c = first;
         int i0, i1;
-        for (long long t = t0; t < t1; ++o) {
-            const int n = mass_segment<PASS>(p, c, t1 - t, i0, i1), nv = p.n_visual[c.b], unit = c.b * Hkv + c.hk;
+        for (; left > 0; ++o) {
+            const int n = mass_segment<PASS>(p, c, left, i0, i1), nv = p.n_visual[c.b], unit = c.b * Hkv + c.hk;
             float m = -INFINITY, l = 0.f, acc = 0.f;
             for (int i = i0; i < i1; ++i, ++it) {
                 const int j = it % kAcc;
@@ -432,8 +452,9 @@ mass_tc_kernel(const MassParams p, const __grid_constant__ CUtensorMap k_map, co
                         const float2 v = pt[q * kMassTile + L];
                         if (v.y > 0.f) Ls += v.y * ex2_approx(v.x - M);
                     }
-                    // the row block's partials are numbered from the first CTA that has a part of it
-                    const int slot = (int)blockIdx.x - range.cta_of(t - c.kt);
+                    // the row block's partials are numbered from the first piece that has a part of it
+                    const long long at = ((long long)p.tile_off[c.b] * Hkv + (long long)c.hk * c.n_kt) * p.n_row_blocks + (long long)c.rb * c.n_kt;
+                    const int slot = piece - range.piece_of(at);
                     if (L < TG && c.rb * TG + L < p.r_tot)
                         p.stats[((size_t)unit * p.stat_slots + slot) * p.r_tot + c.rb * TG + L] = make_float2(M, Ls);
                 } else {
@@ -444,9 +465,8 @@ mass_tc_kernel(const MassParams p, const __grid_constant__ CUtensorMap k_map, co
                     if (key < nv) p.colsum[(size_t)c.hk * p.sum_nv + p.offset[c.b] + key] = sum;
                 }
             }
-            t += n;
-            mass_advance<PASS>(p, c, n);
-            if (PASS == 1 && t < t1 && c.b * Hkv + c.hk != unit) {       // another head: all are past their last look at this one's table
+            mass_step<PASS>(p, range, c, n, piece, left);
+            if (PASS == 1 && left > 0 && c.b * Hkv + c.hk != unit) {       // another head: all are past their last look at this one's table
                 const float *src = p.table_log2 + (size_t)(c.b * Hkv + c.hk) * p.r_tot;
                 for (int x = tid - 64; x < tab_entries; x += kMassConsumers) tab[x] = x < p.r_tot ? src[x] : -INFINITY;
                 asm volatile("bar.sync 1, %0;" ::"n"(kMassConsumers) : "memory");
@@ -471,11 +491,11 @@ __global__ void mass_merge_kernel(const MassParams p) {
     const int r = (int)(x % p.r_tot);
     const int unit = (int)(x / p.r_tot);
     const int b = unit / p.n_kv_heads, hk = unit % p.n_kv_heads, n_kt = p.tile_off[b + 1] - p.tile_off[b];
-    int n = 0;                                // CTAs that have a part of the row's block
+    int n = 0;                                // pieces that have a part of the row's block
     if (n_kt > 0) {
-        const MassRange range{(long long)p.tile_off[p.batch] * p.n_kv_heads * p.n_row_blocks, p.stat_grid};
+        const MassRange range{(long long)p.tile_off[p.batch] * p.n_kv_heads * p.n_row_blocks, p.stat_pieces};
         const long long at = ((long long)p.tile_off[b] * p.n_kv_heads + (long long)hk * n_kt) * p.n_row_blocks + (long long)(r / p.rows_per_block) * n_kt;
-        n = range.cta_of(at + n_kt - 1) - range.cta_of(at) + 1;
+        n = range.piece_of(at + n_kt - 1) - range.piece_of(at) + 1;
     }
     const float2 *src = p.stats + (size_t)unit * p.stat_slots * p.r_tot + r;
     float M = -INFINITY;
@@ -554,7 +574,7 @@ __global__ void mass_generic_sum_kernel(const MassParams p) {
 // ---- host side ---------------------------------------------------------------------------------------------------------
 struct MassPlan {
     bool tc;
-    int T, TG, RB, r_tot, stat_grid, sum_grid, stat_slots;
+    int T, TG, RB, r_tot, stat_grid, stat_pieces, sum_grid, stat_slots;
     size_t stats_off, table_off, colsum_off, total;
 };
 
@@ -575,15 +595,17 @@ static MassPlan mass_plan(int batch, const int32_t *n_visual, int l_txt, int n_q
         if (n > longest) longest = n;
     }
     const int units = batch * n_kv_heads;
-    // one wave, one entry of the flat list per CTA at least; a row block's entries lie in at most stat_slots CTAs' ranges
+    // one wave, one entry of the flat list per CTA at least; a row block's entries lie in at most stat_slots pieces
     const long long stat_total = tiles * n_kv_heads * pl.RB, sum_total = tiles * n_kv_heads;
     auto at_most = [](long long n, int room) { return (int)(n < 1 ? 1 : n < room ? n : room); };
     pl.stat_grid = at_most(stat_total, kNumSMs * MassBuffers<0>::kCtasPerSm);
     pl.sum_grid = at_most(sum_total, kNumSMs * MassBuffers<1>::kCtasPerSm);
+    const long long rounds = pl.RB < kMassRoundBlocks ? 1 : (tiles * n_kv_heads * kMassTile * head_dim * 2 + kMassRoundBytes - 1) / kMassRoundBytes;
+    pl.stat_pieces = at_most(stat_total, (int)(rounds < 1 ? 1 : rounds < kMassMaxRounds ? rounds : kMassMaxRounds) * pl.stat_grid);
     pl.stat_slots = 1;
     if (pl.tc && longest > 0) {
-        const long long least = stat_total / pl.stat_grid;            // entries of the shortest range
-        pl.stat_slots = at_most((longest + least - 1) / least + 1, pl.stat_grid);
+        const long long least = stat_total / pl.stat_pieces;          // entries of the shortest piece
+        pl.stat_slots = at_most((longest + least - 1) / least + 1, pl.stat_pieces);
     }
     pl.stats_off = kWsHeaderBytes;
     pl.table_off = align_up(pl.stats_off + (size_t)units * pl.stat_slots * pl.r_tot * sizeof(float2), 256);
@@ -656,12 +678,12 @@ static int32_t launch_mass_tc(MassParams &p, const MassPlan &pl, long long pool_
         attr_set.mark(dev);
     }
     const int units = p.batch * p.n_kv_heads;
-    p.grid = p.stat_grid;
-    HIPPO_CUDA_TRY(launch_mass_dependent(mass_tc_kernel<D, 0>, p.grid, kMassThreads, smem0, s, p, km, qm));
+    p.pieces = p.stat_pieces;
+    HIPPO_CUDA_TRY(launch_mass_dependent(mass_tc_kernel<D, 0>, pl.stat_grid, kMassThreads, smem0, s, p, km, qm));
     const long long rows = (long long)units * p.r_tot;
     HIPPO_CUDA_TRY(launch_mass_dependent(mass_merge_kernel, (rows + 255) / 256, 256, 0, s, p));
-    p.grid = pl.sum_grid;
-    HIPPO_CUDA_TRY(launch_mass_dependent(mass_tc_kernel<D, 1>, p.grid, kMassThreads, smem1, s, p, km, qm));
+    p.pieces = pl.sum_grid;
+    HIPPO_CUDA_TRY(launch_mass_dependent(mass_tc_kernel<D, 1>, pl.sum_grid, kMassThreads, smem1, s, p, km, qm));
     count_launches(3);
     return HIPPO_OK;
 }
@@ -730,7 +752,7 @@ extern "C" int32_t hippo_attention_mass(int32_t batch, const int32_t *n_visual, 
     p.batch = batch; p.l_txt = l_txt; p.n_q_heads = n_q_heads; p.n_kv_heads = kv->n_kv_heads;
     p.group = n_q_heads / kv->n_kv_heads; p.head_dim = kv->head_dim;
     p.t_per_block = pl.T; p.rows_per_block = pl.TG; p.n_row_blocks = pl.RB; p.r_tot = pl.r_tot;
-    p.grid = 0; p.stat_grid = pl.stat_grid; p.stat_slots = pl.stat_slots; p.sum_nv = (int)sum_nv; p.max_pages_per_seq = kv->max_pages_per_seq;
+    p.pieces = 0; p.stat_pieces = pl.stat_pieces; p.stat_slots = pl.stat_slots; p.sum_nv = (int)sum_nv; p.max_pages_per_seq = kv->max_pages_per_seq;
     p.scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)kv->head_dim);
     p.sl2 = p.scale * kMassLog2e;
     p.weight = weight;

@@ -186,3 +186,13 @@ def test_ranges_that_end_anywhere(hb, nv, L, Hq, Hkv, D):
     qs, ks = rand_case(sum(nv) + L, len(nv), L, Hq, Hkv, D, max(max(nv), 1), "bf16")
     got = gpu_mass(hb, qs, ks, nv, "bf16", shuffle_seed=3)
     check(got, oracle_mass(qs, ks, nv), "bf16", "nv %s" % (nv,))
+
+
+@pytest.mark.parametrize("nv,L,Hq,Hkv", [([33000, 0, 500], 200, 56, 8), ([17000, 16500], 180, 64, 8), ([70000], 90, 64, 4)])
+def test_keys_beyond_the_second_level_cache(hb, nv, L, Hq, Hkv):
+    """Above 64 MB of keys that twelve row blocks or more read, the statistics pass goes through its work in rounds: a row's parts come from pieces of several rounds."""
+    rng = np.random.default_rng(sum(nv))
+    q = W.round_to_storage(rng.standard_normal((len(nv), L, Hq, 128)).astype(np.float32), "bf16")
+    k = W.round_to_storage(rng.standard_normal((len(nv), max(nv), Hkv, 128), dtype=np.float32), "bf16")
+    got = gpu_mass(hb, [q], [k], nv, "bf16", shuffle_seed=4)
+    check(got, oracle_mass([q], [k], nv), "bf16", "nv %s" % (nv,))
