@@ -9,10 +9,11 @@
 // uniform lands within ~1e-15 of a boundary.  Three kernels over the vocabulary, chained with programmatic
 // dependent launches (each waits for its predecessor before it reads anything):
 //   stats   per (sequence, logit row, 4096-token chunk): max and sum of exponentials
-//   weigh   per (sequence, chunk): every CTA merges the chunk stats of its sequence and runs the accept tests
-//           itself (a few hundred values; cheaper than a launch of its own), then scans the residual (or bonus)
-//           weights of its chunk in token order and stores the running sum after every 16 tokens
-//   pick    per sequence: locate the chunk, then the 16-token group, then the token where the CDF crosses
+//   weigh   per (sequence, piece: a chunk, or a quarter of one where that still fits one wave): every CTA merges the
+//           chunk stats of its sequence and runs the accept tests itself (a few hundred values; cheaper than a launch
+//           of its own), then scans the residual (or bonus) weights of its piece in token order and stores the
+//           running sum after every 16 tokens
+//   pick    per sequence: locate the piece, then the 16-token group, then the token where the CDF crosses
 //           u * total; only that one group's weights are evaluated again
 #include <math.h>
 
