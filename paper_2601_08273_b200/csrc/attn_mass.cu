@@ -60,7 +60,6 @@ struct MassParams {
     int r_tot;             // l_txt * G packed rows per KV head
     int pieces;            // of this launch's flat list (tensor-core path): CTA c takes c, c + grid, ...
     int stat_pieces;       // of pass 1's
-    int stat_slots;        // partial results that a row block can have from pass 1 (layout of `stats`)
     int sum_nv;            // total visual tokens
     int max_pages_per_seq;
     float sl2;             // softmax scale * log2(e)
@@ -69,7 +68,8 @@ struct MassParams {
     const int32_t *page_table;
     const void *q;
     const void *k_pages;
-    float2 *stats;         // [batch * n_kv_heads][stat_slots][r_tot]: (max in the log2 domain, sum of 2^(x - max))
+    float2 *stats;         // [pieces + row blocks][T * G]: (max in the log2 domain, sum of 2^(x - max)).  Along the flat list either the
+                           // piece or the row block goes on, so that the sum of their numbers names a piece's part of a row block
     float2 *table;         // CUDA-core path: [batch * n_kv_heads][r_tot] (-max, 1 / sum), natural-log domain
     float *table_log2;     // tensor-core path, same memory: [batch * n_kv_heads][r_tot] -(max + log2 sum), log2 domain
     float *colsum;         // [n_kv_heads][sum_nv]
@@ -452,11 +452,8 @@ mass_tc_kernel(const MassParams p, const __grid_constant__ CUtensorMap k_map, co
                         const float2 v = pt[q * kMassTile + L];
                         if (v.y > 0.f) Ls += v.y * ex2_approx(v.x - M);
                     }
-                    // the row block's partials are numbered from the first piece that has a part of it
-                    const long long at = ((long long)p.tile_off[c.b] * Hkv + (long long)c.hk * c.n_kt) * p.n_row_blocks + (long long)c.rb * c.n_kt;
-                    const int slot = piece - range.piece_of(at);
                     if (L < TG && c.rb * TG + L < p.r_tot)
-                        p.stats[((size_t)unit * p.stat_slots + slot) * p.r_tot + c.rb * TG + L] = make_float2(M, Ls);
+                        p.stats[(size_t)(piece + unit * p.n_row_blocks + c.rb) * TG + L] = make_float2(M, Ls);
                 } else {
                     float sum = acc;
 #pragma unroll
@@ -491,18 +488,21 @@ __global__ void mass_merge_kernel(const MassParams p) {
     const int r = (int)(x % p.r_tot);
     const int unit = (int)(x / p.r_tot);
     const int b = unit / p.n_kv_heads, hk = unit % p.n_kv_heads, n_kt = p.tile_off[b + 1] - p.tile_off[b];
+    const int rb = r / p.rows_per_block;
     int n = 0;                                // pieces that have a part of the row's block
+    const float2 *src = p.stats;
     if (n_kt > 0) {
         const MassRange range{(long long)p.tile_off[p.batch] * p.n_kv_heads * p.n_row_blocks, p.stat_pieces};
-        const long long at = ((long long)p.tile_off[b] * p.n_kv_heads + (long long)hk * n_kt) * p.n_row_blocks + (long long)(r / p.rows_per_block) * n_kt;
-        n = range.piece_of(at + n_kt - 1) - range.piece_of(at) + 1;
+        const long long at = ((long long)p.tile_off[b] * p.n_kv_heads + (long long)hk * n_kt) * p.n_row_blocks + (long long)rb * n_kt;
+        const int piece = range.piece_of(at);
+        n = range.piece_of(at + n_kt - 1) - piece + 1;
+        src += (size_t)(piece + unit * p.n_row_blocks + rb) * p.rows_per_block + r % p.rows_per_block;
     }
-    const float2 *src = p.stats + (size_t)unit * p.stat_slots * p.r_tot + r;
     float M = -INFINITY;
-    for (int s = 0; s < n; ++s) M = fmaxf(M, src[(size_t)s * p.r_tot].x);
+    for (int s = 0; s < n; ++s) M = fmaxf(M, src[(size_t)s * p.rows_per_block].x);
     float Lsum = 0.f;
     for (int s = 0; s < n; ++s) {
-        const float2 v = src[(size_t)s * p.r_tot];
+        const float2 v = src[(size_t)s * p.rows_per_block];
         if (v.y > 0.f) Lsum += v.y * exp2f(v.x - M);
     }
     p.table_log2[x] = Lsum > 0.f ? -(M + log2f(Lsum)) : -INFINITY;
@@ -574,7 +574,7 @@ __global__ void mass_generic_sum_kernel(const MassParams p) {
 // ---- host side ---------------------------------------------------------------------------------------------------------
 struct MassPlan {
     bool tc;
-    int T, TG, RB, r_tot, stat_grid, stat_pieces, sum_grid, stat_slots;
+    int T, TG, RB, r_tot, stat_grid, stat_pieces, sum_grid;
     size_t stats_off, table_off, colsum_off, total;
 };
 
@@ -587,28 +587,21 @@ static MassPlan mass_plan(int batch, const int32_t *n_visual, int l_txt, int n_q
     if (pl.T > l_txt) pl.T = l_txt;
     pl.TG = pl.T * G;
     pl.RB = ceil_div(l_txt, pl.T);
-    long long sum_nv = 0, tiles = 0, longest = 0;         // key tiles of all sequences, of the longest
+    long long sum_nv = 0, tiles = 0;
     for (int b = 0; b < batch; ++b) {
-        const long long n = ceil_div(n_visual[b], kMassTile);
         sum_nv += n_visual[b];
-        tiles += n;
-        if (n > longest) longest = n;
+        tiles += ceil_div(n_visual[b], kMassTile);
     }
     const int units = batch * n_kv_heads;
-    // one wave, one entry of the flat list per CTA at least; a row block's entries lie in at most stat_slots pieces
+    // one wave, one entry of the flat list per CTA at least
     const long long stat_total = tiles * n_kv_heads * pl.RB, sum_total = tiles * n_kv_heads;
     auto at_most = [](long long n, int room) { return (int)(n < 1 ? 1 : n < room ? n : room); };
     pl.stat_grid = at_most(stat_total, kNumSMs * MassBuffers<0>::kCtasPerSm);
     pl.sum_grid = at_most(sum_total, kNumSMs * MassBuffers<1>::kCtasPerSm);
     const long long rounds = pl.RB < kMassRoundBlocks ? 1 : (tiles * n_kv_heads * kMassTile * head_dim * 2 + kMassRoundBytes - 1) / kMassRoundBytes;
     pl.stat_pieces = at_most(stat_total, (int)(rounds < 1 ? 1 : rounds < kMassMaxRounds ? rounds : kMassMaxRounds) * pl.stat_grid);
-    pl.stat_slots = 1;
-    if (pl.tc && longest > 0) {
-        const long long least = stat_total / pl.stat_pieces;          // entries of the shortest piece
-        pl.stat_slots = at_most((longest + least - 1) / least + 1, pl.stat_pieces);
-    }
     pl.stats_off = kWsHeaderBytes;
-    pl.table_off = align_up(pl.stats_off + (size_t)units * pl.stat_slots * pl.r_tot * sizeof(float2), 256);
+    pl.table_off = align_up(pl.stats_off + (size_t)(pl.stat_pieces + units * pl.RB) * pl.TG * sizeof(float2), 256);
     pl.colsum_off = align_up(pl.table_off + (size_t)units * pl.r_tot * sizeof(float2), 256);
     pl.total = align_up(pl.colsum_off + (size_t)n_kv_heads * (size_t)sum_nv * sizeof(float), 256);
     return pl;
@@ -752,7 +745,7 @@ extern "C" int32_t hippo_attention_mass(int32_t batch, const int32_t *n_visual, 
     p.batch = batch; p.l_txt = l_txt; p.n_q_heads = n_q_heads; p.n_kv_heads = kv->n_kv_heads;
     p.group = n_q_heads / kv->n_kv_heads; p.head_dim = kv->head_dim;
     p.t_per_block = pl.T; p.rows_per_block = pl.TG; p.n_row_blocks = pl.RB; p.r_tot = pl.r_tot;
-    p.pieces = 0; p.stat_pieces = pl.stat_pieces; p.stat_slots = pl.stat_slots; p.sum_nv = (int)sum_nv; p.max_pages_per_seq = kv->max_pages_per_seq;
+    p.pieces = 0; p.stat_pieces = pl.stat_pieces; p.sum_nv = (int)sum_nv; p.max_pages_per_seq = kv->max_pages_per_seq;
     p.scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)kv->head_dim);
     p.sl2 = p.scale * kMassLog2e;
     p.weight = weight;

@@ -196,3 +196,15 @@ def test_keys_beyond_the_second_level_cache(hb, nv, L, Hq, Hkv):
     k = W.round_to_storage(rng.standard_normal((len(nv), max(nv), Hkv, 128), dtype=np.float32), "bf16")
     got = gpu_mass(hb, [q], [k], nv, "bf16", shuffle_seed=4)
     check(got, oracle_mass([q], [k], nv), "bf16", "nv %s" % (nv,))
+
+
+def test_workspace_of_the_largest_call_serves_the_smaller_ones(hb):
+    """Sizes do not grow when sequences or the text get shorter (pieces, row blocks and tables all shrink with them)."""
+    rng = np.random.default_rng(9)
+    for _ in range(500):
+        hkv, g = [(4, 7), (8, 4), (8, 8), (2, 7)][rng.integers(4)]
+        nv = [int(2 ** x) for x in rng.uniform(5, 16, size=rng.integers(1, 9))]
+        L = int(rng.integers(16, 257))
+        less = [int(rng.integers(0, n + 1)) for n in nv]
+        size = hb.hippo_attention_mass_workspace_bytes(nv, L, hkv * g, hkv, 128, hb.HIPPO_DTYPE_BF16)
+        assert 0 < hb.hippo_attention_mass_workspace_bytes(less, int(rng.integers(1, L + 1)), hkv * g, hkv, 128, hb.HIPPO_DTYPE_BF16) <= size
