@@ -103,9 +103,41 @@ __device__ __forceinline__ bool softmax_bar_or(bool pred) {
 struct Partition {
     long long total;   // tiles over all units
     int grid;          // CTAs
-    __device__ __forceinline__ long long start_of(int c) const { return (long long)c * total / grid; }
-    __device__ __forceinline__ int cta_of(long long t) const { return (int)(((t + 1) * grid - 1) / total); }
+    __device__ __forceinline__ bool narrow() const { return total < (1 << 22); }      // the products fit 32 bits (at most kExtraSlots CTAs)
+    __device__ __forceinline__ long long start_of(int c) const {
+        return narrow() ? (long long)((uint32_t)c * (uint32_t)total / (uint32_t)grid) : (long long)c * total / grid;
+    }
+    __device__ __forceinline__ int cta_of(long long t) const {
+        return narrow() ? (int)((((uint32_t)t + 1) * (uint32_t)grid - 1) / (uint32_t)total) : (int)(((t + 1) * grid - 1) / total);
+    }
 };
+
+// The flat split of a single layer.  A CTA whose range goes over from one unit to the next pays for a second segment (its Q rows, an
+// empty pipeline, one more partial), about as much as eight pages take: where many units share the CTAs, each has that many empty entries
+// ahead of its pages, fewer where a CTA has few pages anyhow.  Us a call without / with them, 8 kv heads: eight ragged sequences of 9,000
+// keys, 48 rows, 60.2 / 57.9 (11 entries 58.4), of 12,000, 24 rows, 72.1 / 70.8.  32 units or fewer mostly run in the other splits, which
+// stay ahead (eight of 10,406, 4 kv heads 39.5, flat 43.9 / 40.1), and with few pages the empty entries cost (one of 20,000 21.2 / 21.6).
+constexpr int kFlatLead = 8, kFlatLeadUnits = 33;
+__host__ __device__ __forceinline__ int flat_lead(long long tiles, int units, int ctas) {
+    if (units < kFlatLeadUnits) return 0;
+    const long long most = tiles / (4 * (long long)ctas);
+    return most < kFlatLead ? (int)most : kFlatLead;
+}
+__device__ __forceinline__ Partition flat_partition(long long tiles, int units, int ctas, int &lead) {
+    lead = flat_lead(tiles, units, ctas);
+    Partition part;
+    part.total = tiles + (long long)lead * units;
+    // no CTA without a tile between two that share a unit (the merge counts the CTAs from the first to the last)
+    part.grid = part.total >= (long long)ctas ? ctas : part.total > 0 ? (int)part.total : 1;
+    return part;
+}
+// First slot and contributors of unit (b, hk) of T tiles, `before` those of a KV head of the sequences ahead; slot = unit + CTA.
+__device__ __forceinline__ int2 flat_slots(const Partition &part, int lead, int Hkv, int b, int hk, int T, int before) {
+    if (T <= 0) return make_int2(0, 0);
+    const long long u0 = (long long)(before + b * lead) * Hkv + (long long)hk * (T + lead) + lead;
+    const int c0 = part.cta_of(u0), c1 = part.cta_of(u0 + T - 1);
+    return make_int2(b * Hkv + hk + c0, c1 - c0 + 1);
+}
 
 // The work of a sequence is counted in 64-key pages: CTA ranges begin and end on page boundaries, and a CTA forms its
 // 128-key tiles from consecutive pairs of its pages (the last tile of a range may hold a single page).
@@ -400,10 +432,12 @@ attn_tc_kernel(const AttnParams p, const __grid_constant__ LayerSetT<NL> set, co
     const uint32_t tmem = sh->tmem_base;
     const uint32_t col_s = 0, col_o = 2 * Rp, col_l = 3 * Rp;   // S^T[0] | S^T[1] | O^T | partial row sums, Rp columns each
 
-    Partition part;
-    part.total = (long long)sh->tile_prefix[B] * Hkv;
-    // the flat split: no CTA without a tile between two that share a unit (the merge counts the CTAs from the first to the last)
-    part.grid = clustered || aligned || part.total >= (long long)gridDim.x ? (int)gridDim.x : part.total > 0 ? (int)part.total : 1;
+    int lead = 0;
+    Partition part{(long long)sh->tile_prefix[B] * Hkv, (int)gridDim.x};
+    if (!clustered && !aligned) {
+        if (!kMulti) part = flat_partition(part.total, U, (int)gridDim.x, lead);
+        else if (part.total < (long long)gridDim.x) part.grid = part.total > 0 ? (int)part.total : 1;
+    }
     int2 *unit_info = reinterpret_cast<int2 *>(p.counters);   // per unit: first slot, number of contributing CTAs
     if (aligned && !small_problem) {
         // CTAs per unit: one each, the others in proportion to the tile counts (largest remainders first)
@@ -441,6 +475,18 @@ attn_tc_kernel(const AttnParams p, const __grid_constant__ LayerSetT<NL> set, co
     }
     // Range [t_begin, t_end) of the flat tile list that CTA number c streams.  In the single-layer kernel c is the CTA's
     // own index; the multi-layer kernel hands CTA x the range of c = (x + layer * rot) mod grid in layer `layer`.
+    // entry v of the list with `lead` empty entries ahead of each unit -> tile
+    auto flat_tile = [&](long long v) -> long long {
+        if (lead == 0) return v;
+        int lo = 0, hi = B;       // largest b whose first unit begins at v or before
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if ((long long)(sh->tile_prefix[mid] + mid * lead) * Hkv <= v) lo = mid; else hi = mid;
+        }
+        const int T = sh->tile_prefix[lo + 1] - sh->tile_prefix[lo];
+        const int off = (int)(v - (long long)(sh->tile_prefix[lo] + lo * lead) * Hkv);
+        return (long long)sh->tile_prefix[lo] * Hkv + (long long)(off / (T + lead)) * T + max(off % (T + lead) - lead, 0);
+    };
     auto range_of = [&](int c, long long &t_begin, long long &t_end) {
         t_begin = t_end = 0;
         if (clustered) {
@@ -466,19 +512,15 @@ attn_tc_kernel(const AttnParams p, const __grid_constant__ LayerSetT<NL> set, co
                 t_end = unit_start + T * (i + 1) / nc;
             }
         } else if (part.total > 0 && c < part.grid) {
-            t_begin = part.start_of(c);
-            t_end = part.start_of(c + 1);
+            t_begin = flat_tile(part.start_of(c));
+            t_end = flat_tile(part.start_of(c + 1));
         }
     };
     // (first slot, number of contributing CTAs) of a unit, as the combine kernel and the merge warp need it
     auto unit_slots = [&](int u) -> int2 {
         if (aligned) return make_int2(sh->cta_base[u], sh->n_cta[u]);
-        const int b = u / Hkv, hk = u % Hkv;
-        const long long T = sh->tile_prefix[b + 1] - sh->tile_prefix[b];
-        if (T <= 0) return make_int2(0, 0);
-        const long long u0 = (long long)sh->tile_prefix[b] * Hkv + hk * T;
-        const int c0 = part.cta_of(u0), c1 = part.cta_of(u0 + T - 1);
-        return make_int2(u + c0, c1 - c0 + 1);     // slot index = unit + cta
+        const int b = u / Hkv;
+        return flat_slots(part, lead, Hkv, b, u % Hkv, sh->tile_prefix[b + 1] - sh->tile_prefix[b], sh->tile_prefix[b]);
     };
     if (!kMulti && !clustered && blockIdx.x == 0)
         for (int u = tid; u < U; u += kThreads) unit_info[u] = unit_slots(u);
@@ -1282,6 +1324,19 @@ __global__ void __launch_bounds__(kCombineThreads) attn_tc_combine_kernel(const 
     }
 }
 
+// First slot and contributors of unit (b, hk) in the flat split over `grid` CTAs, by one warp from the lengths of at most 32 sequences.
+__device__ __forceinline__ int2 flat_slots_warp(const AttnParams &p, int lane, int grid, int b, int hk) {
+    const int kvl = lane < p.batch ? (p.kv_len ? __ldcg(p.kv_len + lane) : p.max_kv_len) : 0;
+    const int nt = lane < p.batch ? seq_tiles(kvl, p.q_len) : 0;
+    int incl = nt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
+    const int T = __shfl_sync(0xffffffffu, nt, b), before = __shfl_sync(0xffffffffu, incl, b) - T;
+    int lead;
+    const Partition part = flat_partition((long long)__shfl_sync(0xffffffffu, incl, 31) * p.n_kv_heads, p.batch * p.n_kv_heads, grid, lead);
+    return flat_slots(part, lead, p.n_kv_heads, b, hk, T, before);
+}
+
 // The same merge where a unit has a handful of contributors: a warp per row, eight rows per CTA.  Up to eight contributors' values of a
 // row are in flight together (lane j fetches (m, l) of contributor j, every lane its output columns of all of them), so a row is one
 // round trip, and the whole grid is resident while the main kernel runs (the kernel above, a CTA per row with five of its warps idle, is
@@ -1307,12 +1362,14 @@ __global__ void __launch_bounds__(kCombineThreads) attn_tc_combine_rows_kernel(c
         }
         __syncthreads();
     }
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int row = blockIdx.x * (kCombineThreads / 32) + w;
-    if (row >= n_rows) return;
     const int h = row % p.n_q_heads, t = (row / p.n_q_heads) % p.q_len, b = row / (p.n_q_heads * p.q_len);
     const int unit = b * Hkv + h / G, r = t * G + (h % G);
-    const int2 info = main_grid > 0 ? s_info[unit] : reinterpret_cast<const int2 *>(p.counters)[unit];   // first slot, contributors
+    int2 info = make_int2(0, 0);
+    if (main_grid < 0 && row < n_rows) info = flat_slots_warp(p, lane, -main_grid, b, h / G);     // also while the main kernel runs
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (row >= n_rows) return;
+    if (main_grid >= 0) info = main_grid > 0 ? s_info[unit] : reinterpret_cast<const int2 *>(p.counters)[unit];   // first slot, contributors
     const int n = info.y;
     if (n == 1) return;
     const size_t slot_floats = slot_float_count(R, D);
@@ -1475,7 +1532,10 @@ static int choose_split(const AttnParams &p, int rows_padded, const int *max_act
     const float g = groups <= 2 ? 0.f : groups - 2.f, u16 = units < 16 ? units : 16, u32 = units < 32 ? units : 32;
     const int grid = split_grid(p, kNumSMs), even = aligned_longest(p, grid);
     int best = kFlat;
+    const int lead = flat_lead(total_pages, units, grid);
     float best_us = 10.2f + 0.385f * g + (0.703f + 0.037f * g) * (float)((total_pages + grid - 1) / grid) + (0.296f + 0.106f * g) * u16;
+    if (units >= kFlatLeadUnits)       // refitted with the empty entries
+        best_us = 11.6f + 1.4f * g + 0.70f * (float)(total_pages + (long long)lead * units) / grid + 0.6f * (kFlatLead - lead);
     if (even > 0) {
         const float us = 11.6f + 1.32f * g + (0.69f + 0.034f * g) * even + (0.027f - 0.0154f * g) * u32;
         if (us < best_us) { best = kAligned; best_us = us; }
@@ -1576,11 +1636,13 @@ static int32_t launch_tc(const AttnParams &p, int grid, cudaStream_t stream) {
     const int n_rows = p.batch * p.q_len * p.n_q_heads;
     cfg.blockDim = dim3(kCombineThreads);
     cfg.dynamicSmemBytes = 0;
-    // unit-aligned split by one warp (see the kernel): the combine kernel derives the slot table itself
-    const int derive = (mode == kAligned && units <= grid && units <= 32) ? grid : 0;
+    // The combine kernel derives the slot table itself: of a unit-aligned split worked out by one warp (see the kernel); a warp per row also of
+    // a flat split, with a lane per sequence.
+    const bool flat = mode == kFlat || units > grid || units > kMaxAlignedUnits;
+    const int derive = !flat && units <= 32 ? grid : 0;
     if (grid <= 8 * units) {             // one round trip per row
         cfg.gridDim = dim3((unsigned)ceil_div(n_rows, kCombineThreads / 32));
-        HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_combine_rows_kernel<D>, p, derive, n_rows));
+        HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_combine_rows_kernel<D>, p, flat && p.batch <= 32 ? -grid : derive, n_rows));
     } else {
         cfg.gridDim = dim3((unsigned)n_rows);
         HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_combine_kernel<D>, p, derive));
