@@ -394,8 +394,9 @@ attn_tc_kernel(const AttnParams p, const __grid_constant__ LayerSetT<NL> set, co
         // A single-layer call mostly becomes resident while its predecessor ends.  Warp 0 uses that time to work out the tables from the
         // lengths as they stand (eight ragged sequences of 10,406 keys 41.4 -> 39.4 us a call, with the earlier launch that the combine kernel
         // allows) and may ask L2 for the first pages.  The lengths are looked up again after the wait; page ids, which nothing but the
-        // prefetch uses, count only inside the pool.
-        const bool peek = !kMulti && small_problem;
+        // prefetch uses, count only inside the pool.  Not in clusters, whose tables are a prefix sum: 13.9 us a call, 14.1 with the look
+        // ahead (one sequence of 4,000 keys, 8 kv heads, 32 rows).
+        const bool peek = !kMulti && small_problem && !clustered;
         int peeked = 0;
         if (peek && warp == 0) {
             if (lane < B) peeked = p.kv_len ? min(max(tc_peek(p.kv_len + lane), 0), p.max_kv_len) : p.max_kv_len;
@@ -1527,8 +1528,6 @@ static int choose_split(const AttnParams &p, int rows_padded, const int *max_act
     int pages;
     long long total_pages;
     plan_pages(p, pages, total_pages);
-    // a page or two per CTA: one sequence of 1,500 keys, 4 kv heads, 28 rows 11.7 / 10.6 / 10.2, of 4,000, 63 rows 15.6 / 15.9 / 14.7
-    if (total_pages <= 256) return kFlat;
     const float g = groups <= 2 ? 0.f : groups - 2.f, u16 = units < 16 ? units : 16, u32 = units < 32 ? units : 32;
     const int grid = split_grid(p, kNumSMs), even = aligned_longest(p, grid);
     int best = kFlat;
@@ -1536,14 +1535,21 @@ static int choose_split(const AttnParams &p, int rows_padded, const int *max_act
     float best_us = 10.2f + 0.385f * g + (0.703f + 0.037f * g) * (float)((total_pages + grid - 1) / grid) + (0.296f + 0.106f * g) * u16;
     if (units >= kFlatLeadUnits)       // refitted with the empty entries
         best_us = 11.6f + 1.4f * g + 0.70f * (float)(total_pages + (long long)lead * units) / grid + 0.6f * (kFlatLead - lead);
+    // Few units, from one sequence of 1,000 to 7,000 keys with 24 to 72 rows: many partials per row cost the split modes more, clusters of at
+    // most eight take less, larger ones more than the lines say.  28 rows, 4 kv heads, 2,000 keys: cluster of 8 / of 16 / aligned / flat
+    // 10.9 / 11.8 / 12.6 / 13.0; 5,500 keys 15.6 / 14.2 / 15.5 / 15.0; 48 rows, 8 kv heads, 1,000 keys 11.9 / - / 14.4 / 13.6.
+    const bool few = units <= 8;
+    if (few) best_us += units <= 4 ? 1.2f : 2.5f;
     if (even > 0) {
-        const float us = 11.6f + 1.32f * g + (0.69f + 0.034f * g) * even + (0.027f - 0.0154f * g) * u32;
+        const float us = 11.6f + 1.32f * g + (0.69f + 0.034f * g) * even + (0.027f - 0.0154f * g) * u32 + (units <= 4 ? 1.1f : few ? 0.5f : 0.f);
         if (us < best_us) { best = kAligned; best_us = us; }
     }
-    // a cluster of more than eight needs most of a GPC, and only six of them can be counted on to hold one
-    for (int cs = 2; cs <= (units <= 6 ? 16 : 8) && 2 * cs <= pages + 1; ++cs) {
+    // A cluster of more than eight needs most of a GPC, and only six of them can be counted on to hold one; sizes between eight and sixteen
+    // were slower than both (42 rows, 4 kv heads, 3,000 keys, clusters of 8 / 10 / 12 / 14 / 16: 13.5 / 17.3 / 15.7 / 15.1 / 14.5).
+    for (int cs = 2; cs <= (units <= 6 ? 16 : 8) && 2 * cs <= pages + 1; cs = cs == 8 ? 16 : cs + 1) {
         if (units > max_active[cs]) continue;
-        const float us = 9.6f + 1.0f * g + (0.564f + 0.045f * g) * ceil_div(pages, cs) + (0.079f + 0.029f * g) * u32;
+        const float us = 9.6f + 1.0f * g + (0.564f + 0.045f * g) * ceil_div(pages, cs) + (0.079f + 0.029f * g) * u32 +
+                         (cs > 8 ? 0.8f : few ? -1.1f : 0.f);
         if (us < best_us) { best = cs; best_us = us; }
     }
     return best;
