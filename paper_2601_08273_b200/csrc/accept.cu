@@ -671,15 +671,18 @@ static int32_t launch_accept_chain(AcceptParams p, cudaStream_t s) {
 // One launch: the grid is at most what the device keeps resident at once (the CTAs wait for one another between the
 // steps), and never more than the first step has items.
 static int32_t launch_accept_fused(const AcceptParams &p, WsHeader *hdr, cudaStream_t s) {
+    // With the table of the exponentials the kernel's own arrays and these are more than the 48 KB that need no leave.
+    constexpr int kMostDynamic = 40 * 1024;
     const size_t smem = (size_t)p.n_chunks * sizeof(double);
-    if (smem > 40 * 1024) return launch_accept_chain(p, s);
+    if (smem > kMostDynamic) return launch_accept_chain(p, s);
     static std::atomic<int> resident[kMaxDevices];
     int dev = -1;
     HIPPO_CUDA_TRY(cudaGetDevice(&dev));
     int cap = (dev >= 0 && dev < kMaxDevices) ? resident[dev].load(std::memory_order_relaxed) : 0;
     if (cap == 0) {
         int per_sm = 0, sms = 0;
-        HIPPO_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, accept_fused_kernel, kAccThreads, 40 * 1024));
+        HIPPO_CUDA_TRY(cudaFuncSetAttribute(accept_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostDynamic));
+        HIPPO_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, accept_fused_kernel, kAccThreads, kMostDynamic));
         HIPPO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         cap = per_sm * sms;
         if (cap < 1) return launch_accept_chain(p, s);

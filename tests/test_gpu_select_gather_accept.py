@@ -570,9 +570,11 @@ def check_accept(hb, inp, what, forgiven_allowed=0):
     assert np.all(ma >= 0), what
     args = [dev(inp[k]) for k in ("target_logits", "draft_logits", "draft_tokens", "u_accept", "u_resample")]
     # both launch forms of the sampling acceptance (one kernel / three chained kernels), and the library's own choice
-    for form, flag in (("chain", hb.HIPPO_ACCEPT_THREE_LAUNCHES), ("one launch", hb.HIPPO_ACCEPT_ONE_LAUNCH), ("auto", 0)):
+    for form, flag, kernels in (("chain", hb.HIPPO_ACCEPT_THREE_LAUNCHES, 3), ("one launch", hb.HIPPO_ACCEPT_ONE_LAUNCH, 1), ("auto", 0, None)):
         ws = hb.new_workspace(hb.hippo_accept_workspace_bytes(*rout.shape[:1], rout.shape[1] - 1, inp["target_logits"].shape[2]))
+        before = hb.hippo_launch_count()
         n, out = hb.hippo_accept(*args, mode=hb.HIPPO_ACCEPT_SAMPLE | flag, workspace=ws)
+        assert kernels is None or hb.hippo_launch_count() - before == kernels, "%s (%s): not the form that was asked for" % (what, form)
         torch.cuda.synchronize()
         assert hb.hippo_workspace_status(ws) == hb.HIPPO_OK
         n, out = host(n), host(out)
@@ -665,9 +667,11 @@ def test_a_vocabulary_chunk_of_nan_stays_out_of_its_rows_sum(hb, batch):
     for fill in (np.nan, -np.inf):
         tl = c["target_logits"].copy()
         tl[:, 1, 4096:8192] = fill
-        for flag in (hb.HIPPO_ACCEPT_THREE_LAUNCHES, hb.HIPPO_ACCEPT_ONE_LAUNCH):
+        for flag, kernels in ((hb.HIPPO_ACCEPT_THREE_LAUNCHES, 3), (hb.HIPPO_ACCEPT_ONE_LAUNCH, 1)):
+            before = hb.hippo_launch_count()
             n, out = hb.hippo_accept(dev(tl), dev(c["draft_logits"]), dev(x), dev(c["u_accept"]), dev(c["u_resample"]),
                                      mode=hb.HIPPO_ACCEPT_SAMPLE | flag)
+            assert hb.hippo_launch_count() - before == kernels
             res.append((host(n).tolist(), host(out).tolist()))
     assert all(r == res[-1] for r in res)
     assert max(res[-1][0]) >= 2                          # the row with the NaN was tested and passed somewhere
