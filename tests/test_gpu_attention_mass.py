@@ -4,7 +4,7 @@ import pytest
 import torch
 
 import oracle
-from gpu_util import dev, host, paged_cache
+from gpu_util import captured_kernels, dev, host, paged_cache
 from paper_2601_08273_b200 import workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -186,6 +186,24 @@ def test_ranges_that_end_anywhere(hb, nv, L, Hq, Hkv, D):
     qs, ks = rand_case(sum(nv) + L, len(nv), L, Hq, Hkv, D, max(max(nv), 1), "bf16")
     got = gpu_mass(hb, qs, ks, nv, "bf16", shuffle_seed=3)
     check(got, oracle_mass(qs, ks, nv), "bf16", "nv %s" % (nv,))
+
+
+@pytest.mark.parametrize("nv,L,Hq,Hkv,D,threads", [([13063], 16, 14, 2, 64, 512),      # 103 parts a row
+                                                   ([40000], 3, 8, 1, 64, 512),        # 296, more than the threads keep in registers
+                                                   ([3840], 16, 32, 8, 128, 256),      # 30, the most for four warps
+                                                   ([3960], 16, 32, 8, 128, 512),      # and one more
+                                                   ([9000] + [1] * 40, 5, 4, 2, 64, 256),    # two on average, a few dozen of one sequence
+                                                   ([300], 256, 8, 8, 64, 256)])
+def test_parts_of_a_row_are_shared_by_warps(hb, nv, L, Hq, Hkv, D, threads):
+    """The statistics of a row come from as many pieces as its row block lies in: one, or all of them."""
+    qs, ks = rand_case(L, len(nv), L, Hq, Hkv, D, max(nv), "bf16")
+    got = gpu_mass(hb, qs, ks, nv, "bf16", shuffle_seed=3)
+    check(got, oracle_mass(qs, ks, nv), "bf16", "nv %s" % (nv,))
+    kv, _, _ = paged_cache(hb, ks[0], ks[0], nv, "bf16", shuffle_seed=3)
+    mass, q = torch.zeros(sum(nv), dtype=torch.float32, device="cuda"), dev(qs[0], "bf16")
+    ws = hb.new_workspace(hb.hippo_attention_mass_workspace_bytes(nv, L, Hq, Hkv, D, hb.HIPPO_DTYPE_BF16))
+    merge = [k for k in captured_kernels(lambda: hb.hippo_attention_mass(q, kv, nv, 1.0, mass, workspace=ws)) if "mass_merge" in k[0]]
+    assert [k[2] for k in merge] == [threads]
 
 
 @pytest.mark.parametrize("nv,L,Hq,Hkv", [([33000, 0, 500], 200, 56, 8), ([17000, 16500], 180, 64, 8), ([70000], 90, 64, 4)])
