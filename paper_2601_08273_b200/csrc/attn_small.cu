@@ -129,6 +129,10 @@ __device__ __noinline__ void attn_small_redo(const AttnParams &p, int b, int hk,
     }
 }
 
+// The draft's pruned cache is read again by every token: kept in L2 beside a verification pass that streams through it (28 layers hold 11 MB
+// of 126 at 758 keys, 51 at the 32k step's 3,537; beside 104 SMs of verification that step takes 1,425 us with either policy).
+__device__ __forceinline__ uint64_t small_policy(const AttnParams &p) { return p.kv_resident ? l2_policy_evict_last() : l2_policy_evict_first(); }
+
 // Ahead of the wait for the predecessor in the stream: asks L2 for what the warp is going to read.  These are hints and nothing else: a
 // line that the predecessor writes later is current in L2 all the same, and the values used here (length, page ids) are looked up again
 // after the wait.  They may be stale or not yet written, so they count only inside their bounds.  us per call in a chain of 28, cold
@@ -154,7 +158,7 @@ __device__ __forceinline__ void sm_prefetch(const AttnParams &p, int b, int hk, 
     asm volatile("cp.async.bulk.prefetch.L2.global.L2::cache_hint [%0], %1, %2;" ::"l"(src), "r"((uint32_t)(kSmBlock * D * 2)), "l"(pol) : "memory");
 }
 
-template <int D, int NT>   // head size; groups of eight packed rows
+template <int D, int NT, bool kPrefetch>   // head size; groups of eight packed rows; see small_prefetch
 __global__ void __launch_bounds__(D == 64 ? 512 : 256) attn_small_kernel(const __grid_constant__ AttnParams p, const int cluster_size) {
     using S = SmallSmem<D, NT>;
     constexpr int kKV4 = D / 32;          // 16-byte loads of a lane per key of the score operand
@@ -170,16 +174,20 @@ __global__ void __launch_bounds__(D == 64 ? 512 : 256) attn_small_kernel(const _
     const int first = warp * cluster_size + rank;
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");     // this CTA runs: its peers may push into its memory
     const int max_blocks = (p.max_kv_len + kSmBlock - 1) / kSmBlock;
-    // the draft's pruned cache is read again by every token: kept in L2 beside a verification pass that streams through it (28 layers
-    // hold 13 - 25 MB of 126; beside 104 SMs of verification the 32k step takes 1,425 us with either policy)
-    const uint64_t pol = p.kv_resident ? l2_policy_evict_last() : l2_policy_evict_first();
+    // Where the policy and the query rows are worked out decides the order that the compiler gives a step's loads: with up to eight rows of
+    // head size 128, ahead of the wait 178 registers, 4.55 us for 760 keys, 2 kv heads, in L2; after it 221 registers, 4.27 us.  Where the
+    // step is prefetched ahead is better (1,500 keys, 8 kv heads 5.37, 5.57 after), and with head size 64 or more rows.
+    constexpr bool kAhead = D == 64 || NT == 2 || kPrefetch;
+    const uint64_t pol_ahead = kAhead ? small_policy(p) : 0;
     const __nv_bfloat16 *q_rows[NT];                            // this lane's part of its query rows
+    if (kAhead) {
 #pragma unroll
-    for (int n = 0; n < NT; ++n) {
-        const int r = g + 8 * n, tq = r / G, gq = r - tq * G;
-        q_rows[n] = (const __nv_bfloat16 *)p.q + (((size_t)b * p.q_len + tq) * p.n_q_heads + hk * G + gq) * D + t * 8;
+        for (int n = 0; n < NT; ++n) {
+            const int r = g + 8 * n, tq = r / G, gq = r - tq * G;
+            q_rows[n] = (const __nv_bfloat16 *)p.q + (((size_t)b * p.q_len + tq) * p.n_q_heads + hk * G + gq) * D + t * 8;
+        }
     }
-    sm_prefetch<D>(p, b, hk, first, stride, rank == 0 && warp == 0, max_blocks, pol);
+    if (kPrefetch) sm_prefetch<D>(p, b, hk, first, stride, rank == 0 && warp == 0, max_blocks, pol_ahead);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
@@ -187,13 +195,20 @@ __global__ void __launch_bounds__(D == 64 ? 512 : 256) attn_small_kernel(const _
     if (kvl < p.q_len) kvl = 0;                                 // skipped: its row of the page table may hold anything
 
     // query rows as A operand; the contraction order is the one of the keys' loads
+    if (!kAhead) {
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            const int r = g + 8 * n, tq = r / G, gq = r - tq * G;
+            q_rows[n] = (const __nv_bfloat16 *)p.q + (((size_t)b * p.q_len + tq) * p.n_q_heads + hk * G + gq) * D + t * 8;
+        }
+    }
     uint4 qr[NT][kKV4];
 #pragma unroll
     for (int n = 0; n < NT; ++n)
 #pragma unroll
         for (int j = 0; j < kKV4; ++j) qr[n][j] = g + 8 * n < R ? sm_ldg(q_rows[n] + j * 32) : make_uint4(0, 0, 0, 0);
     const float sl2 = p.scale * kSmLog2e;
-
+    const uint64_t pol = kAhead ? pol_ahead : small_policy(p);
     float o[NT][kDT][4], m[NT], l[NT];
 #pragma unroll
     for (int n = 0; n < NT; ++n) {
@@ -391,9 +406,10 @@ template <int D, int NT>
 static int32_t small_setup(int &dev) {
     static PerDeviceOnce attr_set;
     if (attr_set.needed(dev)) {
-        HIPPO_CUDA_TRY(cudaFuncSetAttribute(attn_small_kernel<D, NT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        HIPPO_CUDA_TRY(cudaFuncSetAttribute(attn_small_kernel<D, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)SmallSmem<D, NT>::bytes(kSmMaxWarps)));
+        for (auto *kernel : {attn_small_kernel<D, NT, false>, attn_small_kernel<D, NT, true>}) {
+            HIPPO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+            HIPPO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SmallSmem<D, NT>::bytes(kSmMaxWarps)));
+        }
         attr_set.mark(dev);
     }
     return HIPPO_OK;
@@ -419,7 +435,7 @@ static int small_room(int warps, int cs) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, attn_small_kernel<D, NT>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); n = 1 << 30; }
+        if (cudaOccupancyMaxActiveClusters(&n, attn_small_kernel<D, NT, true>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); n = 1 << 30; }
         room.store(n < (1 << 30) ? n + 1 : 1 << 30, std::memory_order_relaxed);
     }
     return room.load(std::memory_order_relaxed) - 1;
@@ -478,6 +494,17 @@ bool attn_small_beats_layers(const AttnParams &p, int dtype, int max_ctas) {
     return plan.steps == 1 && (max_ctas <= 0 || p.batch * p.n_kv_heads * plan.cluster <= max_ctas);
 }
 
+// Whether the kernel asks ahead of its wait for what it is going to read (sm_prefetch).  us per call in a chain of 28, without / with, keys
+// x kv heads; "cold": the caches of the chain are not in L2 when it begins.  Head size 64: 760 x 4 cold 4.11 / 3.80, in L2 3.52 / 3.47;
+// 3,500 x 2 cold 4.83 / 4.17; 9,000 x 8 9.38 / 8.17.  Head size 128, up to eight rows: 1,500 x 8 5.99 / 5.35, 1,500 x 4 4.77 / 4.76; a smaller
+// call of a chain that stays in L2 loses, 340 x 8 4.20 / 4.32 and 760 x 2 4.27 / 4.40, against cold 5.07 / 4.76 and 4.85 / 4.70, so the line lies
+// where the two are even.  Above, the call before has the memory busy to its end: eight sequences of 3,500 keys x 8, head size 64, 14.4 / 16.4;
+// 32 of 1,500 x 4 13.7 / 14.1.
+static bool small_prefetch(const AttnParams &p) {
+    const long long bytes = (long long)p.batch * p.n_kv_heads * p.max_kv_len * p.head_dim * 4;
+    return bytes <= (40 << 20) && (p.head_dim == 64 || p.rows > 8 || bytes >= (1 << 20));
+}
+
 template <int D, int NT>
 static int32_t launch_small(const AttnParams &p, cudaStream_t stream) {
     int dev;
@@ -502,7 +529,7 @@ static int32_t launch_small(const AttnParams &p, cudaStream_t stream) {
     for (;;) {
         attr[1].val.clusterDim.x = (unsigned)cs;
         cfg.gridDim = dim3((unsigned)(units * cs));
-        const cudaError_t e = cudaLaunchKernelEx(&cfg, attn_small_kernel<D, NT>, p, cs);
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, small_prefetch(p) ? attn_small_kernel<D, NT, true> : attn_small_kernel<D, NT, false>, p, cs);
         if (e == cudaSuccess) break;
         (void)cudaGetLastError();
         if (cs <= 8) return cuda_fail(e, "attention (small) launch");
