@@ -321,7 +321,8 @@ __device__ __forceinline__ void prefetch_first_pages(const AttnParams &p, const 
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"((uint32_t)(kPageSize * D * 2)) : "memory");
 }
 
-template <int D, int NL>
+// clustered: one cluster per unit, merge through shared memory
+template <int D, int NL, bool clustered = false>
 __global__ void __launch_bounds__(NL == 1 ? kTcThreads : kTcThreads + 32, 1)
 attn_tc_kernel(const AttnParams p, const __grid_constant__ LayerSetT<NL> set, const MultiCtl mc,
                const int Rp, const int n_slots, const int tmem_cols, const int cluster_size, const int spare_cols) {
@@ -347,8 +348,7 @@ attn_tc_kernel(const AttnParams p, const __grid_constant__ LayerSetT<NL> set, co
 
     // ---- set-up: barriers, tile prefix, CTA split, tensor memory
     const int U = B * Hkv;
-    const bool clustered = cluster_size > 1;                  // one cluster per unit, merge through shared memory
-    const bool aligned = cluster_size == 0 && U <= (int)gridDim.x && U <= kMaxAlignedUnits;
+    const bool aligned = !clustered && cluster_size == 0 && U <= (int)gridDim.x && U <= kMaxAlignedUnits;
     const bool small_problem = U <= 32;                       // tile prefix and CTA split by warp 0 alone, no block barriers
     {
         // one barrier per thread of warps 1..: [0, n_slots) full, [n_slots, 2 n_slots) empty, then the fixed ones
@@ -1586,7 +1586,8 @@ static int32_t launch_tc(const AttnParams &p, int grid, cudaStream_t stream) {
     int dev;
     if (attr_set.needed(dev)) {
         HIPPO_CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<D, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-        HIPPO_CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<D, 1>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        HIPPO_CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<D, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        HIPPO_CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<D, 1, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         attr_set.mark(dev);
     }
     const int units = p.batch * p.n_kv_heads;
@@ -1603,7 +1604,7 @@ static int32_t launch_tc(const AttnParams &p, int grid, cudaStream_t stream) {
             q.gridDim = dim3((unsigned)(c * kNumSMs)); q.blockDim = dim3(kTcThreads); q.dynamicSmemBytes = (size_t)plan.total;
             q.attrs = qa; q.numAttrs = 1;
             int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, attn_tc_kernel<D, 1>, &q) != cudaSuccess) { n = 0; (void)cudaGetLastError(); }
+            if (cudaOccupancyMaxActiveClusters(&n, attn_tc_kernel<D, 1, true>, &q) != cudaSuccess) { n = 0; (void)cudaGetLastError(); }
             max_active[plan.slots][c] = n;
         }
         have_active[plan.slots].store(true, std::memory_order_release);
@@ -1628,7 +1629,7 @@ static int32_t launch_tc(const AttnParams &p, int grid, cudaStream_t stream) {
         cfg.numAttrs = 2;
         cfg.gridDim = dim3((unsigned)(units * split));
         if (slot_float_count(p.rows, D) * sizeof(float) <= (size_t)plan.slots * kBlockN * D * 2 &&
-            cudaLaunchKernelEx(&cfg, attn_tc_kernel<D, 1>, p, set, mc, sh.Rp, plan.slots, sh.tmem_cols, split, sh.spare_cols) == cudaSuccess) {
+            cudaLaunchKernelEx(&cfg, attn_tc_kernel<D, 1, true>, p, set, mc, sh.Rp, plan.slots, sh.tmem_cols, split, sh.spare_cols) == cudaSuccess) {
             count_launches(1);
             return HIPPO_OK;
         }
