@@ -321,8 +321,9 @@ __device__ __forceinline__ void prefetch_first_pages(const AttnParams &p, const 
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"((uint32_t)(kPageSize * D * 2)) : "memory");
 }
 
-// clustered: one cluster per unit, merge through shared memory
-template <int D, int NL, bool clustered = false>
+// The forms of a single-layer call, an instantiation each; the multi-layer kernel tells the unit-aligned and the flat split by its grid.
+constexpr int kAligned = 0, kClustered = 1, kFlat = 2, kByGrid = 3;
+template <int D, int NL, int kForm>
 __global__ void __launch_bounds__(NL == 1 ? kTcThreads : kTcThreads + 32, 1)
 attn_tc_kernel(const AttnParams p, const __grid_constant__ LayerSetT<NL> set, const MultiCtl mc,
                const int Rp, const int n_slots, const int tmem_cols, const int cluster_size, const int spare_cols) {
@@ -348,7 +349,8 @@ attn_tc_kernel(const AttnParams p, const __grid_constant__ LayerSetT<NL> set, co
 
     // ---- set-up: barriers, tile prefix, CTA split, tensor memory
     const int U = B * Hkv;
-    const bool aligned = !clustered && cluster_size == 0 && U <= (int)gridDim.x && U <= kMaxAlignedUnits;
+    constexpr bool clustered = kForm == kClustered;           // one cluster per unit, merge through shared memory
+    const bool aligned = kForm == kAligned || (kForm == kByGrid && U <= (int)gridDim.x && U <= kMaxAlignedUnits);
     const bool small_problem = U <= 32;                       // tile prefix and CTA split by warp 0 alone, no block barriers
     {
         // one barrier per thread of warps 1..: [0, n_slots) full, [n_slots, 2 n_slots) empty, then the fixed ones
@@ -436,7 +438,7 @@ attn_tc_kernel(const AttnParams p, const __grid_constant__ LayerSetT<NL> set, co
     int lead = 0;
     Partition part{(long long)sh->tile_prefix[B] * Hkv, (int)gridDim.x};
     if (!clustered && !aligned) {
-        if (!kMulti) part = flat_partition(part.total, U, (int)gridDim.x, lead);
+        if (kForm == kFlat) part = flat_partition(part.total, U, (int)gridDim.x, lead);
         else if (part.total < (long long)gridDim.x) part.grid = part.total > 0 ? (int)part.total : 1;
     }
     int2 *unit_info = reinterpret_cast<int2 *>(p.counters);   // per unit: first slot, number of contributing CTAs
@@ -1515,15 +1517,14 @@ static int aligned_longest(const AttnParams &p, int grid) {
     return longest;
 }
 
-// How a single-layer call is split: > 1 one cluster of so many CTAs per unit, kAligned or kFlat.  The times, in us of a call in a chain of
+// How a single-layer call is split: kAligned, kFlat, or kClustered with the CTAs per unit in `cluster`.  The times, in us of a call in a chain of
 // them, are fitted to 75 shapes (head size 128, 1 to 64 units, 14 to 72 packed rows; 5 to 8 % off, the mean loss of the choice 1.4 %): a
 // constant, the pages of the longest CTA (the average for the flat split), the units, and the groups of 16 rows beyond 32 in each.
 // Measured, clusters / aligned / flat: eight ragged sequences of 10,406 keys, 4 kv heads, 42 rows 45.9 / 40.2 / 44.1; of 12,000, 8 kv heads,
 // 24 rows 70.3 / 80.9 / 72.5; of 9,000, 8 kv heads, 48 rows 65.2 / 67.2 / 60.5; four of 13,000, 8 kv heads, 24 rows 42.6 / 45.0 / 45.4, of 3,000
 // with 72 rows 26.4 / 24.0 / 29.8; one of 3,000, 48 rows 14.2 / 15.8 / 18.4, of 9,000, 4 kv heads, 28 rows 16.7 / 15.4 / 15.0.  Head size 64,
 // eight of 10,406, 42 rows: 38.8 / 34.2 / 37.2.
-constexpr int kAligned = 0, kFlat = -1;
-static int choose_split(const AttnParams &p, int rows_padded, const int *max_active) {
+static int choose_split(const AttnParams &p, int rows_padded, const int *max_active, int &cluster) {
     const int units = p.batch * p.n_kv_heads, groups = rows_padded / 16;
     int pages;
     long long total_pages;
@@ -1550,7 +1551,7 @@ static int choose_split(const AttnParams &p, int rows_padded, const int *max_act
         if (units > max_active[cs]) continue;
         const float us = 9.6f + 1.0f * g + (0.564f + 0.045f * g) * ceil_div(pages, cs) + (0.079f + 0.029f * g) * u32 +
                          (cs > 8 ? 0.8f : few ? -1.1f : 0.f);
-        if (us < best_us) { best = cs; best_us = us; }
+        if (us < best_us) { best = kClustered; cluster = cs; best_us = us; }
     }
     return best;
 }
@@ -1585,9 +1586,9 @@ static int32_t launch_tc(const AttnParams &p, int grid, cudaStream_t stream) {
     static PerDeviceOnce attr_set;
     int dev;
     if (attr_set.needed(dev)) {
-        HIPPO_CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<D, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-        HIPPO_CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<D, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-        HIPPO_CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<D, 1, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        for (auto *kernel : {attn_tc_kernel<D, 1, kAligned>, attn_tc_kernel<D, 1, kClustered>, attn_tc_kernel<D, 1, kFlat>})
+            HIPPO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        HIPPO_CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<D, 1, kClustered>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         attr_set.mark(dev);
     }
     const int units = p.batch * p.n_kv_heads;
@@ -1604,12 +1605,13 @@ static int32_t launch_tc(const AttnParams &p, int grid, cudaStream_t stream) {
             q.gridDim = dim3((unsigned)(c * kNumSMs)); q.blockDim = dim3(kTcThreads); q.dynamicSmemBytes = (size_t)plan.total;
             q.attrs = qa; q.numAttrs = 1;
             int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, attn_tc_kernel<D, 1, true>, &q) != cudaSuccess) { n = 0; (void)cudaGetLastError(); }
+            if (cudaOccupancyMaxActiveClusters(&n, attn_tc_kernel<D, 1, kClustered>, &q) != cudaSuccess) { n = 0; (void)cudaGetLastError(); }
             max_active[plan.slots][c] = n;
         }
         have_active[plan.slots].store(true, std::memory_order_release);
     }
-    const int split = p.num_splits > 0 ? kAligned : choose_split(p, sh.Rp, max_active[plan.slots]);
+    int cluster = 0;
+    const int form = p.num_splits > 0 ? kAligned : choose_split(p, sh.Rp, max_active[plan.slots], cluster);
     // Both kernels are launched with programmatic stream serialization and wait (griddepcontrol.wait) before they
     // touch memory, so stream order is kept while launch latency overlaps the previous kernel's tail.
     cudaLaunchAttribute attr[2];
@@ -1620,16 +1622,16 @@ static int32_t launch_tc(const AttnParams &p, int grid, cudaStream_t stream) {
     cfg.dynamicSmemBytes = (size_t)plan.total;
     cfg.stream = stream;
     cfg.attrs = attr;
-    if (split > 1) {
+    if (form == kClustered) {
         // one cluster per unit; the partial of a CTA (m, l, O) must fit in its ring memory
         attr[1].id = cudaLaunchAttributeClusterDimension;
-        attr[1].val.clusterDim.x = (unsigned)split;
+        attr[1].val.clusterDim.x = (unsigned)cluster;
         attr[1].val.clusterDim.y = 1;
         attr[1].val.clusterDim.z = 1;
         cfg.numAttrs = 2;
-        cfg.gridDim = dim3((unsigned)(units * split));
+        cfg.gridDim = dim3((unsigned)(units * cluster));
         if (slot_float_count(p.rows, D) * sizeof(float) <= (size_t)plan.slots * kBlockN * D * 2 &&
-            cudaLaunchKernelEx(&cfg, attn_tc_kernel<D, 1, true>, p, set, mc, sh.Rp, plan.slots, sh.tmem_cols, split, sh.spare_cols) == cudaSuccess) {
+            cudaLaunchKernelEx(&cfg, attn_tc_kernel<D, 1, kClustered>, p, set, mc, sh.Rp, plan.slots, sh.tmem_cols, cluster, sh.spare_cols) == cudaSuccess) {
             count_launches(1);
             return HIPPO_OK;
         }
@@ -1637,15 +1639,15 @@ static int32_t launch_tc(const AttnParams &p, int grid, cudaStream_t stream) {
     }
     cfg.numAttrs = 1;
     cfg.gridDim = dim3((unsigned)grid);
-    const int mode = split == kFlat ? kFlat : kAligned;
-    HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_kernel<D, 1>, p, set, mc, sh.Rp, plan.slots, sh.tmem_cols, mode, sh.spare_cols));
+    const bool flat = form == kFlat || units > grid || units > kMaxAlignedUnits;
+    HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, flat ? attn_tc_kernel<D, 1, kFlat> : attn_tc_kernel<D, 1, kAligned>, p, set, mc, sh.Rp, plan.slots,
+                                      sh.tmem_cols, 0, sh.spare_cols));
     count_launches(1);
     const int n_rows = p.batch * p.q_len * p.n_q_heads;
     cfg.blockDim = dim3(kCombineThreads);
     cfg.dynamicSmemBytes = 0;
     // The combine kernel derives the slot table itself: of a unit-aligned split worked out by one warp (see the kernel); a warp per row also of
     // a flat split, with a lane per sequence.
-    const bool flat = mode == kFlat || units > grid || units > kMaxAlignedUnits;
     const int derive = !flat && units <= 32 ? grid : 0;
     if (grid <= 8 * units) {             // one round trip per row
         cfg.gridDim = dim3((unsigned)ceil_div(n_rows, kCombineThreads / 32));
@@ -1706,7 +1708,7 @@ static int packed_room(int dev, const TcSmemPlan &plan) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, attn_tc_kernel<D, kLayersPerLaunch>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
+        if (cudaOccupancyMaxActiveClusters(&n, attn_tc_kernel<D, kLayersPerLaunch, kByGrid>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
         room.store(n + 1, std::memory_order_relaxed);
     }
     return room.load(std::memory_order_relaxed) - 1;
@@ -1723,7 +1725,7 @@ static int32_t launch_tc_layers(AttnParams p, int n_layers, const void *const *q
     static std::atomic<int> sm_count[kMaxDevices];
     int dev;
     if (attr_set.needed(dev)) {
-        HIPPO_CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<D, NL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        HIPPO_CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<D, NL, kByGrid>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
         if (dev >= 0) {
             int n = 0;
             HIPPO_CUDA_TRY(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
@@ -1816,7 +1818,7 @@ static int32_t launch_tc_layers(AttnParams p, int n_layers, const void *const *q
             set.out[i] = out[l0 + i];
             set.lse[i] = lse ? lse[l0 + i] : nullptr;
         }
-        HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_kernel<D, NL>, p, set, mc, sh.Rp, sh.plan.slots, sh.tmem_cols, 0, sh.spare_cols));
+        HIPPO_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tc_kernel<D, NL, kByGrid>, p, set, mc, sh.Rp, sh.plan.slots, sh.tmem_cols, 0, sh.spare_cols));
         count_launches(1);
     }
     return HIPPO_OK;
