@@ -1455,6 +1455,12 @@ bool attn_tc_supported(const AttnParams &p, int dtype) {
            p.rows <= kMaxRows;
 }
 
+// Pages of sequence b as far as the host knows.
+static int seq_pages(const AttnParams &p, int b) {
+    const int kvl = p.kv_len_host ? (p.kv_len_host[b] < p.max_kv_len ? p.kv_len_host[b] : p.max_kv_len) : p.max_kv_len;
+    return kvl < p.q_len ? 0 : ceil_div(kvl, kPageSize);
+}
+
 // Pages of the longest unit and of all units together, from the host copy of the lengths when there is one.
 static void plan_pages(const AttnParams &p, int &longest, long long &total) {
     const int bound = ceil_div(p.max_kv_len, kPageSize);
@@ -1464,9 +1470,7 @@ static void plan_pages(const AttnParams &p, int &longest, long long &total) {
         longest = 0;
         total = 0;
         for (int b = 0; b < p.batch; ++b) {
-            int kvl = p.kv_len_host[b];
-            if (kvl > p.max_kv_len) kvl = p.max_kv_len;
-            const int pg = kvl < p.q_len ? 0 : ceil_div(kvl, kPageSize);
+            const int pg = seq_pages(p, b);
             if (pg > longest) longest = pg;
             total += (long long)pg * p.n_kv_heads;
         }
@@ -1489,10 +1493,7 @@ static int split_grid(const AttnParams &p, int sms) {
 static int aligned_longest(const AttnParams &p, int grid) {
     const int U = p.batch * p.n_kv_heads;
     if (U > grid || U > kMaxAlignedUnits) return 0;
-    auto pages = [&](int b) {
-        const int kvl = p.kv_len_host ? (p.kv_len_host[b] < p.max_kv_len ? p.kv_len_host[b] : p.max_kv_len) : p.max_kv_len;
-        return kvl < p.q_len ? 0 : ceil_div(kvl, kPageSize);
-    };
+    auto pages = [&](int b) { return seq_pages(p, b); };
     long long total = 0;
     int live = 0, given = 0;
     for (int b = 0; b < p.batch; ++b) { total += (long long)pages(b) * p.n_kv_heads; live += pages(b) > 0 ? p.n_kv_heads : 0; }
@@ -1517,40 +1518,45 @@ static int aligned_longest(const AttnParams &p, int grid) {
     return longest;
 }
 
-// How a single-layer call is split: kAligned, kFlat, or kClustered with the CTAs per unit in `cluster`.  The times, in us of a call in a chain of
-// them, are fitted to 75 shapes (head size 128, 1 to 64 units, 14 to 72 packed rows; 5 to 8 % off, the mean loss of the choice 1.4 %): a
-// constant, the pages of the longest CTA (the average for the flat split), the units, and the groups of 16 rows beyond 32 in each.
-// Measured, clusters / aligned / flat: eight ragged sequences of 10,406 keys, 4 kv heads, 42 rows 45.9 / 40.2 / 44.1; of 12,000, 8 kv heads,
-// 24 rows 70.3 / 80.9 / 72.5; of 9,000, 8 kv heads, 48 rows 65.2 / 67.2 / 60.5; four of 13,000, 8 kv heads, 24 rows 42.6 / 45.0 / 45.4, of 3,000
-// with 72 rows 26.4 / 24.0 / 29.8; one of 3,000, 48 rows 14.2 / 15.8 / 18.4, of 9,000, 4 kv heads, 28 rows 16.7 / 15.4 / 15.0.  Head size 64,
-// eight of 10,406, 42 rows: 38.8 / 34.2 / 37.2.
+// How a single-layer call is split: kAligned, kFlat, or kClustered with the CTAs per unit in `cluster`.  The form with the least estimated
+// time.  The estimates are least-squares fits (relative error, of the times within half of a shape's best) to 901 random calls in chains,
+// each run in all forms: head size 64 and 128, one to 33 sequences, equal and ragged, 1, 2, 4, 8 or 16 kv heads of 2 to 16 heads each, 2 to
+// 9 query tokens, 300 to 66,000 keys; off by 4 % (clusters), 6 (aligned) and 9 (flat).  The choice costs 0.9 % on average against the best
+// form of each shape, 16 of the 901 more than 8 %; to repeat the fit, time each form and solve for the factors below.
+// Measured, clusters / aligned / flat: eight ragged sequences of 10,406 keys, 4 kv heads, 42 rows 45.9 / 38.3 / 43.6; of 9,000, 8 kv heads, 48
+// rows 65.2 / 66.1 / 56.9; one of 327 keys, 8 kv heads, 64 rows 14.3 / 10.5 / 10.2; of 2,000, 4 kv heads, 28 rows 10.6 / 11.4 / 11.7.
+// A cluster of more than eight needs most of a GPC, and only six of them can be counted on to hold one; sizes between eight and sixteen
+// were slower than both (42 rows, 4 kv heads, 3,000 keys, clusters of 8 / 10 / 12 / 14 / 16: 13.5 / 17.3 / 15.7 / 15.1 / 14.5).
 static int choose_split(const AttnParams &p, int rows_padded, const int *max_active, int &cluster) {
-    const int units = p.batch * p.n_kv_heads, groups = rows_padded / 16;
+    const int units = p.batch * p.n_kv_heads, grid = split_grid(p, kNumSMs), even = aligned_longest(p, grid);
     int pages;
-    long long total_pages;
-    plan_pages(p, pages, total_pages);
-    const float g = groups <= 2 ? 0.f : groups - 2.f, u16 = units < 16 ? units : 16, u32 = units < 32 ? units : 32;
-    const int grid = split_grid(p, kNumSMs), even = aligned_longest(p, grid);
+    long long total;
+    plan_pages(p, pages, total);
+    bool equal = p.batch == 1 || p.kv_len_host;                                            // as far as the host knows
+    for (int b = 1; equal && b < p.batch; ++b) equal = seq_pages(p, b) == seq_pages(p, 0);
+    const float groups = (float)(rows_padded / 16), more = groups > 2.f ? groups - 2.f : 0.f, d = (float)p.head_dim / 128.f;
+    const float stream = d * (float)total / (float)kNumSMs;                                // HBM's share
+    const float per_unit = (float)grid / (float)units, waves = (float)((long long)p.batch * p.q_len * p.n_q_heads) / 1184.f;
+    const float few = per_unit < 8.f ? per_unit / 8.f : 1.f;                               // contributors of a row: up to 8, up to 32, beyond
+    const float some = per_unit < 8.f ? 0.f : per_unit < 32.f ? (per_unit - 8.f) / 24.f : 1.f, many = per_unit < 32.f ? 0.f : (per_unit - 32.f) / 32.f;
+    const bool by_row = grid <= 8 * units, wide = units > 32;                              // a warp merges a row; tables by the whole block
+    // the flat split: a CTA that goes over from one unit to the next has two segments
+    const int lead = flat_lead(total, units, grid);
+    const bool crossing = grid < total && !(equal && grid % units == 0);
     int best = kFlat;
-    const int lead = flat_lead(total_pages, units, grid);
-    float best_us = 10.2f + 0.385f * g + (0.703f + 0.037f * g) * (float)((total_pages + grid - 1) / grid) + (0.296f + 0.106f * g) * u16;
-    if (units >= kFlatLeadUnits)       // refitted with the empty entries
-        best_us = 11.6f + 1.4f * g + 0.70f * (float)(total_pages + (long long)lead * units) / grid + 0.6f * (kFlatLead - lead);
-    // Few units, from one sequence of 1,000 to 7,000 keys with 24 to 72 rows: many partials per row cost the split modes more, clusters of at
-    // most eight take less, larger ones more than the lines say.  28 rows, 4 kv heads, 2,000 keys: cluster of 8 / of 16 / aligned / flat
-    // 10.9 / 11.8 / 12.6 / 13.0; 5,500 keys 15.6 / 14.2 / 15.5 / 15.0; 48 rows, 8 kv heads, 1,000 keys 11.9 / - / 14.4 / 13.6.
-    const bool few = units <= 8;
-    if (few) best_us += units <= 4 ? 1.2f : 2.5f;
+    float best_us = 9.17f + 1.47f * d + 0.77f * more + 0.26f * (float)(total + (long long)lead * units) / (float)grid + 0.45f * stream - 2.49f * few +
+                    2.9f * some + 2.64f * many + (by_row ? 0.89f * waves : 0.33f - 0.28f * groups + 6.45f * waves) - (wide ? 1.21f : 0.f) +
+                    (crossing ? 2.27f + 0.74f * groups : 0.f);
     if (even > 0) {
-        const float us = 11.6f + 1.32f * g + (0.69f + 0.034f * g) * even + (0.027f - 0.0154f * g) * u32 + (units <= 4 ? 1.1f : few ? 0.5f : 0.f);
+        const float us = 12.04f + 0.93f * d + 0.53f * more + 0.36f * (float)even + 0.39f * stream - 4.99f * few + 3.05f * some + 2.55f * many +
+                         (by_row ? 1.34f * waves : -0.1f - 0.18f * groups + 10.11f * waves) + (wide ? 1.44f : 0.f);
         if (us < best_us) { best = kAligned; best_us = us; }
     }
-    // A cluster of more than eight needs most of a GPC, and only six of them can be counted on to hold one; sizes between eight and sixteen
-    // were slower than both (42 rows, 4 kv heads, 3,000 keys, clusters of 8 / 10 / 12 / 14 / 16: 13.5 / 17.3 / 15.7 / 15.1 / 14.5).
     for (int cs = 2; cs <= (units <= 6 ? 16 : 8) && 2 * cs <= pages + 1; cs = cs == 8 ? 16 : cs + 1) {
         if (units > max_active[cs]) continue;
-        const float us = 9.6f + 1.0f * g + (0.564f + 0.045f * g) * ceil_div(pages, cs) + (0.079f + 0.029f * g) * u32 +
-                         (cs > 8 ? 0.8f : few ? -1.1f : 0.f);
+        const float tiles = (float)ceil_div(ceil_div(pages, cs), 2);
+        const float us = 7.24f + 2.57f * d + 1.33f * more + (0.84f + 0.08f * groups) * tiles + 0.17f * stream + 0.9f / 64.f * groups * (units < 32 ? units : 32) -
+                         1.3f / 8.f * cs + (cs > 8 ? 2.45f : 0.f);
         if (us < best_us) { best = kClustered; cluster = cs; best_us = us; }
     }
     return best;
