@@ -52,8 +52,9 @@ typedef enum hippo_status {
 typedef enum hippo_dtype { HIPPO_DTYPE_FP32 = 0, HIPPO_DTYPE_BF16 = 1 } hippo_dtype_t;
 
 typedef enum hippo_accept_mode { HIPPO_ACCEPT_SAMPLE = 0, HIPPO_ACCEPT_GREEDY = 1 } hippo_accept_mode_t;
-/* optional flags OR-ed into the mode of the sampling acceptance: force one of its two launch forms (same arithmetic, same
- * results; without a flag the library picks the faster one for the shape) */
+/* optional flags OR-ed into the mode of the sampling acceptance: force one of its two launch forms (the same device code; the
+ * forms cut the vocabulary into different pieces for few sequences, so their running sums may round differently and a draw
+ * differ where its uniform lies within that rounding of a token's boundary; without a flag the library picks the faster form) */
 #define HIPPO_ACCEPT_ONE_LAUNCH 16      /* one kernel, its CTAs meet at two counters in the workspace header */
 #define HIPPO_ACCEPT_THREE_LAUNCHES 32  /* three chained kernels */
 

@@ -671,8 +671,8 @@ static int32_t make_k_map(CUtensorMap *m, const void *pool, long long rows, int 
     return HIPPO_OK;
 }
 
-// Each kernel of the chain begins with griddepcontrol.wait: its set-up (barriers, tensor memory, cleared tiles) overlaps the end of the
-// one before.
+// Each kernel of the chain waits (griddepcontrol.wait) before it touches global memory: its set-up (barriers, tensor memory, cleared tiles; the
+// merge's search for its parts) overlaps the end of the one before.  The merge releases pass 2 at its start; the others after their wait.
 template <typename... Args>
 static cudaError_t launch_mass_dependent(void (*kernel)(Args...), long long grid, int threads, size_t smem, cudaStream_t s, Args... args) {
     cudaLaunchAttribute attr[1];

@@ -16,15 +16,16 @@
 // recomputed and O^T and the partial sums are rescaled in tensor memory.
 //
 // Work split (persistent CTAs, one per SM).  Three modes, chosen on the host from the shape:
-//  * cluster: one thread-block cluster (2, 4, 8 or 16 CTAs) per unit.  The CTAs of a cluster split the unit's
+//  * cluster: one thread-block cluster (2 to 8 or 16 CTAs) per unit.  The CTAs of a cluster split the unit's
 //    tiles evenly, leave their partial (m, l, O) in their own shared memory, and after a cluster barrier every CTA
 //    merges a share of the rows by reading its peers' partials through distributed shared memory.  One launch, no
-//    trip through global memory; used whenever clusters of that size keep enough SMs busy.
+//    trip through global memory; best for short caches.
 //  * unit-aligned split + combine kernel: with no more (sequence, kv head) units than CTAs, every unit gets a
 //    whole number of CTAs in proportion to its tile count (at least one; largest-remainder rounding) and each CTA
 //    streams one contiguous range of its unit's tiles: one "segment" per CTA, no pipeline drain in the middle.
-//  * flat split + combine kernel: with more units than CTAs the tiles of all units form one flat list cut into
-//    gridDim.x equal ranges, and a CTA walks its range segment by segment.
+//  * flat split + combine kernel: the tiles of all units form one flat list cut into gridDim.x equal ranges, and a
+//    CTA walks its range segment by segment; always with more units than CTAs, and where units and CTAs fit badly.
+// choose_split estimates the time of each; each is an instantiation of its own.
 // Without clusters a segment yields either the final output (it covers the whole unit) or a partial
 // (m, l, O) in a workspace slot; CTA 0 records per unit the first slot and the number of contributors, and the
 // combine kernel merges them.
@@ -344,8 +345,9 @@ attn_tc_kernel(const AttnParams p, const __grid_constant__ LayerSetT<NL> set, co
     const int R = p.rows, G = p.group, Hkv = p.n_kv_heads, B = p.batch;
     const int n_layers = kMulti ? mc.n_layers : 1;
     // Launched with programmatic stream serialization: the CTAs may be scheduled while the previous kernel of the
-    // stream drains.  Barriers and tensor memory are set up meanwhile; global memory is not touched before that
-    // kernel has completed (griddepcontrol.wait below).
+    // stream runs.  Barriers and tensor memory are set up meanwhile.  Before that kernel has completed
+    // (griddepcontrol.wait below) nothing is written to global memory, and what is read there - lengths and page ids -
+    // is either looked up again after the wait or used for prefetches only, inside the bounds of the pool.
 
     // ---- set-up: barriers, tile prefix, CTA split, tensor memory
     const int U = B * Hkv;
@@ -1618,8 +1620,11 @@ static int32_t launch_tc(const AttnParams &p, int grid, cudaStream_t stream) {
     }
     int cluster = 0;
     const int form = p.num_splits > 0 ? kAligned : choose_split(p, sh.Rp, max_active[plan.slots], cluster);
-    // Both kernels are launched with programmatic stream serialization and wait (griddepcontrol.wait) before they
-    // touch memory, so stream order is kept while launch latency overlaps the previous kernel's tail.
+    // Both kernels are launched with programmatic stream serialization, so that launch latency overlaps the previous
+    // kernel's tail.  Stream order is kept: both wait (griddepcontrol.wait) before they write to global memory and before
+    // they use what the kernel ahead may write.  What the main kernel reads ahead of its wait is a hint or looked up again;
+    // the merge reads the lengths ahead of its own, which are complete because the main kernel lets it be launched only
+    // after its wait.  The merge in turn releases the next call at its start, whose wait covers the merge and so this call.
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;

@@ -278,8 +278,9 @@ class HippoStep:
         """The whole step on the current stream, with draft and verify forked onto their own streams.
 
         The verification leg reads neither the selection nor the pruned cache.  With `verify_beside_select` it is forked
-        first and runs beside select and gather too; otherwise it starts once the selection has finished (the selection's
-        kernels take every SM) and runs beside the draft calls only."""
+        first and runs beside select and gather too; otherwise it starts once the selection has finished and runs beside the
+        draft calls only.  The selection's tiles are planned in whole waves over every SM, so beside a verification pass a wave
+        becomes two: 32k tokens, verification on 96 SMs, 1.51 ms beside the selection, 1.33 after it."""
         main = torch.cuda.current_stream(self.device)
         if self.verify_beside_select:
             self.stream_v.wait_stream(main)
